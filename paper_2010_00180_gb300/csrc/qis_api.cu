@@ -63,7 +63,7 @@ struct qis_ctx {
   std::vector<uint64_t> init_host;   // [max_inst * R][Wmax]
   std::vector<char> init_from_host;  // instance whose initial states wait in init_host
   // init_E / init_q hold the energies of the instance's current initial states (formed by
-  // k_init_energy or k_init_search; the fused search kernel's deferred values do not count here:
+  // launch_init_energy or k_init_search; the fused search kernel's deferred values do not count here:
   // a run that failed may have formed them from bad fields)
   std::vector<char> e0_valid;
   // instances whose searches were started with their initial energies left to the fused search
@@ -162,6 +162,16 @@ int check_status(qis_ctx* ctx) {
                 "a search produced more survivors than survivor_cap (raise survivor_cap); the searches are "
                 "undefined until qis_reset");
   if (st) return fail(ctx, QIS_ERR_STATE, "device reported an inconsistent search state");
+  return 0;
+}
+
+// After the last copy of rescored energies is enqueued: wait for the stream, and fail if a wait of
+// the rescoring kernel (or of an earlier one) gave up.
+int sync_energies(qis_ctx* ctx) {
+  int st = 0;
+  CK(cudaMemcpyAsync(&st, ctx->P.status, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  CK(cudaStreamSynchronize(ctx->stream));
+  if (st & kStatTimeout) return check_status(ctx);
   return 0;
 }
 
@@ -489,16 +499,14 @@ int qis_create(const qis_config* cfg, qis_ctx** out) {
     ALLOC(P.mrg_ref, (size_t)ctx->max_inst * K1);
     ALLOC(P.mrg_src, (size_t)ctx->max_inst * K1);
     ALLOC(P.mrg_count, ctx->max_inst);
-    ctx->scratch_states = 4096;
+    ctx->scratch_states = 16384;   // states rescored per launch
     ALLOC(ctx->scratch_bits, (size_t)ctx->scratch_states * W);
     ALLOC(ctx->scratch_E, ctx->scratch_states);
-    {   // partial energy sums of the rescoring when a state group's rows are split over blocks
+    {   // integer sums of the energies from scratch: the states of one launch at most
       size_t m = std::max<size_t>((size_t)ctx->max_inst * K1, (size_t)B);
       m = std::max<size_t>(m, (size_t)ctx->scratch_states);
-      ALLOC(P.rs_acc, 2 * m * 32);   // [state][row part][2], at most 32 parts
-      int sms = 0;
-      CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->cfg.device));
-      P.sms = sms;
+      ALLOC(P.en_acc, 2 * m);
+      ALLOC(P.en_left, m / 128 + (size_t)ctx->max_inst + 1);
     }
     // Zobrist keys of the sites (SplitMix64 stream with a fixed key)
     std::vector<uint64_t> z(kMaxN);
@@ -610,6 +618,9 @@ int describe_instance(qis_ctx* ctx, int id, int n, const double* st, InstDesc& d
   d.rounded = 0;
   d.j4max = 0.f;
   d.j4max64 = 4.0 * maxJ;   // exact (power-of-two scaling)
+  // energies from scratch: integers J 2^eq, exact where 58 bits hold every coupling
+  frexp(std::max(maxJ, maxh), &d.etop);
+  d.eq = std::min(maxfrac, 58 - d.etop);
   if (ctx->mode != QIS_FP64) {
     double S = 0.0;
     for (int i = 0; i < n; ++i) S += st[4 + i];
@@ -681,7 +692,7 @@ namespace {
 // defer (qis_iterate, when the fused search kernel runs at least one iteration): the initial
 // energies of the split modes are not computed here; the kernel forms them from the exact fields
 // of the first iteration (E = (sum_i s_i f_i + sum_i s_i h_i) / 2), which the tensor-core GEMM
-// computes for every initial state anyway. Otherwise they come from k_init_energy, or from
+// computes for every initial state anyway. Otherwise they come from launch_init_energy, or from
 // init_E / init_q when those still hold them.
 int flush_init(qis_ctx* ctx, bool defer) {
   const int ni = (int)ctx->init_pending.size();
@@ -724,7 +735,9 @@ int flush_init(qis_ctx* ctx, bool defer) {
     } else if (grouped && !known) {
       int max_n = 0;
       for (int x = a; x < e; ++x) max_n = std::max(max_n, ctx->inst[x].n);
-      LAUNCH(launch_init_energy(ctx->P, a, e - a, max_n, ctx->stream));
+      int dg = 1;
+      for (int x = a; x < e; ++x) dg = std::max(dg, energy_digits(ctx->inst[x].etop, ctx->inst[x].q));
+      LAUNCH(launch_init_energy(ctx->P, a, e - a, max_n, dg, ctx->stream));
     }
     LAUNCH(launch_init_search(ctx->P, ctx->inst[a].first_search, (e - a) * ctx->R, ctx->stream,
                               known || (grouped && !deferred), deferred));
@@ -1437,14 +1450,15 @@ int qis_topk_states(qis_ctx* ctx, int instance_id, int k, uint64_t* bits_out, do
     DevPtrs Q = ctx->P;
     Q.mrg_ref = ctx->P.mrg_ref + off;   // shift the view so row 0 is entry `off`
     LAUNCH(launch_gather_merged(Q, instance_id, d, c, ctx->scratch_bits, s));
-    LAUNCH(launch_rescore(ctx->P, d, ctx->scratch_bits, c, d.W, ctx->scratch_E, s));
+    LAUNCH(launch_energies(ctx->P, instance_id, d, ctx->scratch_bits, c, d.W, ctx->scratch_E, s));
     if (bits_out) CK(cudaMemcpyAsync(bits_out + (size_t)off * d.W, ctx->scratch_bits, sizeof(uint64_t) * c * d.W,
                                      cudaMemcpyDeviceToHost, s));
     if (E_out) CK(cudaMemcpyAsync(E_out + off, ctx->scratch_E, sizeof(double) * c, cudaMemcpyDeviceToHost, s));
     if (src_out && off == 0)
       CK(cudaMemcpyAsync(src_out, ctx->P.mrg_src + (size_t)instance_id * ctx->K1, sizeof(uint64_t) * m,
                          cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
+    const int rc = sync_energies(ctx);
+    if (rc) return rc;
   }
   if (n_out) *n_out = m;
   return 0;
@@ -1464,13 +1478,12 @@ int qis_topk_states_all(qis_ctx* ctx, int k, uint64_t* bits_out, double* E_out, 
   }
   const int ni = (int)ctx->inst.size(), Wm = ctx->Wmax;
   if (k > 0) {
-    bool exact = ctx->mode != QIS_FP64;
-    int max_n = 0;
+    int max_n = 0, dg = 1;
     for (const InstDesc& d : ctx->inst) {
-      exact = exact && !d.rounded;
       max_n = std::max(max_n, d.n);
+      dg = std::max(dg, energy_digits(d.etop, ctx->mode != QIS_FP64 && !d.rounded ? d.q : d.eq));
     }
-    LAUNCH(launch_topk_all(ctx->P, k, exact, max_n, ctx->all_bits, ctx->all_E, s));
+    LAUNCH(launch_energies_merged(ctx->P, k, max_n, dg, ctx->all_bits, ctx->all_E, s));
   }
   int rc = sync_and_check(ctx);
   if (rc) return rc;
@@ -1510,9 +1523,10 @@ int qis_energies(qis_ctx* ctx, int instance_id, int count, const uint64_t* bits,
   for (int off = 0; off < count; off += ctx->scratch_states) {
     const int c = (count - off < ctx->scratch_states) ? count - off : ctx->scratch_states;
     CK(cudaMemcpyAsync(ctx->scratch_bits, bits + (size_t)off * d.W, sizeof(uint64_t) * c * d.W, cudaMemcpyHostToDevice, s));
-    LAUNCH(launch_rescore(ctx->P, d, ctx->scratch_bits, c, d.W, ctx->scratch_E, s));
+    LAUNCH(launch_energies(ctx->P, instance_id, d, ctx->scratch_bits, c, d.W, ctx->scratch_E, s));
     CK(cudaMemcpyAsync(E_out + off, ctx->scratch_E, sizeof(double) * c, cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
+    const int rc = sync_energies(ctx);
+    if (rc) return rc;
   }
   return 0;
 }

@@ -37,6 +37,8 @@ struct InstDesc {
   float j4max;        // max |fl32(4 J_ij)|
   double j4max64;    // 4 max |J_ij| (exact in FP64)
   int rounded;        // input was rounded onto the grid
+  int etop;           // every |J_ij|, |h_i| < 2^etop
+  int eq;             // exponent of the integers J 2^eq that energies from scratch are summed in
 };
 
 // Device pointers of one context (passed to kernels by value).
@@ -113,10 +115,8 @@ struct DevPtrs {
   int* mrg_ref;           // [inst][K1] search*K1 + slot
   uint64_t* mrg_src;      // [inst][K1]
   int* mrg_count;         // [inst]
-  // rescoring from scratch: partial sums (sum of J over differing spins, sum of all J; int64 or
-  // FP64) per output state and row part when the rows of a group of states are split over blocks
-  unsigned long long* rs_acc;   // [states][32][2]
-  int sms;                      // streaming multiprocessors of the device
+  unsigned long long* en_acc;   // [states][2] integer sums of the energies from scratch (zero between calls)
+  int* en_left;                 // [states / 128, rounded up per instance] blocks done of a state tile (zero between calls)
 };
 
 __host__ __device__ inline int words_of(int n) { return (n + 63) >> 6; }
@@ -199,6 +199,13 @@ __device__ inline unsigned long long dkey(double x) {
   return (u & 0x8000000000000000ull) ? ~u : (u | 0x8000000000000000ull);
 }
 
+// Digits of 12 bits that hold the integers J 2^q of an instance with every |J|, |h| < 2^top (a bit
+// to spare for the balanced digits).
+__host__ __device__ inline int energy_digits(int top, int q) {
+  const int x = (top + q + 2 + 11) / 12;
+  return x < 1 ? 1 : x > kMaxDigits ? kMaxDigits : x;
+}
+
 // order-preserving key of an exact integer energy E 2^q (signed -> unsigned)
 __host__ __device__ inline unsigned long long qkey(long long x) { return (unsigned long long)x ^ (1ull << 63); }
 
@@ -211,6 +218,29 @@ __host__ __device__ inline int next_pow2(int x) {
 // FP64 energy change of the pair flip (i, j): (a_i + a_j) + 4 s_i s_j J_ij, the product exact
 __device__ inline double dE64(double ai, double aj, double j, int flip) {
   return __dadd_rn(__dadd_rn(ai, aj), flip ? -4.0 * j : 4.0 * j);
+}
+
+// x 2^q rounded to the nearest integer, ties to even (what __double2ll_rn(ldexp(x, q)) gives),
+// from the bit pattern of x with integer operations only (GB300's FP64 pipe is narrow). x is
+// finite (validated) and |x 2^q| < 2^62 (the grid is chosen so).
+__device__ __forceinline__ long long fixed_point_rn(double x, int q) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)((u >> 52) & 0x7ff);
+  unsigned long long m = u & 0xfffffffffffffull;
+  if (e == 0 && m == 0) return 0;
+  if (e != 0) m |= 1ull << 52;                    // normal: the implicit bit
+  const int sh = (e == 0 ? 1 : e) - 1075 + q;     // |x| 2^q = m 2^sh
+  long long v;
+  if (sh >= 0) {
+    v = (long long)(m << sh);
+  } else if (sh <= -54) {
+    v = 0;   // below 1/2
+  } else {
+    const int r = -sh;
+    const unsigned long long t = m >> r, rem = m & ((1ull << r) - 1), half = 1ull << (r - 1);
+    v = (long long)(t + ((rem > half || (rem == half && (t & 1ull))) ? 1ull : 0ull));
+  }
+  return (u >> 63) ? -v : v;
 }
 
 __device__ inline double dkey_inv(unsigned long long k) {
@@ -342,11 +372,11 @@ cudaError_t launch_merge(const DevPtrs& P, cudaStream_t s);
 cudaError_t launch_final_merge(const DevPtrs& P, cudaStream_t s);
 size_t merge_smem(int K1, int cap, int merge_cand);
 size_t final_merge_smem(int K1);
-cudaError_t launch_rescore(const DevPtrs& P, const InstDesc& d, const uint64_t* bits, int count, int Wn,
-                           double* E_out, cudaStream_t s);
-cudaError_t launch_topk_all(const DevPtrs& P, int k, bool all_exact, int max_n, uint64_t* out, double* E,
-                            cudaStream_t s);
-cudaError_t launch_init_energy(const DevPtrs& P, int inst0, int n_inst, int max_n, cudaStream_t s);
+cudaError_t launch_energies(const DevPtrs& P, int inst, const InstDesc& d, const uint64_t* states, int count, int Wn,
+                            double* E_out, cudaStream_t s);
+cudaError_t launch_energies_merged(const DevPtrs& P, int k, int max_n, int digits, uint64_t* words, double* E_out,
+                                   cudaStream_t s);
+cudaError_t launch_init_energy(const DevPtrs& P, int inst0, int n_inst, int max_n, int digits, cudaStream_t s);
 cudaError_t launch_gather_merged(const DevPtrs& P, int inst, const InstDesc& d, int k, uint64_t* bits_out,
                                  cudaStream_t s);
 

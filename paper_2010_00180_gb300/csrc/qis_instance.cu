@@ -1,4 +1,4 @@
-// qis_instance.cu -- per-instance preparation, search initialisation and FP64 rescoring.
+// qis_instance.cu -- per-instance preparation and search initialisation.
 //
 // Instance data (H0 of Eq. (1)) lives in padded n_pad x n_pad planes:
 //   J64  FP64 couplings as given (zero padding)
@@ -162,29 +162,6 @@ __global__ void k_quantize(const double* J64, const double* h64, int n, int n_pa
   if (e < n_pad) hq[e] = (e < n) ? __double2ll_rn(ldexp(h64[e], q)) : 0;
 }
 
-// x 2^q rounded to the nearest integer, ties to even (what __double2ll_rn(ldexp(x, q)) gives),
-// from the bit pattern of x with integer operations only (GB300's FP64 pipe is narrow). x is
-// finite (validated) and |x 2^q| < 2^62 (the grid is chosen so).
-__device__ __forceinline__ long long fixed_point_rn(double x, int q) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
-  const int e = (int)((u >> 52) & 0x7ff);
-  unsigned long long m = u & 0xfffffffffffffull;
-  if (e == 0 && m == 0) return 0;
-  if (e != 0) m |= 1ull << 52;                    // normal: the implicit bit
-  const int sh = (e == 0 ? 1 : e) - 1075 + q;     // |x| 2^q = m 2^sh
-  long long v;
-  if (sh >= 0) {
-    v = (long long)(m << sh);
-  } else if (sh <= -54) {
-    v = 0;   // below 1/2
-  } else {
-    const int r = -sh;
-    const unsigned long long t = m >> r, rem = m & ((1ull << r) - 1), half = 1ull << (r - 1);
-    v = (long long)(t + ((rem > half || (rem == half && (t & 1ull))) ? 1ull : 0ull));
-  }
-  return (u >> 63) ? -v : v;
-}
-
 // Instances first .. first+count-1 at once (blockIdx.y), descriptors read on the device; rows
 // i = blockIdx.x, blockIdx.x + gridDim.x, ..., the threads over the columns (no index division).
 // Jq = rn(J 2^q), J4 = fl32(4 Jq 2^-q) (= fl32(Jq) 2^(2-q): scaling by a power of two commutes
@@ -270,8 +247,8 @@ cudaError_t launch_rowmax4(const DevPtrs& P, const InstDesc& d, cudaStream_t s) 
 
 // ---------------------------------------------------------------- search initialisation
 // Alg. 3 initial list: [psi0, K placeholders], E(psi0) from Eq. (1), nothing used.
-// mode 1 (cached): E(psi0) is taken from init_E / init_q, written by k_init_energy (split modes:
-// exact int64 E 2^q, several states per block) or by an earlier launch for the same initial
+// mode 1 (cached): E(psi0) is taken from init_E / init_q, written by launch_init_energy (split modes:
+// exact int64 E 2^q) or by an earlier launch for the same initial
 // states. Mode 2 (deferred, split modes): E(psi0) is left to the first iteration of the fused
 // search kernel, which forms it from the exact fields of psi0 that the iteration computes anyway;
 // the entry holds 0 until then and e0_pend marks the search. Mode 0 (FP64 mode): one thread adds
@@ -344,189 +321,6 @@ cudaError_t launch_init_search(const DevPtrs& P, int b0, int nb, cudaStream_t s,
   return cudaGetLastError();
 }
 
-// ---------------------------------------------------------------- rescoring from scratch
-// E = sum_{i<j} J_ij s_i s_j + sum_i h_i s_i (Eq. 1) of up to kRG states of one instance per
-// block of 256 threads. With x_ij = 1 where s_i != s_j (s = -1 where the bit is set),
-// s_i s_j = 1 - 2 x_ij and s_i = 1 - 2 sigma_i, so
-//   E = Q - 2 P,  Q = sum_{i<j} J_ij + sum_i h_i,  P = sum_{i<j, x_ij = 1} J_ij + sum_{sigma_i = 1} h_i:
-// one pass over the upper triangle serves every state of the block. mask[j] holds the block's
-// spins of site j as bits; a coupling loaded once is added to the accumulator of every state
-// whose two spins differ. Warp w takes rows w, w + 8, ... of the block's row range, its lanes the
-// columns j > i (coalesced). T = long long: the exact fixed-point couplings Jq, hq of an instance
-// on its grid 2^-q (every summation order gives the same integer); T = double: the FP64
-// couplings, summed in an order fixed by the block shape and not by the state's place in the
-// group. When there are few groups (large n, few states), the rows are split over `parts`
-// blocks per group, whose partial sums a second kernel adds in part order (the FP64 form takes a
-// number of parts fixed by n alone, so every call forms a state's energy the same way).
-constexpr int kRG = 16;
-
-// Rows [i0, i1) of the upper triangle (and the h terms if with_h): red[g] = P_g, red[kRG] = Q.
-template <typename T>
-__device__ void rescore_part(const T* __restrict__ Jm, const T* __restrict__ hv, int n, int n_pad, int i0, int i1,
-                             bool with_h, const uint16_t* __restrict__ mask, T* red /* [9][kRG + 1] */) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  T q = 0, p[kRG];
-#pragma unroll
-  for (int g = 0; g < kRG; ++g) p[g] = 0;
-  for (int i = i0 + warp; i < i1; i += 8) {
-    const T* __restrict__ row = Jm + (long long)i * n_pad;
-    const unsigned mi = mask[i];
-#pragma unroll 2
-    for (int j = i + 1 + lane; j < n; j += 32) {
-      const T v = row[j];
-      const unsigned x = mi ^ mask[j];
-      q += v;
-#pragma unroll
-      for (int g = 0; g < kRG; ++g)
-        if ((x >> g) & 1u) p[g] += v;
-    }
-  }
-  if (with_h)
-    for (int i = threadIdx.x; i < n; i += 256) {
-      const T v = hv[i];
-      const unsigned m = mask[i];
-      q += v;
-#pragma unroll
-      for (int g = 0; g < kRG; ++g)
-        if ((m >> g) & 1u) p[g] += v;
-    }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    q += __shfl_xor_sync(0xffffffffu, q, o);
-#pragma unroll
-    for (int g = 0; g < kRG; ++g) p[g] += __shfl_xor_sync(0xffffffffu, p[g], o);
-  }
-  if (lane == 0) {
-#pragma unroll
-    for (int g = 0; g < kRG; ++g) red[warp * (kRG + 1) + g] = p[g];
-    red[warp * (kRG + 1) + kRG] = q;
-  }
-  __syncthreads();
-  if (threadIdx.x <= kRG) {
-    T t = 0;
-    for (int w = 0; w < 8; ++w) t += red[w * (kRG + 1) + threadIdx.x];
-    red[8 * (kRG + 1) + threadIdx.x] = t;
-  }
-  __syncthreads();
-  if (threadIdx.x <= kRG) red[threadIdx.x] = red[8 * (kRG + 1) + threadIdx.x];
-  __syncthreads();
-}
-
-// First row of part b of `parts` row ranges with about equal shares of the triangle (rows i..n-1
-// hold (n - i)^2 / 2 of its pairs): n - round(n sqrt(1 - b / parts)); part 0 starts at row 0.
-__device__ inline int part_row(int n, int b, int parts) {
-  if (b <= 0) return 0;
-  if (b >= parts) return n;
-  const int r = n - (int)lrintf((float)n * sqrtf(1.f - (float)b / (float)parts));
-  return min(max(r, 0), n);
-}
-
-constexpr int kRPmax = 32;   // row parts per group at most
-
-// Rows of part blockIdx.y of `parts`, then E of the group's states (one part), or their partial
-// sums (P, Q) into part[(g * PS + blockIdx.y) * 2 ...] for the states g = 0 .. cnt - 1 of the
-// group (several parts; PS >= parts, the stride of one state). Calls out(g, E) for g < cnt in the
-// first case.
-template <typename T, typename Out>
-__device__ void rescore_group(const T* Jm, const T* hv, int n, int n_pad, const uint16_t* mask, T* red, int cnt,
-                              int parts, T* part, int PS, Out out) {
-  const int b = blockIdx.y;
-  rescore_part<T>(Jm, hv, n, n_pad, part_row(n, b, parts), part_row(n, b + 1, parts), b == 0, mask, red);
-  if (threadIdx.x < cnt) {
-    if (parts == 1) {
-      out((int)threadIdx.x, red[kRG] - 2 * red[threadIdx.x]);
-    } else {
-      T* x = part + ((long long)threadIdx.x * PS + b) * 2;
-      x[0] = red[threadIdx.x];
-      x[1] = red[kRG];
-    }
-  }
-}
-
-// E = Q - 2 P of a state from its `parts` partial sums (stride 2 between parts), added in order.
-template <typename T>
-__device__ inline T rs_energy(const T* part, int parts) {
-  T p = 0, q = 0;
-  for (int b = 0; b < parts; ++b) {
-    p += part[2 * b];
-    q += part[2 * b + 1];
-  }
-  return q - 2 * p;
-}
-
-// The spin masks of cnt <= kRG states (their words at src[g], Wn words each) into mask[0..n).
-__device__ void group_masks(const uint64_t* const* src, int cnt, int n, uint16_t* mask) {
-  for (int j = threadIdx.x; j < n; j += blockDim.x) {
-    unsigned m = 0;
-    for (int g = 0; g < cnt; ++g) m |= (unsigned)((src[g][j >> 6] >> (j & 63)) & 1ull) << g;
-    mask[j] = (uint16_t)m;
-  }
-}
-
-// Row parts of the FP64 form: a number fixed by n alone, so that a state's energy is summed the
-// same way whichever call and group rescore it.
-__host__ __device__ inline int fp64_parts(int n) { return n / 512 < 1 ? 1 : (n / 512 > kRPmax ? kRPmax : n / 512); }
-
-// Row parts per group. Exact form: one unless the groups alone leave the SMs idle (any split
-// gives the same integers). FP64 form: fp64_parts(n).
-int rescore_parts(const DevPtrs& P, int groups, int n, bool exact) {
-  if (!exact) return fp64_parts(n);
-  if (groups <= 0) return 1;
-  const int target = 4 * (P.sms > 0 ? P.sms : 148);
-  int parts = (target + groups - 1) / groups;
-  parts = std::min(std::min(parts, kRPmax), std::max(1, n / 256));
-  return std::max(parts, 1);
-}
-
-// Energies of `count` states (Wn words each, consecutive) of one instance: block x takes
-// states kRG x ... kRG x + kRG - 1, block y its part of the rows.
-template <typename T>
-__global__ void __launch_bounds__(256) k_rescore(const T* Jm, const T* hv, int n, int n_pad, double scale,
-                                                 const uint64_t* states, int Wn, int count, double* E_out,
-                                                 unsigned long long* acc) {
-  extern __shared__ __align__(16) unsigned char rsm[];
-  T* red = reinterpret_cast<T*>(rsm);
-  uint16_t* mask = reinterpret_cast<uint16_t*>(red + 9 * (kRG + 1));
-  __shared__ const uint64_t* src[kRG];
-  const int g0 = blockIdx.x * kRG, cnt = min(kRG, count - g0);
-  if (threadIdx.x < kRG) src[threadIdx.x] = states + (long long)(g0 + min((int)threadIdx.x, cnt - 1)) * Wn;
-  __syncthreads();
-  group_masks(src, cnt, n, mask);
-  __syncthreads();
-  rescore_group<T>(Jm, hv, n, n_pad, mask, red, cnt, gridDim.y, reinterpret_cast<T*>(acc) + 2ll * g0 * gridDim.y,
-                   gridDim.y, [&](int g, T E) { E_out[g0 + g] = (double)E * scale; });
-}
-
-template <typename T>
-__global__ void k_rescore_finish(const unsigned long long* acc, int count, int parts, double scale, double* E_out) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s < count) E_out[s] = (double)rs_energy(reinterpret_cast<const T*>(acc) + 2ll * s * parts, parts) * scale;
-}
-
-size_t rescore_smem(int n, int bytes_T) { return (size_t)9 * (kRG + 1) * bytes_T + (size_t)n * 2; }
-
-cudaError_t launch_rescore(const DevPtrs& P, const InstDesc& d, const uint64_t* bits, int count, int Wn,
-                           double* E_out, cudaStream_t s) {
-  if (count <= 0) return cudaSuccess;
-  const int groups = (count + kRG - 1) / kRG;
-  const size_t sm = rescore_smem(d.n, 8);
-  const bool exact = P.mode != QIS_FP64 && !d.rounded;
-  const int parts = rescore_parts(P, groups, d.n, exact);
-  if (exact) {
-    if (sm > 48 * 1024) cudaFuncSetAttribute(k_rescore<long long>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_rescore<long long><<<dim3(groups, parts), 256, sm, s>>>(P.Jq + d.off_mat, P.hq + d.off_vec, d.n, d.n_pad,
-                                                              d.inv_scale, bits, Wn, count, E_out, P.rs_acc);
-    if (parts > 1)
-      k_rescore_finish<long long><<<(count + 255) / 256, 256, 0, s>>>(P.rs_acc, count, parts, d.inv_scale, E_out);
-  } else {
-    if (sm > 48 * 1024) cudaFuncSetAttribute(k_rescore<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_rescore<double><<<dim3(groups, parts), 256, sm, s>>>(P.J64 + d.off_mat, P.h64 + d.off_vec, d.n, d.n_pad, 1.0,
-                                                           bits, Wn, count, E_out, P.rs_acc);
-    if (parts > 1) k_rescore_finish<double><<<(count + 255) / 256, 256, 0, s>>>(P.rs_acc, count, parts, 1.0, E_out);
-  }
-  return cudaGetLastError();
-}
-
 // ---------------------------------------------------------------- merged-list gather
 __global__ void k_gather_merged(DevPtrs P, int inst, int k, int Wn, uint64_t* out) {
   const int r = blockIdx.x;
@@ -541,122 +335,6 @@ cudaError_t launch_gather_merged(const DevPtrs& P, int inst, const InstDesc& d, 
                                  cudaStream_t s) {
   if (k <= 0) return cudaSuccess;
   k_gather_merged<<<k, 32, 0, s>>>(P, inst, k, d.W, bits_out);
-  return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------- initial energies
-// E(psi0) 2^q of the initial states of instances inst0, inst0 + 1, ... in the split modes
-// (exact int64, Eq. 1), kRG states of one instance per block (row parts as above), into
-// init_q / init_E; the search initialisation then takes them as cached values.
-__device__ inline void init_energy_out(const DevPtrs& P, const InstDesc& d, long long b, long long Eq) {
-  P.init_q[b] = Eq;
-  P.init_E[b] = ldexp((double)Eq, -d.q);
-}
-
-__global__ void __launch_bounds__(256) k_init_energy(DevPtrs P, int inst0, int ng) {
-  const int inst = inst0 + blockIdx.x / ng, g0 = (blockIdx.x % ng) * kRG;
-  const int cnt = min(kRG, P.R - g0);
-  const InstDesc d = P.inst[inst];
-  extern __shared__ __align__(16) unsigned char rsm[];
-  long long* red = reinterpret_cast<long long*>(rsm);
-  uint16_t* mask = reinterpret_cast<uint16_t*>(red + 9 * (kRG + 1));
-  __shared__ const uint64_t* src[kRG];
-  const long long b0 = (long long)d.first_search + g0;
-  if (threadIdx.x < kRG) src[threadIdx.x] = P.init_bits + (b0 + min((int)threadIdx.x, cnt - 1)) * P.Wmax;
-  __syncthreads();
-  group_masks(src, cnt, d.n, mask);
-  __syncthreads();
-  rescore_group<long long>(P.Jq + d.off_mat, P.hq + d.off_vec, d.n, d.n_pad, mask, red, cnt, gridDim.y,
-                           reinterpret_cast<long long*>(P.rs_acc) + 2 * b0 * gridDim.y, gridDim.y,
-                           [&](int g, long long Eq) { init_energy_out(P, d, b0 + g, Eq); });
-}
-
-__global__ void k_init_energy_finish(DevPtrs P, int b0, int nb, int parts) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= nb) return;
-  const long long b = (long long)b0 + x;
-  init_energy_out(P, P.inst[b / P.R], b, rs_energy(reinterpret_cast<const long long*>(P.rs_acc) + 2 * b * parts, parts));
-}
-
-cudaError_t launch_init_energy(const DevPtrs& P, int inst0, int n_inst, int max_n, cudaStream_t s) {
-  if (n_inst <= 0) return cudaSuccess;
-  const int ng = (P.R + kRG - 1) / kRG;
-  const int parts = rescore_parts(P, n_inst * ng, max_n, true);
-  const long long b0 = (long long)inst0 * P.R, nb = (long long)n_inst * P.R;
-  const size_t sm = rescore_smem(P.NP, 8);
-  if (sm > 48 * 1024) cudaFuncSetAttribute(k_init_energy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_init_energy<<<dim3(n_inst * ng, parts), 256, sm, s>>>(P, inst0, ng);
-  if (parts > 1) k_init_energy_finish<<<(int)((nb + 255) / 256), 256, 0, s>>>(P, (int)b0, (int)nb, parts);
-  return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------- every instance's merged list
-// Block (inst, group) for the states group * kRG ... of the first min(k, count of inst) of the
-// merged list: their bits into out[inst][r][Wmax] and their energies, rescored as above, into
-// E[inst][r]. The row parts: the exact form's when every instance is rescored exactly (split
-// modes, on the grid), else the FP64 form's.
-__global__ void __launch_bounds__(256) k_topk_all(DevPtrs P, int k, int all_exact, uint64_t* out, double* E) {
-  const int ng = (k + kRG - 1) / kRG;
-  const int inst = blockIdx.x / ng, g0 = (blockIdx.x % ng) * kRG;
-  const int cnt = min(kRG, min(k, P.mrg_count[inst]) - g0);
-  if (cnt <= 0) return;
-  const InstDesc d = P.inst[inst];
-  const bool exact = P.mode != QIS_FP64 && !d.rounded;
-  // this instance's parts: the grid's when every instance is exact, else its FP64 number
-  const int parts = all_exact ? (int)gridDim.y : fp64_parts(d.n);
-  if ((int)blockIdx.y >= parts) return;
-  extern __shared__ __align__(16) unsigned char rsm[];
-  long long* redq = reinterpret_cast<long long*>(rsm);
-  double* redd = reinterpret_cast<double*>(rsm);
-  uint16_t* mask = reinterpret_cast<uint16_t*>(redq + 9 * (kRG + 1));
-  __shared__ const uint64_t* src[kRG];
-  if (threadIdx.x < kRG) {
-    const int ref = P.mrg_ref[inst * P.K1 + g0 + min((int)threadIdx.x, cnt - 1)];
-    src[threadIdx.x] = P.lst_bits + (long long)ref * P.Wmax;
-  }
-  __syncthreads();
-  if (blockIdx.y == 0)
-    for (int x = threadIdx.x; x < cnt * P.Wmax; x += blockDim.x) {
-      const int g = x / P.Wmax, w = x - g * P.Wmax;
-      out[((long long)inst * k + g0 + g) * P.Wmax + w] = (w < d.W) ? src[g][w] : 0ull;
-    }
-  group_masks(src, cnt, d.n, mask);
-  __syncthreads();
-  const long long o = (long long)inst * k + g0;
-  const int PS = gridDim.y;
-  if (exact)
-    rescore_group<long long>(P.Jq + d.off_mat, P.hq + d.off_vec, d.n, d.n_pad, mask, redq, cnt, parts,
-                             reinterpret_cast<long long*>(P.rs_acc) + 2 * o * PS, PS,
-                             [&](int g, long long Eq) { E[o + g] = (double)Eq * d.inv_scale; });
-  else
-    rescore_group<double>(P.J64 + d.off_mat, P.h64 + d.off_vec, d.n, d.n_pad, mask, redd, cnt, parts,
-                          reinterpret_cast<double*>(P.rs_acc) + 2 * o * PS, PS,
-                          [&](int g, double Ev) { E[o + g] = Ev; });
-}
-
-__global__ void k_topk_all_finish(DevPtrs P, int k, int all_exact, int PS, double* E) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int inst = x / k, r = x - inst * k;
-  if (inst >= P.n_inst || r >= min(k, P.mrg_count[inst])) return;
-  const InstDesc d = P.inst[inst];
-  const int parts = all_exact ? PS : fp64_parts(d.n);
-  if (parts == 1) return;   // written by the rescoring block itself
-  if (P.mode != QIS_FP64 && !d.rounded)
-    E[x] = (double)rs_energy(reinterpret_cast<const long long*>(P.rs_acc) + 2ll * x * PS, parts) * d.inv_scale;
-  else
-    E[x] = rs_energy(reinterpret_cast<const double*>(P.rs_acc) + 2ll * x * PS, parts);
-}
-
-cudaError_t launch_topk_all(const DevPtrs& P, int k, bool all_exact, int max_n, uint64_t* out, double* E,
-                            cudaStream_t s) {
-  if (k <= 0 || P.n_inst <= 0) return cudaSuccess;
-  const int groups = P.n_inst * ((k + kRG - 1) / kRG);
-  const int parts = rescore_parts(P, groups, max_n, all_exact);
-  const long long nstates = (long long)P.n_inst * k;
-  const size_t sm = rescore_smem(P.NP, 8);
-  if (sm > 48 * 1024) cudaFuncSetAttribute(k_topk_all, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_topk_all<<<dim3(groups, parts), 256, sm, s>>>(P, k, all_exact ? 1 : 0, out, E);
-  if (parts > 1) k_topk_all_finish<<<(int)((nstates + 255) / 256), 256, 0, s>>>(P, k, all_exact ? 1 : 0, parts, E);
   return cudaGetLastError();
 }
 
