@@ -139,7 +139,7 @@ int qis_instance_n(qis_ctx* ctx, int instance_id, int* n);
  * The searches start (initial energies, lists) with one launch for every instance set since,
  * at the next call that reads or advances them; the caller's buffer is free on return. When
  * that call is qis_iterate with at least one iteration of the fused search kernel (the exact
- * modes with a padded n up to 1024), the initial energies are formed in the first iteration
+ * modes; a padded n up to 1024, or single flips), the initial energies are formed in the first iteration
  * from the initial states' exact local fields, E = (sum_i s_i f_i + sum_i s_i h_i) / 2 (Eq. 1
  * with f = J s + h), which that iteration computes anyway; every other call forms them by a
  * separate rescoring launch. Both give the same exact value. */
@@ -256,6 +256,9 @@ int qis_candidate_count(qis_ctx* ctx, uint64_t* pairs, uint64_t* singles);
  *                  every iteration (the per-kernel form); 2 = dense register tiles (shaped by
  *                  scan_chunk_nc and scan_search_group); 0 = automatic (1 where allowed, else 2;
  *                  the environment variable QIS_DENSE_SCAN=1 makes 2 the default).
+ *                  QIS_FLIPS_SINGLE has no pairs to scan: its search kernel runs every iteration
+ *                  of a call in one block per search at any n (K+1 <= 256, fields by update), 3
+ *                  (where it is allowed) and QIS_FUSED=0 the per-kernel form.
  *                  Every form gives the same kept lists. QIS_FP64 scans every pair in its plain
  *                  FP64 form whatever this says; qis_get_tuning reports 2 there. */
 typedef struct {

@@ -87,6 +87,7 @@ struct qis_ctx {
   bool no_fused = false;                    // QIS_FUSED=0: the per-kernel form of every iteration
   cudaGraphExec_t graph_exec = nullptr;     // one iteration, captured for the current instances
   int graph_n = 0;                          // fused form: the iteration count the graph was captured for
+  uint64_t graph_launches = 0;              // fused form: kernels in the graph
   int last_n = 0;                           // fused form: the iteration count of the previous call
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev[8];
   size_t ev_used[8] = {0};
@@ -231,7 +232,11 @@ static bool sparse_allowed(const qis_ctx* ctx) { return ctx->mode != QIS_FP64 &&
 static bool sparse_scan(const qis_ctx* ctx) { return sparse_allowed(ctx) && ctx->tune.pair_scan != 2; }
 // The fused search kernel: the output-sensitive scan (pair_scan 0 or 1) with fields by update,
 // a padded n and a list small enough for its shared-memory arrays (QIS_FUSED=0 turns it off).
+// Single flips have no pairs to scan: their kernel takes any n, and only pair_scan 3 (the
+// per-kernel form) is read.
 static bool fused_search(const qis_ctx* ctx) {
+  if (ctx->cfg.flips == QIS_FLIPS_SINGLE)
+    return ctx->P.pw_n > 0 && ctx->tune.pair_scan != 3 && ctx->P.inc_on && !ctx->fields_simt && !ctx->no_fused;
   return sparse_scan(ctx) && ctx->tune.pair_scan != 3 && ctx->NP <= kSearchMaxNP && ctx->K1 <= kSearchMaxK1 &&
          ctx->P.inc_on && !ctx->fields_simt && !ctx->no_fused;
 }
@@ -251,7 +256,11 @@ int launch_iterations_fused(qis_ctx* ctx, int n, cudaStream_t s) {
   LAUNCH(launch_fields_tc(P, ctx->D16, P.S16, ctx->max_inst, ctx->digits_used, P.gemm_nt, s));
   CK(prof_end(ctx, 1));
   CK(prof_begin(ctx, 5));
-  LAUNCH(launch_search(P, n, s));
+  if (ctx->cfg.flips == QIS_FLIPS_SINGLE) {
+    for (int i = 0; i < n; i += P.pw_n) LAUNCH(launch_single(P, std::min(n - i, P.pw_n), i == 0, s));
+  } else {
+    LAUNCH(launch_search(P, n, s));
+  }
   CK(prof_end(ctx, 5));
   return 0;
 }
@@ -435,6 +444,12 @@ int qis_create(const qis_config* cfg, qis_ctx** out) {
     ALLOC(P.lst_used, B * K1);
     ALLOC(P.lst_ord, B * K1);
     ALLOC(P.lst_count, B);
+    P.pw_n = 0;
+    if (ctx->mode != QIS_FP64 && ctx->cfg.flips == QIS_FLIPS_SINGLE && ctx->K1 <= kSearchMaxK1) {
+      // the parents' words of a launch's iterations: as many as fit in 1 GiB, 8 .. 128
+      P.pw_n = (int)std::min<size_t>(128, std::max<size_t>(8, (1ull << 30) / (B * W * sizeof(uint64_t))));
+      ALLOC(P.pw, B * (size_t)P.pw_n * W);
+    }
     ALLOC(P.par_bits, B * W);
     ALLOC(P.par_E, B);
     ALLOC(P.par_q, B);
@@ -507,10 +522,12 @@ int qis_create(const qis_config* cfg, qis_ctx** out) {
       m = std::max<size_t>(m, (size_t)ctx->scratch_states);
       ALLOC(P.en_acc, 2 * m);
       ALLOC(P.en_left, m / 128 + (size_t)ctx->max_inst + 1);
+      CK(cudaDeviceGetAttribute(&P.sms, cudaDevAttrMultiProcessorCount, ctx->cfg.device));
     }
     // Zobrist keys of the sites (SplitMix64 stream with a fixed key)
     std::vector<uint64_t> z(kMaxN);
-    for (int i = 0; i < kMaxN; ++i) z[i] = splitmix64(0x2F0A7B6C5D4E3F21ull, (uint64_t)i);
+    for (int i = 0; i < kMaxN; ++i)   // the site itself in the low bits (qis_single.cu reads it there)
+      z[i] = (splitmix64(0x2F0A7B6C5D4E3F21ull, (uint64_t)i) & ~(uint64_t)kSiteMask) | (uint64_t)i;
     CK(cudaMemcpy(ctx->zob, z.data(), kMaxN * sizeof(uint64_t), cudaMemcpyHostToDevice));
     // kernel attributes for the large dynamic shared-memory users
     CK(cudaDeviceSynchronize());
@@ -987,7 +1004,10 @@ int qis_iterate(qis_ctx* ctx, int n_iters, int* n_active) {
       if (!ctx->graph_exec) {
         cudaGraph_t g = nullptr;
         CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+        const uint64_t before = ctx->launches;
         const int rc = launch_iterations_fused(ctx, n_iters, s);
+        ctx->graph_launches = ctx->launches - before;
+        ctx->launches = before;   // counted at each replay below
         cudaError_t ec = cudaStreamEndCapture(s, &g);
         if (rc) {
           if (g) cudaGraphDestroy(g);
@@ -998,10 +1018,9 @@ int qis_iterate(qis_ctx* ctx, int n_iters, int* n_active) {
         cudaGraphDestroy(g);
         CK(ec);
         ctx->graph_n = n_iters;
-        ctx->launches -= 4;   // counted at each replay below
       }
       CK(cudaGraphLaunch(ctx->graph_exec, s));
-      ctx->launches += 4;
+      ctx->launches += ctx->graph_launches;
     } else {
       const int rc = launch_iterations_fused(ctx, n_iters, s);
       if (rc) return rc;
@@ -1687,7 +1706,7 @@ int qis_autotune(qis_ctx* ctx, int iters, qis_tuning* best, double* best_ms) {
   // coordinate search: scan form, then chunk width and search group (the dense form's
   // shapes), GEMM tile, each with the others fixed
   cur.pair_scan = sparse_scan(ctx) ? 1 : 2;
-  if (sparse_allowed(ctx)) {
+  if (sparse_allowed(ctx) && ctx->cfg.flips != QIS_FLIPS_SINGLE) {
     qis_tuning t = cur;
     t.pair_scan = 3 - cur.pair_scan;
     consider(t);

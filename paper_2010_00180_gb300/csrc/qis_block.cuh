@@ -317,5 +317,68 @@ static __device__ __forceinline__ int sparse_bucket(float x, float lo, float inv
   return f < (float)kSparseNB ? max(0, (int)f) : kSparseNB - 1;
 }
 
+__host__ __device__ inline int align_up(int x, int a) { return (x + a - 1) / a * a; }
+
+constexpr int kMBits = 7, kMB = 1 << kMBits;   // buckets of the merge's new keys
+
+// More kept candidates than the bucket ranking takes at once (rare): keep the K+1 lowest keys
+// (ties included), compacted in place; returns their number. Out of line.
+static __device__ __noinline__ int keep_lowest(unsigned long long* sk, unsigned long long* se, int nv, int K1,
+                                               int* rhist, int* wsum) {
+  const unsigned long long x = radix_select<unsigned long long>(sk, nv, K1 - 1, rhist);
+  int kept = 0;
+  for (int u0 = 0; u0 < nv; u0 += blockDim.x) {
+    const int e = u0 + threadIdx.x;
+    unsigned long long kk = 0, ee = 0;
+    bool keep = false;
+    if (e < nv) {
+      kk = sk[e];
+      ee = se[e];
+      keep = kk <= x;
+    }
+    int total;
+    const int pos = kept + block_exclusive_sum(keep ? 1 : 0, wsum, &total);
+    if (keep) {
+      sk[pos] = kk;
+      se[pos] = ee;
+    }
+    kept += total;
+    __syncthreads();
+  }
+  return kept;
+}
+
+// (key, entry) sort of nv candidates in place, any size (rare: more than the bucket ranking
+// takes after keep_lowest, i.e. many equal keys). Out of line.
+static __device__ __noinline__ void sort_pairs_any(unsigned long long* sk, unsigned long long* se, int nv) {
+  const int m2 = next_pow2(nv);
+  for (int x = nv + threadIdx.x; x < m2; x += blockDim.x) {
+    sk[x] = ~0ull;
+    se[x] = ~0ull;
+  }
+  __syncthreads();
+  bitonic_sort_smem(sk, se, m2);
+}
+
+// Exact energy E 2^q of an initial state whose energy the search initialisation left to this
+// kernel, from the exact fields of its first iteration (Eq. 1): with f = J s + h,
+// sum_i s_i f_i = 2 sum_{i<j} J_ij s_i s_j + sum_i h_i s_i, so E = (sum_i s_i f_i + sum_i s_i h_i) / 2,
+// and s_i f_i = -aq_i / 2. Both halvings are exact (aq_i is even; the sum is twice an integer).
+// red: blockDim.x / 32 free words of shared memory. Out of line (once per search and run).
+static __device__ __noinline__ long long initial_energy(const DevPtrs& P, const InstDesc& d, const uint64_t* pb,
+                                                        const long long* aq, long long* red) {
+  long long acc = 0;
+  for (int i = threadIdx.x; i < d.n; i += blockDim.x) {
+    const long long hq = P.hq[d.off_vec + i];
+    acc += (sigma_of(pb, i) ? -hq : hq) - aq[i] / 2;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  long long tot = 0;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];
+  return tot / 2;
+}
 
 }  // namespace qis

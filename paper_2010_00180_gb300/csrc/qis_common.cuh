@@ -14,6 +14,7 @@ constexpr int kTile = 64;        // scan tile edge (sites)
 constexpr int kPad = 128;        // n is padded to a multiple of this (tensor-core M tile)
 constexpr int kMaxDigits = 5;    // 12-bit signed digits (base 4096) of the fixed-point couplings
 constexpr int kMaxN = 16384;
+constexpr int kSiteMask = kMaxN - 1;   // the low bits of a site's Zobrist key hold the site
 constexpr int kScan64Group = 4;  // searches per block of the FP64 pair scan
 
 // Device error flags (bit mask in ctx status word).
@@ -65,6 +66,8 @@ struct DevPtrs {
   uint64_t* lst_stamp;    // [b][K1]
   uint64_t* lst_hash;     // [b][K1]
   uint8_t* lst_used;      // [b][K1]
+  uint64_t* pw;           // [b][pw_n][Wmax] parents' words of the iterations of a launch (single flips)
+  int pw_n;               // iterations per launch of the single-flip search kernel
   int* lst_ord;           // [b][K1] slot of rank r
   int* lst_count;         // [b]
   uint64_t* par_bits;     // [b][Wmax]
@@ -117,6 +120,7 @@ struct DevPtrs {
   int* mrg_count;         // [inst]
   unsigned long long* en_acc;   // [states][2] integer sums of the energies from scratch (zero between calls)
   int* en_left;                 // [states / 128, rounded up per instance] blocks done of a state tile (zero between calls)
+  int sms;                      // streaming multiprocessors of the device
 };
 
 __host__ __device__ inline int words_of(int n) { return (n + 63) >> 6; }
@@ -349,6 +353,8 @@ constexpr int kSparseMaxNP = 4096;   // the sparse pair scan's largest padded n 
 constexpr int kSearchMaxNP = 1024;
 constexpr int kSearchMaxK1 = 256;
 cudaError_t launch_search(const DevPtrs& P, int n_iters, cudaStream_t s);
+// Single flips: any padded n, at most P.pw_n iterations per launch.
+cudaError_t launch_single(const DevPtrs& P, int n_iters, int ext, cudaStream_t s);
 size_t search_smem(const DevPtrs& P);
 cudaError_t launch_validate(const DevPtrs& P, int inst, int n, long long off_mat, long long off_vec,
                             double* stats, cudaStream_t s);

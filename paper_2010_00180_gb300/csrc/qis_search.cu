@@ -1,5 +1,5 @@
 // qis_search.cu -- every iteration of one search in one thread block (the fused, persistent
-// form of the iteration of Alg. 3 in the split precision modes).
+// form of the iteration of Alg. 3 in the split precision modes; single flips alone: qis_single.cu).
 //
 // The R searches of an instance, and the instances, share nothing until the Alg. 4 merge, so
 // one block can take one search through all the iterations of a qis_iterate call without ever
@@ -42,9 +42,6 @@ struct SearchLayout {
 };
 
 constexpr int kSSV = 512;   // survivors held in shared memory (more go to the global buffer)
-constexpr int kMBits = 7, kMB = 1 << kMBits;   // buckets of the merge's new keys
-
-__host__ __device__ inline int align_up(int x, int a) { return (x + a - 1) / a * a; }
 
 __host__ __device__ inline SearchLayout search_layout(int NP, int Wmax, int K1, int cap, int merge_cand) {
   SearchLayout L;
@@ -108,67 +105,8 @@ static __device__ __noinline__ void fields_full(const DevPtrs& P, const InstDesc
   }
 }
 
-// More kept candidates than the bucket ranking takes at once (rare): keep the K+1 lowest keys
-// (ties included), compacted in place; returns their number. Out of line.
-static __device__ __noinline__ int keep_lowest(unsigned long long* sk, unsigned long long* se, int nv, int K1,
-                                               int* rhist, int* wsum) {
-  const unsigned long long x = radix_select<unsigned long long>(sk, nv, K1 - 1, rhist);
-  int kept = 0;
-  for (int u0 = 0; u0 < nv; u0 += blockDim.x) {
-    const int e = u0 + threadIdx.x;
-    unsigned long long kk = 0, ee = 0;
-    bool keep = false;
-    if (e < nv) {
-      kk = sk[e];
-      ee = se[e];
-      keep = kk <= x;
-    }
-    int total;
-    const int pos = kept + block_exclusive_sum(keep ? 1 : 0, wsum, &total);
-    if (keep) {
-      sk[pos] = kk;
-      se[pos] = ee;
-    }
-    kept += total;
-    __syncthreads();
-  }
-  return kept;
-}
-
-// (key, entry) sort of nv candidates in place, any size (rare: more than the bucket ranking
-// takes after keep_lowest, i.e. many equal keys). Out of line.
-static __device__ __noinline__ void sort_pairs_any(unsigned long long* sk, unsigned long long* se, int nv) {
-  const int m2 = next_pow2(nv);
-  for (int x = nv + threadIdx.x; x < m2; x += blockDim.x) {
-    sk[x] = ~0ull;
-    se[x] = ~0ull;
-  }
-  __syncthreads();
-  bitonic_sort_smem(sk, se, m2);
-}
-
-// Exact energy E 2^q of an initial state whose energy the search initialisation left to this
-// kernel, from the exact fields of its first iteration (Eq. 1): with f = J s + h,
-// sum_i s_i f_i = 2 sum_{i<j} J_ij s_i s_j + sum_i h_i s_i, so E = (sum_i s_i f_i + sum_i s_i h_i) / 2,
-// and s_i f_i = -aq_i / 2. Both halvings are exact (aq_i is even; the sum is twice an integer).
-// red: kSNT / 32 free words of shared memory. Out of line (once per search and run).
-static __device__ __noinline__ long long initial_energy(const DevPtrs& P, const InstDesc& d, const uint64_t* pb,
-                                                        const long long* aq, long long* red) {
-  long long acc = 0;
-  for (int i = threadIdx.x; i < d.n; i += blockDim.x) {
-    const long long hq = P.hq[d.off_vec + i];
-    acc += (sigma_of(pb, i) ? -hq : hq) - aq[i] / 2;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  long long tot = 0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];
-  return tot / 2;
-}
-
-// FL: flip set (QIS_FLIPS_*). One block of kSNT threads per search; n_iters >= 1.
+// FL: flip set, QIS_FLIPS_SINGLE_PAIR or QIS_FLIPS_EXCHANGE (single flips alone: qis_single.cu). One
+// block of kSNT threads per search; n_iters >= 1.
 template <int FL>
 __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_iters) {
   constexpr bool EX = FL == QIS_FLIPS_EXCHANGE;
@@ -386,7 +324,7 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
     int nu = 0;
     if (EX)
       for (int w = 0; w < W; ++w) nu += __popcll(pb[w]);
-    const long long Ccand = FL == QIS_FLIPS_SINGLE ? (long long)n : EX ? (long long)nu * (n - nu) : (long long)n * (n + 1) / 2;
+    const long long Ccand = EX ? (long long)nu * (n - nu) : (long long)n * (n + 1) / 2;
     if (Ccand > k && k <= kSubMax) {
       // the bound's histograms (cleared before the fields barrier): site bins, the second spin
       // class's site bins (exchanges), the subset values' counts and their per-bin maxima
@@ -397,9 +335,7 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
       int* sites = reinterpret_cast<int*>(vmax + 256);                 // [kSubSites]
       const int want = min(3 * k, kSubMax);
       int t0 = 0, t1 = 0;
-      if (FL == QIS_FLIPS_SINGLE) {
-        t0 = k;
-      } else if (EX) {
+      if (EX) {
         const int nd = n - nu;
         int m0 = max(1, (int)sqrtf((float)want));
         while (m0 * m0 < want) ++m0;
@@ -441,8 +377,8 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
       // clamp to the end bins, which keeps the binning monotone)
       const float cut0 = __fadd_ru(amin, __fdiv_ru((float)(s_bin + 2), scale));
       const float cut1 = EX ? __fadd_ru(amin, __fdiv_ru((float)(s_bin2 + 2), scale)) : cut0;
-      const float hi_v = FL == QIS_FLIPS_SINGLE ? cut0 : __fadd_ru(__fadd_ru(cut0, cut1), d.j4max);
-      const float lo_b = FL == QIS_FLIPS_SINGLE ? amin : __fsub_rd(__fadd_rd(amin, amin), d.j4max);
+      const float hi_v = __fadd_ru(__fadd_ru(cut0, cut1), d.j4max);
+      const float lo_b = __fsub_rd(__fadd_rd(amin, amin), d.j4max);
       const float scale_v = 255.99f / fmaxf(hi_v - lo_b, 1e-30f);
       auto put_value = [&](float v) {
         const int bin = min(255, max(0, (int)((v - lo_b) * scale_v)));
@@ -453,15 +389,11 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
         const int c = EX ? sigma_of(pb, i) : 0;
         if (bin_of(i) > (c ? s_bin2 : s_bin)) continue;
         const int slot = atomicAdd(c ? &s_n2 : &s_nsites, 1);
-        if (FL == QIS_FLIPS_SINGLE) {
-          if (slot < kSubMax) put_value(as[i].x);
-        } else if (slot < (c ? t1 : lim0)) {
-          sites[c ? lim0 + slot : slot] = i;
-        }
+        if (slot < (c ? t1 : lim0)) sites[c ? lim0 + slot : slot] = i;
       }
       __syncthreads();
       const int mm = min(s_nsites, lim0), m2 = min(s_n2, t1);
-      const int M = FL == QIS_FLIPS_SINGLE ? min(s_nsites, kSubMax) : EX ? mm * m2 : mm + mm * (mm - 1) / 2;
+      const int M = EX ? mm * m2 : mm + mm * (mm - 1) / 2;
       auto member = [&](int q, int& i, int& j) {   // exchanges: (class 0 site, class 1 site)
         i = sites[q / m2];
         j = sites[lim0 + q % m2];
@@ -471,7 +403,7 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
           j = tmp;
         }
       };
-      if (M >= k && FL != QIS_FLIPS_SINGLE) {
+      if (M >= k) {
         if (!EX) {
           // the subset's singles, then its pairs row by row: warp w takes the rows x = w, w + 4,
           // ..., its lanes the partners y > x (no index decoding; a warp reads one row of 4J~)
@@ -529,18 +461,9 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
       const float delta = __fmul_ru(big, 0x1p-21f);
       thr = fminf(__fadd_ru(tE, delta), __fadd_ru(Uf, 2.f * delta));
     }
-    // single flips: dE_i = a_i (not candidates under exchanges; with pairs, tested in the
-    // live-row pass below)
-    if (FL == QIS_FLIPS_SINGLE) {
-      for (int i = tid; i < n; i += kSNT) {
-        if (as[i].x <= thr) {
-          const int slot = atomicAdd(&s_ns, 1);
-          put_surv(slot, surv_entry(i, -1));
-        }
-      }
-    }
-    // ---------------------------------------------------------------- scan (pairs)
-    if (FL != QIS_FLIPS_SINGLE) {
+    // ---------------------------------------------------------------- scan (pairs; the single
+    // flips, dE_i = a_i, no candidates under exchanges, are tested in the live-row pass)
+    {
       int* li = reinterpret_cast<int*>(scr);   // [NP] live rows
       int* pc = li + NP;                       // [NP] their rm, then list offsets
       int* cj = pc + NP;                       // [NP] columns in bucket order
@@ -963,17 +886,15 @@ size_t search_smem(const DevPtrs& P) { return (size_t)search_layout(P.NP, P.Wmax
 cudaError_t launch_search(const DevPtrs& P, int n_iters, cudaStream_t s) {
   if (n_iters <= 0 || P.B == 0) return cudaSuccess;
   const size_t sm = search_smem(P);
-  static size_t attr[3] = {0, 0, 0};
-  const int fl = P.flips;
-  if (attr[fl] < sm) {
-    cudaError_t e = fl == QIS_FLIPS_SINGLE ? cudaFuncSetAttribute(k_search<QIS_FLIPS_SINGLE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)
-                  : fl == QIS_FLIPS_EXCHANGE ? cudaFuncSetAttribute(k_search<QIS_FLIPS_EXCHANGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)
-                                             : cudaFuncSetAttribute(k_search<QIS_FLIPS_SINGLE_PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  static size_t attr[2] = {0, 0};
+  const int ex = P.flips == QIS_FLIPS_EXCHANGE;
+  if (attr[ex] < sm) {
+    const cudaError_t e = ex ? cudaFuncSetAttribute(k_search<QIS_FLIPS_EXCHANGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)
+                             : cudaFuncSetAttribute(k_search<QIS_FLIPS_SINGLE_PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    attr[fl] = sm;
+    attr[ex] = sm;
   }
-  if (fl == QIS_FLIPS_SINGLE) k_search<QIS_FLIPS_SINGLE><<<P.B, kSNT, sm, s>>>(P, n_iters);
-  else if (fl == QIS_FLIPS_EXCHANGE) k_search<QIS_FLIPS_EXCHANGE><<<P.B, kSNT, sm, s>>>(P, n_iters);
+  if (ex) k_search<QIS_FLIPS_EXCHANGE><<<P.B, kSNT, sm, s>>>(P, n_iters);
   else k_search<QIS_FLIPS_SINGLE_PAIR><<<P.B, kSNT, sm, s>>>(P, n_iters);
   return cudaGetLastError();
 }
