@@ -370,7 +370,9 @@ int qis_init_states_learned(qis_ctx* ctx, int instance_id, qis_mlp* m);
  * the CUDA allocator, plugins whose process owns device memory through another pool).
  *
  * For one parent state psi of an n-spin instance it evaluates every single flip and every
- * pair flip with the library's FP64 arithmetic (E' = E(psi) + dE, as in QIS_FP64) and writes
+ * pair flip with the library's FP64 arithmetic (E' = E(psi) + dE, fields and dE as in QIS_FP64;
+ * E(psi) summed from the fields, which for couplings off any grid can differ from the
+ * pair-by-pair sum of QIS_FP64 in its last bits) and writes
  * the k candidates of lowest (E', c), ascending, c the candidate index of the conventions
  * above. Unlike every other entry point, all pointers here are DEVICE pointers owned by the
  * caller:
