@@ -942,12 +942,11 @@ int qis_init_states_learned(qis_ctx* ctx, int instance_id, qis_mlp* m) {
                      sizeof(uint64_t) * (size_t)ctx->R * ctx->Wmax, ctx->stream));
   CK(mlp_propose_states(m, ctx->J64 + d.off_mat, d.n_pad, ctx->h64 + d.off_vec, d.n, ctx->R, key,
                         ctx->P.init_bits + (size_t)d.first_search * ctx->Wmax, ctx->Wmax, ctx->stream));
-  ctx->launches += 5;
+  ctx->launches += 3;
   ctx->init_pending[instance_id] = 1;
   ctx->e0_valid[instance_id] = 0;
   ctx->inst_ready[instance_id] = 1;
   ctx->merged_fresh = false;
-  CK(cudaStreamSynchronize(ctx->stream));
   return 0;
 }
 

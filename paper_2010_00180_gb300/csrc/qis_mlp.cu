@@ -15,6 +15,7 @@
 #include <cuda_bf16.h>
 #include <math.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -25,32 +26,49 @@ namespace qis {
 constexpr int kF = 8;   // features per site
 
 // ---------------------------------------------------------------- features
-// J row i at J + i * stride (n valid entries), h[0..n).
-__global__ void k_mlp_features(const double* J, long long stride, const double* h, int n, float* X) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+// J row i at J + i * stride (n valid entries), h[0..n). A warp per row, its lanes over the columns
+// (a thread per row read them uncoalesced, a chain of n FP64 additions: 148 us at n = 300, now 4).
+// |v|, the signs of h and the extrema are integer operations on the bits (FP64 has two lanes per SM).
+__global__ void __launch_bounds__(256) k_mlp_features(const double* J, long long stride, const double* h, int n, float* X) {
+  const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (i >= n) return;   // warp-uniform
   const double* row = J + (long long)i * stride;
-  double s = 0, a = 0, q = 0, mx = -INFINITY, mn = INFINITY, jh = 0, js = 0;
-  for (int j = 0; j < n; ++j) {
-    const double v = row[j];
+  double s = 0, a = 0, q = 0, jh = 0, js = 0;
+  unsigned long long mx = 0, mn = ~0ull;   // order keys of the extrema over j != i
+#pragma unroll 4
+  for (int j = lane; j < n; j += 32) {
+    const double v = row[j], hj = h[j];
     s += v;
     a += fabs(v);
-    q += v * v;
-    jh += v * h[j];
-    js += v * (double)((h[j] > 0) - (h[j] < 0));
+    q = fma(v, v, q);
+    jh = fma(v, hj, jh);
+    const long long hb = __double_as_longlong(hj);
+    if (hb << 1) js += hb < 0 ? -v : v;   // h_j != 0
+    const unsigned long long k = dkey(v);
     if (j != i) {
-      mx = fmax(mx, v);
-      mn = fmin(mn, v);
+      mx = max(mx, k);
+      mn = min(mn, k);
     }
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    s += __shfl_xor_sync(0xffffffffu, s, o);
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    q += __shfl_xor_sync(0xffffffffu, q, o);
+    jh += __shfl_xor_sync(0xffffffffu, jh, o);
+    js += __shfl_xor_sync(0xffffffffu, js, o);
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+  }
+  if (lane) return;
   const double rn = sqrt((double)n);
   float* x = X + (long long)i * kF;
   x[0] = (float)h[i];
   x[1] = (float)(s / rn);
   x[2] = (float)(a / n);
   x[3] = (float)sqrt(q / n);
-  x[4] = (float)mx;
-  x[5] = (float)mn;
+  x[4] = (float)dkey_inv(mx);
+  x[5] = (float)dkey_inv(mn);
   x[6] = (float)(jh / rn);
   x[7] = (float)(js / rn);
 }
@@ -60,125 +78,292 @@ __global__ void k_mlp_labels(const uint64_t* bits, int n, float* y) {
   if (i < n) y[i] = ((bits[i >> 6] >> (i & 63)) & 1ull) ? 0.f : 1.f;   // y = 1 <=> s_i = +1
 }
 
-// ---------------------------------------------------------------- GEMM (SIMT, FP32 accumulate)
-// C[M x N] (+)= op(A)[M x K] op(B)[K x N]; A stored [M x K] (TA: [K x M]), B stored [K x N]
-// (TB: [N x K]); row-major. Optional epilogue: C = relu(C + bias). gridDim.z splits K and
-// accumulates with atomics (C must be zero then).
-template <bool TA, bool TB, typename TBt, bool BIAS_RELU>
-__global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, const float* A, const TBt* B, float* C,
-                                              const float* bias) {
-  __shared__ float As[16][64 + 4];
-  __shared__ float Bs[16][64 + 4];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-  const int kchunk = (K + gridDim.z - 1) / gridDim.z;
-  const int k_lo = blockIdx.z * kchunk, k_hi = min(K, k_lo + kchunk);
-  float acc[4][4] = {};
-  for (int k0 = k_lo; k0 < k_hi; k0 += 16) {
-    for (int e = threadIdx.x; e < 16 * 64; e += 256) {
-      const int kk = e / 64, mm = e % 64;       // As[kk][mm] = op(A)[m0+mm][k0+kk]
-      const int m = m0 + mm, k = k0 + kk;
-      float v = 0.f;
-      if (m < M && k < k_hi) v = TA ? A[(long long)k * M + m] : A[(long long)m * K + k];
-      As[kk][mm] = v;
-      const int nn = e % 64, n = n0 + nn;       // Bs[kk][nn] = op(B)[k0+kk][n0+nn]
-      float w = 0.f;
-      if (n < N && k < k_hi) {
-        if constexpr (TB) w = (float)B[(long long)n * K + k];
-        else w = (float)B[(long long)k * N + n];
+// ---------------------------------------------------------------- network
+// out = in W for TM rows of activations in shared memory (in: TM x K, row-major) and BF16 weights W
+// (K x H, row-major). A warp takes RT rows x 128 columns, a lane 4 adjacent columns: one weight
+// load per k serves RT rows, the activations are broadcast reads, and every sum is one chain of
+// FP32 fused multiply-adds over k ascending (the logits' bits do not depend on the tile). The
+// next eight rows of W are loaded while the current eight are used. put(row, column, the sums of
+// 4 columns) receives the results; in and the results must not share memory.
+constexpr int kCT = 4;   // columns of a lane
+template <int RT, typename Put>
+static __device__ __forceinline__ void mlp_layer(const float* in, int K, const __nv_bfloat16* __restrict__ W, int H, int TM,
+                                                 Put put) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int CG = (H + 32 * kCT - 1) / (32 * kCT);
+  for (int u = warp; u < TM / RT * CG; u += 8) {
+    const int r0 = u / CG * RT, c = (u % CG) * 32 * kCT + lane * kCT;
+    if (c >= H) continue;   // H is a multiple of 16: a lane's columns are all in or all out
+    float acc[RT][kCT];
+#pragma unroll
+    for (int r = 0; r < RT; ++r)
+#pragma unroll
+      for (int x = 0; x < kCT; ++x) acc[r][x] = 0.f;
+    uint2 w[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) w[k] = *reinterpret_cast<const uint2*>(W + (long long)k * H + c);
+#pragma unroll 1
+    for (int k0 = 0; k0 < K; k0 += 8) {
+      uint2 v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        v[k] = w[k];
+        if (k0 + 8 < K) w[k] = *reinterpret_cast<const uint2*>(W + (long long)(k0 + 8 + k) * H + c);
       }
-      Bs[kk][nn] = w;
+#pragma unroll
+      for (int k4 = 0; k4 < 8; k4 += 4) {
+        float4 a[RT];
+#pragma unroll
+        for (int r = 0; r < RT; ++r) a[r] = *reinterpret_cast<const float4*>(in + (r0 + r) * K + k0 + k4);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const uint32_t* p = reinterpret_cast<const uint32_t*>(&v[k4 + k]);
+          float b[kCT];
+#pragma unroll
+          for (int x = 0; x < kCT; x += 2) {
+            b[x] = __uint_as_float(p[x / 2] << 16);
+            b[x + 1] = __uint_as_float(p[x / 2] & 0xffff0000u);
+          }
+#pragma unroll
+          for (int r = 0; r < RT; ++r) {
+            const float ar = k == 0 ? a[r].x : k == 1 ? a[r].y : k == 2 ? a[r].z : a[r].w;
+#pragma unroll
+            for (int x = 0; x < kCT; ++x) acc[r][x] = fmaf(ar, b[x], acc[r][x]);
+          }
+        }
+      }
     }
+#pragma unroll
+    for (int r = 0; r < RT; ++r) put(r0 + r, c, acc[r]);
+  }
+}
+
+// Everything of a pass but the weight gradients, for TM rows per block: the three layers, the logits,
+// and with labels y the loss (added to *loss) and the gradients of the pre-activations d3, d2, d1
+// (d_l = (d_{l+1} W_{l+1}^T) where h_l > 0, with the transposed weights W2t, W3t), all from one
+// block's shared memory; h1, h2, h3 and d1, d2, d3 are written for the weight gradients. G (grads
+// values, or NULL) is cleared for them.
+// FP32 issue bounds it (M (4 H^2 + ..) multiply-adds); it replaces eleven launches whose tiles of
+// 64 x 64 fed four accumulators per shared-memory read. Loss and gradients of 4096 rows at H = 256
+// from host memory, with the weight gradients' kernel below (which took 3 x 90 us): 542 -> 195 us;
+// warm start of 120 instances of n = 300 and their searches: 44.1 -> 14.7 ms.
+struct MlpNet {
+  const float* P;                   // master parameters (biases are read from it)
+  const __nv_bfloat16 *Pb, *W2t, *W3t;
+  int H, oW1, ob1, oW2, ob2, oW3, ob3, ow4, ob4;
+};
+
+template <int TM, int RT>
+__global__ void __launch_bounds__(256) k_mlp_pass(MlpNet N, int M, const float* X, const float* y, float* z, float* dz,
+                                                  double* loss, float inv_m, float* h1, float* h2, float* h3, float* d1,
+                                                  float* d2, float* d3, float* G, int grads) {
+  extern __shared__ __align__(16) float act[];
+  const int H = N.H, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float* A = act;              // [TM][H]
+  float* B = act + TM * H;     // [TM][H]
+  __shared__ float sdz[TM];
+  __shared__ double sl[TM];
+  const int m0 = blockIdx.x * TM, rows = min(TM, M - m0);
+  if (G)
+    for (int e = blockIdx.x * 256 + tid; e < grads; e += gridDim.x * 256) G[e] = 0.f;
+  for (int e = tid; e < TM * kF; e += 256) B[e] = e < rows * kF ? X[(long long)m0 * kF + e] : 0.f;
+  __syncthreads();
+  // h = relu(in W + b) into `out`, and to global memory for a pass with labels
+  auto forward = [&](const float* in, int K, int oW, int ob, float* out, float* h) {
+    mlp_layer<RT>(in, K, N.Pb + oW, H, TM, [&](int r, int c, const float* s) {
+#pragma unroll
+      for (int x = 0; x < kCT; x += 4) {
+        const float4 b = *reinterpret_cast<const float4*>(N.P + ob + c + x);
+        const float4 v = make_float4(fmaxf(s[x] + b.x, 0.f), fmaxf(s[x + 1] + b.y, 0.f), fmaxf(s[x + 2] + b.z, 0.f),
+                                     fmaxf(s[x + 3] + b.w, 0.f));
+        *reinterpret_cast<float4*>(out + r * H + c + x) = v;
+        if (y && r < rows) *reinterpret_cast<float4*>(h + (long long)(m0 + r) * H + c + x) = v;
+      }
+    });
     __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        a[u] = As[kk][ty * 4 + u];
-        b[u] = Bs[kk][tx * 4 + u];
+  };
+  forward(B, kF, N.oW1, N.ob1, A, h1);
+  forward(A, H, N.oW2, N.ob2, B, h2);
+  forward(B, H, N.oW3, N.ob3, A, h3);
+  // z = h3 w4 + b4, loss and dz = (sigmoid(z) - y) / M: a warp per row
+  const __nv_bfloat16* w4 = N.Pb + N.ow4;
+  for (int r = warp; r < TM; r += 8) {
+    float s = 0.f;
+    for (int k = lane; k < H; k += 32) s = fmaf(A[r * H + k], __bfloat162float(w4[k]), s);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) {
+      const float zz = s + N.P[N.ob4];
+      float g = 0.f;
+      double l = 0.0;
+      if (r < rows) {
+        z[m0 + r] = zz;
+        if (y) {
+          const float yy = y[m0 + r];
+          const float sp = fmaxf(zz, 0.f) + log1pf(expf(-fabsf(zz)));   // softplus
+          l = (double)(sp - yy * zz) * inv_m;
+          g = (1.f / (1.f + expf(-zz)) - yy) * inv_m;
+          dz[m0 + r] = g;
+        }
       }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
+      sdz[r] = g;
+      sl[r] = l;
     }
+  }
+  if (!y) return;
+  __syncthreads();
+  if (tid == 0) {
+    double l = 0.0;
+    for (int r = 0; r < rows; ++r) l += sl[r];
+    atomicAdd(loss, l);
+  }
+  // d3 = outer(dz, w4) where h3 > 0, in the place of h3
+  for (int e = tid; e < TM * H; e += 256) {
+    const int r = e / H, k = e - r * H;
+    const float v = A[e] > 0.f ? sdz[r] * __bfloat162float(w4[k]) : 0.f;
+    A[e] = v;
+    if (r < rows) d3[(long long)m0 * H + e] = v;
+  }
+  __syncthreads();
+  auto backward = [&](const float* in, const __nv_bfloat16* Wt, const float* h, float* out, float* d) {
+    mlp_layer<RT>(in, H, Wt, H, TM, [&](int r, int c, const float* s) {
+#pragma unroll
+      for (int x = 0; x < kCT; x += 4) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < rows) {
+          const long long at = (long long)(m0 + r) * H + c + x;
+          const float4 g = *reinterpret_cast<const float4*>(h + at);   // (this block's own rows)
+          v = make_float4(g.x > 0.f ? s[x] : 0.f, g.y > 0.f ? s[x + 1] : 0.f, g.z > 0.f ? s[x + 2] : 0.f,
+                          g.w > 0.f ? s[x + 3] : 0.f);
+          *reinterpret_cast<float4*>(d + at) = v;
+        }
+        *reinterpret_cast<float4*>(out + r * H + c + x) = v;
+      }
+    });
     __syncthreads();
+  };
+  backward(A, N.W3t, h2, B, d2);
+  backward(B, N.W2t, h1, A, d1);
+}
+
+// ---------------------------------------------------------------- weight gradients
+// dW3 = h2^T d3, dW2 = h1^T d2 (128 x 64 tiles, the rows of the batch split over blockIdx.y, the
+// parts added with vector atomics), db3, db2 (the column sums of the staged d tiles, by the blocks
+// of the first tile row), and in the blocks past those tiles dW1 = X^T d1, db1, dw4 = h3^T dz, db4
+// (128 rows each, a thread per column). G is zero on entry.
+constexpr int kWM = 128, kWN = 64, kWK = 16;
+__global__ void __launch_bounds__(256) k_mlp_wgrad(MlpNet N, int M, int rows_per, const float* X, const float* h1,
+                                                   const float* h2, const float* h3, const float* d1, const float* d2,
+                                                   const float* d3, const float* dz, float* G) {
+  const int H = N.H, tid = threadIdx.x;
+  const int tm = (H + kWM - 1) / kWM, tn = (H + kWN - 1) / kWN, tiles = 2 * tm * tn;
+  __shared__ __align__(16) float As[2][kWK][kWM], Bs[2][kWK][kWN];
+  if ((int)blockIdx.x >= tiles) {
+    // the thin gradients: column c of 128 rows
+    const int x = blockIdx.x - tiles, cgs = (H + 255) / 256;
+    const int c = (x % cgs) * 256 + tid;
+    const int r0 = ((x / cgs) * gridDim.y + blockIdx.y) * 128, r1 = min(M, r0 + 128);
+    if (r0 >= M) return;   // block-uniform
+    float* xs = &As[0][0][0];   // [128][8] features, then [128] dz
+    float* zs = xs + 128 * kF;
+    for (int e = tid; e < (r1 - r0) * kF; e += 256) xs[e] = X[(long long)r0 * kF + e];
+    for (int e = tid; e < r1 - r0; e += 256) zs[e] = dz[r0 + e];
+    __syncthreads();
+    if (c < H) {
+      float g[kF] = {}, gb = 0.f, g4 = 0.f;
+#pragma unroll 4
+      for (int r = r0; r < r1; ++r) {
+        const float d = d1[(long long)r * H + c], hh = h3[(long long)r * H + c];
+        gb += d;
+        g4 = fmaf(hh, zs[r - r0], g4);
+#pragma unroll
+        for (int f = 0; f < kF; ++f) g[f] = fmaf(xs[(r - r0) * kF + f], d, g[f]);
+      }
+#pragma unroll
+      for (int f = 0; f < kF; ++f) atomicAdd(&G[N.oW1 + f * H + c], g[f]);
+      atomicAdd(&G[N.ob1 + c], gb);
+      atomicAdd(&G[N.ow4 + c], g4);
+    }
+    if (x % cgs == 0 && tid < 32) {
+      float s = 0.f;
+      for (int r = tid; r < r1 - r0; r += 32) s += zs[r];
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (tid == 0) atomicAdd(&G[N.ob4], s);
+    }
+    return;
   }
+  const int layer = blockIdx.x / (tm * tn), t = blockIdx.x % (tm * tn);
+  const int m0 = t / tn * kWM, n0 = t % tn * kWN;
+  const float* A = layer ? h1 : h2;
+  const float* D = layer ? d2 : d3;
+  const int r0 = blockIdx.y * rows_per, r1 = min(M, r0 + rows_per);
+  if (r0 >= M) return;   // block-uniform
+  const int tx = tid & 15, ty = tid >> 4;
+  float4 ra[2], rb;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto fetch = [&](int k0) {
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int m = m0 + ty * 4 + u;
-    if (m >= M) continue;
+    for (int u = 0; u < 2; ++u) {
+      const int e = tid + 256 * u, r = k0 + (e >> 5), c = m0 + (e & 31) * 4;
+      ra[u] = r < r1 && c < H ? *reinterpret_cast<const float4*>(A + (long long)r * H + c) : zero;
+    }
+    const int r = k0 + (tid >> 4), c = n0 + (tid & 15) * 4;
+    rb = r < r1 && c < H ? *reinterpret_cast<const float4*>(D + (long long)r * H + c) : zero;
+  };
+  float acc[8][4] = {};
+  float gb = 0.f;
+  fetch(r0);
+  int buf = 0;
+  for (int k0 = r0; k0 < r1; k0 += kWK, buf ^= 1) {
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const int n = n0 + tx * 4 + v;
-      if (n >= N) continue;
-      if constexpr (BIAS_RELU) {
-        C[(long long)m * N + n] = fmaxf(acc[u][v] + bias[n], 0.f);
-      } else if (gridDim.z > 1) {
-        atomicAdd(&C[(long long)m * N + n], acc[u][v]);
-      } else {
-        C[(long long)m * N + n] = acc[u][v];
+    for (int u = 0; u < 2; ++u) {
+      const int e = tid + 256 * u;
+      *reinterpret_cast<float4*>(&As[buf][e >> 5][(e & 31) * 4]) = ra[u];
+    }
+    *reinterpret_cast<float4*>(&Bs[buf][tid >> 4][(tid & 15) * 4]) = rb;
+    __syncthreads();   // (two buffers: the writes of the next step follow this step's reads)
+    if (k0 + kWK < r1) fetch(k0 + kWK);
+#pragma unroll
+    for (int k = 0; k < kWK; ++k) {
+      const float4 b = *reinterpret_cast<const float4*>(&Bs[buf][k][tx * 4]);
+      const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][k][ty * 8]);
+      const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][k][ty * 8 + 4]);
+      const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        acc[u][0] = fmaf(a[u], b.x, acc[u][0]);
+        acc[u][1] = fmaf(a[u], b.y, acc[u][1]);
+        acc[u][2] = fmaf(a[u], b.z, acc[u][2]);
+        acc[u][3] = fmaf(a[u], b.w, acc[u][3]);
       }
     }
+    if (m0 == 0 && tid < kWN)
+#pragma unroll
+      for (int k = 0; k < kWK; ++k) gb += Bs[buf][k][tid];
   }
-}
-
-// z = h3 w4 + b4 (one output), loss and dz = (sigmoid(z) - y) / M
-__global__ void k_mlp_head(int M, int H, const float* h3, const __nv_bfloat16* w4, const float* b4, const float* y,
-                           float* z, float* dz, double* loss, float inv_m) {
-  const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (r >= M) return;
-  float s = 0.f;
-  for (int k = lane; k < H; k += 32) s = fmaf(h3[(long long)r * H + k], __bfloat162float(w4[k]), s);
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) {
-    const float zz = s + b4[0];
-    z[r] = zz;
-    if (y) {
-      const float yy = y[r];
-      const float sp = fmaxf(zz, 0.f) + log1pf(expf(-fabsf(zz)));   // softplus
-      atomicAdd(loss, (double)(sp - yy * zz) * inv_m);
-      dz[r] = (1.f / (1.f + expf(-zz)) - yy) * inv_m;
+  float* g = G + (layer ? N.oW2 : N.oW3);
+  if (n0 + tx * 4 < H)
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int m = m0 + ty * 8 + u;
+      if (m < H)
+        atomicAdd(reinterpret_cast<float4*>(g + (long long)m * H + n0 + tx * 4),
+                  make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]));
     }
-  }
+  if (m0 == 0 && tid < kWN && n0 + tid < H) atomicAdd(&G[(layer ? N.ob2 : N.ob3) + n0 + tid], gb);
 }
 
-// da3 = outer(dz, w4) * (h3 > 0)
-__global__ void k_mlp_head_back(int M, int H, const float* dz, const __nv_bfloat16* w4, const float* h3, float* da) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (long long)M * H) return;
-  const int r = (int)(e / H), k = (int)(e % H);
-  da[e] = h3[e] > 0.f ? dz[r] * __bfloat162float(w4[k]) : 0.f;
+// BF16 copies of parameter e of value p: the flat copy, and the transposed ones of W2 and W3.
+__device__ __forceinline__ void mlp_copy_bf16(const MlpNet& N, int e, float p, __nv_bfloat16* Pb, __nv_bfloat16* W2t,
+                                              __nv_bfloat16* W3t) {
+  const __nv_bfloat16 q = __float2bfloat16_rn(p);
+  Pb[e] = q;
+  const int H = N.H, a = e - N.oW2, b = e - N.oW3;
+  if (a >= 0 && a < H * H) W2t[a % H * H + a / H] = q;
+  if (b >= 0 && b < H * H) W3t[b % H * H + b / H] = q;
 }
 
-__global__ void k_relu_mask(long long count, const float* h, float* d) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < count && !(h[e] > 0.f)) d[e] = 0.f;
-}
-
-// column sums of d [M x N] into g (atomic)
-__global__ void k_colsum(int M, int N, const float* d, float* g) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  const int rows = (M + gridDim.y - 1) / gridDim.y, r0 = blockIdx.y * rows, r1 = min(M, r0 + rows);
-  float s = 0.f;
-  for (int r = r0; r < r1; ++r) s += d[(long long)r * N + n];
-  atomicAdd(&g[n], s);
-}
-
-// dw4 = h3^T dz
-__global__ void k_head_wgrad(int M, int H, const float* h3, const float* dz, float* g) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= H) return;
-  const int rows = (M + gridDim.y - 1) / gridDim.y, r0 = blockIdx.y * rows, r1 = min(M, r0 + rows);
-  float s = 0.f;
-  for (int r = r0; r < r1; ++r) s = fmaf(h3[(long long)r * H + k], dz[r], s);
-  atomicAdd(&g[k], s);
-}
-
-__global__ void k_adam(int count, float* p, const float* g, float* m, float* v, float lr, float b1, float b2, float eps,
-                       float c1, float c2) {
+__global__ void k_adam(MlpNet N, int count, float* p, const float* g, float* m, float* v, float lr, float b1, float b2,
+                       float eps, float c1, float c2, __nv_bfloat16* Pb, __nv_bfloat16* W2t, __nv_bfloat16* W3t) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= count) return;
   const float gg = g[e];
@@ -186,37 +371,37 @@ __global__ void k_adam(int count, float* p, const float* g, float* m, float* v, 
   const float vv = b2 * v[e] + (1.f - b2) * gg * gg;
   m[e] = mm;
   v[e] = vv;
-  p[e] -= lr * (mm / c1) / (sqrtf(vv / c2) + eps);
+  const float x = p[e] - lr * (mm / c1) / (sqrtf(vv / c2) + eps);
+  p[e] = x;
+  mlp_copy_bf16(N, e, x, Pb, W2t, W3t);
 }
 
-__global__ void k_to_bf16(int count, const float* p, __nv_bfloat16* q) {
+__global__ void k_to_bf16(MlpNet N, int count, const float* p, __nv_bfloat16* Pb, __nv_bfloat16* W2t, __nv_bfloat16* W3t) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < count) q[e] = __float2bfloat16_rn(p[e]);
+  if (e < count) mlp_copy_bf16(N, e, p[e], Pb, W2t, W3t);
 }
 
 // Initial states from logits: search 0 takes s_i = sign(z_i) (s_i = +1 when z_i >= 0), search
 // r >= 1 draws s_i = +1 with probability sigmoid(z_i) using value (r n + i) of the SplitMix64
 // stream keyed by `key` (the top 53 bits as a uniform in [0, 1)).
-__global__ void k_mlp_sample(const float* z, int n, int R, uint64_t key, uint64_t* bits, int Wstride) {
-  const int r = blockIdx.y;
-  const int w = blockIdx.x * blockDim.x + threadIdx.x;
-  const int W = (n + 63) >> 6;
-  if (w >= W || r >= R) return;
-  uint64_t word = 0;
-  for (int b = 0; b < 64; ++b) {
-    const int i = w * 64 + b;
-    if (i >= n) break;
-    int sigma;
+// A warp per 32 sites and 8 searches: a lane forms its site's probability once, the ballot of the
+// lanes is half a word (a thread per word drew 64 sites in a row: 62 us at n = 300, R = 32, now 4).
+constexpr int kSampleR = 8;
+__global__ void __launch_bounds__(32) k_mlp_sample(const float* z, int n, int R, uint64_t key, uint64_t* bits, int Wstride) {
+  const int half = blockIdx.x, i = half * 32 + (int)threadIdx.x;
+  const float zi = i < n ? z[i] : 0.f;
+  const double p = 1.0 / (1.0 + exp(-(double)zi));
+  for (int r = blockIdx.y * kSampleR; r < min(R, (int)(blockIdx.y + 1) * kSampleR); ++r) {
+    bool sigma;
     if (r == 0) {
-      sigma = z[i] < 0.f;
+      sigma = zi < 0.f;
     } else {
       const double u = (double)(splitmix64(key, (uint64_t)r * n + i) >> 11) * 0x1.0p-53;
-      const double p = 1.0 / (1.0 + exp(-(double)z[i]));
       sigma = !(u < p);
     }
-    word |= (uint64_t)sigma << b;
+    const unsigned m = __ballot_sync(0xffffffffu, sigma && i < n);
+    if (threadIdx.x == 0) reinterpret_cast<uint32_t*>(bits + (long long)r * Wstride)[half] = m;   // little-endian halves
   }
-  bits[(long long)r * Wstride + w] = word;
 }
 
 }  // namespace qis
@@ -234,15 +419,19 @@ struct qis_mlp {
   float* Mm = nullptr;         // Adam first moment
   float* Vv = nullptr;         // Adam second moment
   __nv_bfloat16* Pb = nullptr; // BF16 copy of all parameters (biases read from P)
+  __nv_bfloat16 *W2t = nullptr, *W3t = nullptr;   // BF16 copies of W2 and W3, transposed
   float* X = nullptr;          // training features [cap x F]
   float* Y = nullptr;          // labels [cap]
   int n_examples = 0;          // rows of X / Y in use
-  float *h1 = nullptr, *h2 = nullptr, *h3 = nullptr, *d1 = nullptr, *d2 = nullptr, *zb = nullptr, *dzb = nullptr;
+  float *h1 = nullptr, *h2 = nullptr, *h3 = nullptr, *d1 = nullptr, *d2 = nullptr, *d3 = nullptr, *zb = nullptr, *dzb = nullptr;
   double* loss = nullptr;
   double* Jst = nullptr;       // staging of one instance's couplings [max_n^2]
   double* hst = nullptr;
   uint64_t* bst = nullptr;
   float* Xq = nullptr;         // query features [max_n x F]
+  float* Yq = nullptr;         // labels of a query
+  cudaEvent_t busy = nullptr;  // the last use of the network's buffers on a context's stream
+  int sms = 0;
   int adam_t = 0;
   std::string err = "no error";
   // offsets into the flattened parameter vector
@@ -281,49 +470,53 @@ int malloc_m(qis_mlp* m, T** p, size_t count) {
     if (rc_) return rc_;                        \
   } while (0)
 
-template <bool TA, bool TB, typename TBt, bool BR>
-void gemm(int M, int N, int K, const float* A, const TBt* B, float* C, const float* bias, int splitk, cudaStream_t s) {
-  dim3 g((N + 63) / 64, (M + 63) / 64, splitk);
-  k_gemm<TA, TB, TBt, BR><<<g, 256, 0, s>>>(M, N, K, A, B, C, bias);
+MlpNet net_of(const qis_mlp* m) {
+  return MlpNet{m->P, m->Pb, m->W2t, m->W3t, m->H, m->oW1, m->ob1, m->oW2, m->ob2, m->oW3, m->ob3, m->ow4, m->ob4};
 }
 
-// forward of rows X[0..M) into h1, h2, h3 and z (and loss / dz when y is given)
-void mlp_forward(qis_mlp* m, int M, const float* X, const float* y, cudaStream_t s) {
-  const int H = m->H;
-  gemm<false, false, __nv_bfloat16, true>(M, H, m->F, X, m->Pb + m->oW1, m->h1, m->P + m->ob1, 1, s);
-  gemm<false, false, __nv_bfloat16, true>(M, H, H, m->h1, m->Pb + m->oW2, m->h2, m->P + m->ob2, 1, s);
-  gemm<false, false, __nv_bfloat16, true>(M, H, H, m->h2, m->Pb + m->oW3, m->h3, m->P + m->ob3, 1, s);
-  k_mlp_head<<<(M + 7) / 8, 256, 0, s>>>(M, H, m->h3, m->Pb + m->ow4, m->P + m->ob4, y, m->zb, m->dzb, m->loss,
-                                         1.f / (float)M);
+template <int TM, int RT>
+cudaError_t pass_tm(qis_mlp* m, int M, const float* X, const float* y, cudaStream_t s) {
+  const size_t sm = (size_t)2 * TM * m->H * sizeof(float);
+  if (sm > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(k_mlp_pass<TM, RT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+  }
+  k_mlp_pass<TM, RT><<<(M + TM - 1) / TM, 256, sm, s>>>(net_of(m), M, X, y, m->zb, m->dzb, m->loss, 1.f / (float)M, m->h1,
+                                                            m->h2, m->h3, m->d1, m->d2, m->d3, y ? m->G : nullptr,
+                                                            m->n_params);
+  return cudaGetLastError();
 }
 
-// gradients of the mean loss over rows X[0..M) into G (zeroed here)
-void mlp_backward(qis_mlp* m, int M, const float* X, cudaStream_t s) {
-  const int H = m->H;
-  cudaMemsetAsync(m->G, 0, sizeof(float) * m->n_params, s);
-  const int sk = (M + 511) / 512;                 // split the row reduction of the weight grads
-  const int ry = (M + 255) / 256;
-  k_head_wgrad<<<dim3((H + 255) / 256, ry), 256, 0, s>>>(M, H, m->h3, m->dzb, m->G + m->ow4);
-  k_colsum<<<dim3(1, ry), 32, 0, s>>>(M, 1, m->dzb, m->G + m->ob4);
-  k_mlp_head_back<<<(unsigned)(((long long)M * H + 255) / 256), 256, 0, s>>>(M, H, m->dzb, m->Pb + m->ow4, m->h3, m->d1);
-  // layer 3: dW3 = h2^T d3, db3 = colsum d3, d2 = d3 W3^T * (h2 > 0)
-  gemm<true, false, float, false>(H, H, M, m->h2, m->d1, m->G + m->oW3, nullptr, sk, s);
-  k_colsum<<<dim3((H + 255) / 256, ry), 256, 0, s>>>(M, H, m->d1, m->G + m->ob3);
-  gemm<false, true, __nv_bfloat16, false>(M, H, H, m->d1, m->Pb + m->oW3, m->d2, nullptr, 1, s);
-  k_relu_mask<<<(unsigned)(((long long)M * H + 255) / 256), 256, 0, s>>>((long long)M * H, m->h2, m->d2);
-  // layer 2
-  gemm<true, false, float, false>(H, H, M, m->h1, m->d2, m->G + m->oW2, nullptr, sk, s);
-  k_colsum<<<dim3((H + 255) / 256, ry), 256, 0, s>>>(M, H, m->d2, m->G + m->ob2);
-  gemm<false, true, __nv_bfloat16, false>(M, H, H, m->d2, m->Pb + m->oW2, m->d1, nullptr, 1, s);
-  k_relu_mask<<<(unsigned)(((long long)M * H + 255) / 256), 256, 0, s>>>((long long)M * H, m->h1, m->d1);
-  // layer 1
-  gemm<true, false, float, false>(m->F, H, M, X, m->d1, m->G + m->oW1, nullptr, sk, s);
-  k_colsum<<<dim3((H + 255) / 256, ry), 256, 0, s>>>(M, H, m->d1, m->G + m->ob1);
+// Rows X[0..M): the logits, and with labels the loss and the gradients of the pre-activations (G
+// cleared). Rows per block: few for small batches, whose latency is the blocks' own work, more
+// where a weight load then serves more rows and the SMs are still full. Measured, call of
+// qis_mlp_forward at H = 256 with 4 / 8 / 16 / 32 (8 columns a lane) rows: M = 300 45 / 47 / 58 /
+// 72 us, M = 2000 72 / 60 / 60 / 73, M = 4096 104 / 92 / 72 / 81; of qis_mlp_loss_grad M = 700 111 /
+// 114 / 135 / 172, M = 2000 160 / 127 / 142 / 176, M = 4096 232 / 207 / 180 / 194.
+cudaError_t mlp_pass(qis_mlp* m, int M, const float* X, const float* y, cudaStream_t s) {
+  if (M <= 8 * m->sms) return pass_tm<4, 1>(m, M, X, y, s);
+  if (M <= 18 * m->sms) return pass_tm<8, 2>(m, M, X, y, s);
+  return pass_tm<16, 4>(m, M, X, y, s);
+}
+
+// Gradients of the mean loss over the rows of the last mlp_pass with labels, into G.
+cudaError_t mlp_weight_grads(qis_mlp* m, int M, const float* X, cudaStream_t s) {
+  const int H = m->H, tiles = 2 * ((H + kWM - 1) / kWM) * ((H + kWN - 1) / kWN);
+  // the batch split so that two blocks share an SM, 32 rows at least
+  const int parts = std::max(1, std::min(std::min(2 * m->sms / tiles, (M + 31) / 32), 64));
+  const int per = ((M + parts - 1) / parts + kWK - 1) / kWK * kWK;
+  const int thin = ((M + 127) / 128 + parts - 1) / parts * ((H + 255) / 256);
+  k_mlp_wgrad<<<dim3(tiles + thin, parts), 256, 0, s>>>(net_of(m), M, per, X, m->h1, m->h2, m->h3, m->d1, m->d2, m->d3,
+                                                        m->dzb, m->G);
+  return cudaGetLastError();
 }
 
 void refresh_bf16(qis_mlp* m, cudaStream_t s) {
-  k_to_bf16<<<(m->n_params + 255) / 256, 256, 0, s>>>(m->n_params, m->P, m->Pb);
+  k_to_bf16<<<(m->n_params + 255) / 256, 256, 0, s>>>(net_of(m), m->n_params, m->P, m->Pb, m->W2t, m->W3t);
 }
+
+// The network's stream waits for the last use of its buffers on a context's stream.
+cudaError_t wait_idle(qis_mlp* m) { return cudaStreamWaitEvent(m->stream, m->busy, 0); }
 }  // namespace
 
 extern "C" {
@@ -359,6 +552,10 @@ int qis_mlp_create(const qis_mlp_config* cfg, qis_mlp** out) {
     MALLOC(m->Mm, m->n_params);
     MALLOC(m->Vv, m->n_params);
     MALLOC(m->Pb, m->n_params);
+    MALLOC(m->W2t, (size_t)H * H);
+    MALLOC(m->W3t, (size_t)H * H);
+    MCK(cudaEventCreateWithFlags(&m->busy, cudaEventDisableTiming));
+    MCK(cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, cfg->device));
     MALLOC(m->X, (size_t)m->cap * F);
     MALLOC(m->Y, m->cap);
     const size_t rows = (size_t)std::max(m->batch, m->max_n);
@@ -367,6 +564,8 @@ int qis_mlp_create(const qis_mlp_config* cfg, qis_mlp** out) {
     MALLOC(m->h3, rows * H);
     MALLOC(m->d1, rows * H);
     MALLOC(m->d2, rows * H);
+    MALLOC(m->d3, rows * H);
+    MALLOC(m->Yq, rows);
     MALLOC(m->zb, rows);
     MALLOC(m->dzb, rows);
     MALLOC(m->loss, 1);
@@ -406,6 +605,10 @@ void qis_mlp_destroy(qis_mlp* m) {
   if (!m) return;
   cudaSetDevice(m->cfg.device);
   if (m->stream) cudaStreamSynchronize(m->stream);
+  if (m->busy) {
+    cudaEventSynchronize(m->busy);
+    cudaEventDestroy(m->busy);
+  }
   for (void* p : m->allocs) cudaFree(p);
   if (m->stream) cudaStreamDestroy(m->stream);
   delete m;
@@ -430,6 +633,7 @@ int qis_mlp_get_params(qis_mlp* m, float* flat) {
 int qis_mlp_set_params(qis_mlp* m, const float* flat) {
   if (!m || !flat) return mfail(m, QIS_ERR_INVALID_ARG, "NULL argument");
   MCK(cudaSetDevice(m->cfg.device));
+  MCK(wait_idle(m));
   MCK(cudaStreamSynchronize(m->stream));
   MCK(cudaMemcpy(m->P, flat, sizeof(float) * m->n_params, cudaMemcpyHostToDevice));
   MCK(cudaMemset(m->Mm, 0, sizeof(float) * m->n_params));
@@ -445,9 +649,10 @@ int qis_mlp_features(qis_mlp* m, int n, const double* J, const double* h, float*
   if (n < 2 || n > m->max_n) return mfail(m, QIS_ERR_INVALID_ARG, "n must be in [2, max_n]");
   MCK(cudaSetDevice(m->cfg.device));
   cudaStream_t s = m->stream;
+  MCK(wait_idle(m));
   MCK(cudaMemcpyAsync(m->Jst, J, sizeof(double) * n * n, cudaMemcpyHostToDevice, s));
   MCK(cudaMemcpyAsync(m->hst, h, sizeof(double) * n, cudaMemcpyHostToDevice, s));
-  k_mlp_features<<<(n + 127) / 128, 128, 0, s>>>(m->Jst, n, m->hst, n, m->Xq);
+  k_mlp_features<<<(n + 7) / 8, 256, 0, s>>>(m->Jst, n, m->hst, n, m->Xq);
   MCK(cudaGetLastError());
   MCK(cudaMemcpyAsync(X_out, m->Xq, sizeof(float) * n * kF, cudaMemcpyDeviceToHost, s));
   MCK(cudaStreamSynchronize(s));
@@ -466,10 +671,11 @@ int qis_mlp_add_example(qis_mlp* m, int n, const double* J, const double* h, con
   if (m->n_examples + n > m->cap) return mfail(m, QIS_ERR_CAPACITY, "training set full (max_sites)");
   MCK(cudaSetDevice(m->cfg.device));
   cudaStream_t s = m->stream;
+  MCK(wait_idle(m));
   MCK(cudaMemcpyAsync(m->Jst, J, sizeof(double) * n * n, cudaMemcpyHostToDevice, s));
   MCK(cudaMemcpyAsync(m->hst, h, sizeof(double) * n, cudaMemcpyHostToDevice, s));
   MCK(cudaMemcpyAsync(m->bst, bits, sizeof(uint64_t) * ((n + 63) / 64), cudaMemcpyHostToDevice, s));
-  k_mlp_features<<<(n + 127) / 128, 128, 0, s>>>(m->Jst, n, m->hst, n, m->X + (size_t)m->n_examples * kF);
+  k_mlp_features<<<(n + 7) / 8, 256, 0, s>>>(m->Jst, n, m->hst, n, m->X + (size_t)m->n_examples * kF);
   k_mlp_labels<<<(n + 127) / 128, 128, 0, s>>>(m->bst, n, m->Y + m->n_examples);
   MCK(cudaGetLastError());
   MCK(cudaStreamSynchronize(s));   // staging buffers are reused by the next call
@@ -482,9 +688,9 @@ int qis_mlp_forward(qis_mlp* m, int M, const float* X, float* z_out) {
   if (M > std::max(m->batch, m->max_n)) return mfail(m, QIS_ERR_INVALID_ARG, "M exceeds the activation buffers");
   MCK(cudaSetDevice(m->cfg.device));
   cudaStream_t s = m->stream;
+  MCK(wait_idle(m));
   MCK(cudaMemcpyAsync(m->Xq, X, sizeof(float) * M * kF, cudaMemcpyHostToDevice, s));
-  mlp_forward(m, M, m->Xq, nullptr, s);
-  MCK(cudaGetLastError());
+  MCK(mlp_pass(m, M, m->Xq, nullptr, s));
   MCK(cudaMemcpyAsync(z_out, m->zb, sizeof(float) * M, cudaMemcpyDeviceToHost, s));
   MCK(cudaStreamSynchronize(s));
   return 0;
@@ -495,13 +701,12 @@ int qis_mlp_loss_grad(qis_mlp* m, int M, const float* X, const float* y, double*
   if (M > std::max(m->batch, m->max_n)) return mfail(m, QIS_ERR_INVALID_ARG, "M exceeds the activation buffers");
   MCK(cudaSetDevice(m->cfg.device));
   cudaStream_t s = m->stream;
+  MCK(wait_idle(m));
   MCK(cudaMemcpyAsync(m->Xq, X, sizeof(float) * M * kF, cudaMemcpyHostToDevice, s));
-  float* ylab = m->d2;   // labels staged in a gradient buffer that is only written after the head
-  MCK(cudaMemcpyAsync(ylab, y, sizeof(float) * M, cudaMemcpyHostToDevice, s));
+  MCK(cudaMemcpyAsync(m->Yq, y, sizeof(float) * M, cudaMemcpyHostToDevice, s));
   MCK(cudaMemsetAsync(m->loss, 0, sizeof(double), s));
-  mlp_forward(m, M, m->Xq, ylab, s);
-  mlp_backward(m, M, m->Xq, s);
-  MCK(cudaGetLastError());
+  MCK(mlp_pass(m, M, m->Xq, m->Yq, s));
+  MCK(mlp_weight_grads(m, M, m->Xq, s));
   if (loss) MCK(cudaMemcpyAsync(loss, m->loss, sizeof(double), cudaMemcpyDeviceToHost, s));
   if (grad_out) MCK(cudaMemcpyAsync(grad_out, m->G, sizeof(float) * m->n_params, cudaMemcpyDeviceToHost, s));
   MCK(cudaStreamSynchronize(s));
@@ -513,6 +718,7 @@ int qis_mlp_train(qis_mlp* m, int epochs, float lr, double* final_loss) {
   if (m->n_examples < 1) return mfail(m, QIS_ERR_STATE, "no training examples");
   MCK(cudaSetDevice(m->cfg.device));
   cudaStream_t s = m->stream;
+  MCK(wait_idle(m));
   const int N = m->n_examples, Bt = m->batch;
   double last = 0.0;
   for (int ep = 0; ep < epochs; ++ep) {
@@ -521,13 +727,13 @@ int qis_mlp_train(qis_mlp* m, int epochs, float lr, double* final_loss) {
     for (int r0 = 0; r0 < N; r0 += Bt, ++nb) {
       const int M = std::min(Bt, N - r0);
       const float* X = m->X + (size_t)r0 * kF;
-      mlp_forward(m, M, X, m->Y + r0, s);
-      mlp_backward(m, M, X, s);
+      MCK(mlp_pass(m, M, X, m->Y + r0, s));
+      MCK(mlp_weight_grads(m, M, X, s));
       ++m->adam_t;
       const float b1 = 0.9f, b2 = 0.999f;
       const float c1 = 1.f - powf(b1, (float)m->adam_t), c2 = 1.f - powf(b2, (float)m->adam_t);
-      k_adam<<<(m->n_params + 255) / 256, 256, 0, s>>>(m->n_params, m->P, m->G, m->Mm, m->Vv, lr, b1, b2, 1e-8f, c1, c2);
-      refresh_bf16(m, s);
+      k_adam<<<(m->n_params + 255) / 256, 256, 0, s>>>(net_of(m), m->n_params, m->P, m->G, m->Mm, m->Vv, lr, b1, b2, 1e-8f,
+                                                       c1, c2, m->Pb, m->W2t, m->W3t);
     }
     MCK(cudaGetLastError());
     double sum = 0.0;
@@ -545,13 +751,18 @@ int qis_mlp_train(qis_mlp* m, int epochs, float lr, double* final_loss) {
 namespace qis {
 cudaError_t mlp_propose_states(qis_mlp* m, const double* J64, long long stride, const double* h64, int n, int R,
                                uint64_t key, uint64_t* init_bits, int Wstride, cudaStream_t s) {
-  // the network runs on the context's stream; its own stream must be idle
+  // the network runs on the context's stream: after its own stream's work (idle once a call has
+  // returned) and after an earlier use on any other context's
   cudaError_t e = cudaStreamSynchronize(m->stream);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(s, m->busy, 0);
   if (e != cudaSuccess) return e;
-  k_mlp_features<<<(n + 127) / 128, 128, 0, s>>>(J64, stride, h64, n, m->Xq);
-  mlp_forward(m, n, m->Xq, nullptr, s);
-  k_mlp_sample<<<dim3(((n + 63) / 64 + 31) / 32, R), 32, 0, s>>>(m->zb, n, R, key, init_bits, Wstride);
-  return cudaGetLastError();
+  k_mlp_features<<<(n + 7) / 8, 256, 0, s>>>(J64, stride, h64, n, m->Xq);
+  e = cudaGetLastError();
+  if (e == cudaSuccess) e = mlp_pass(m, n, m->Xq, nullptr, s);
+  if (e != cudaSuccess) return e;
+  k_mlp_sample<<<dim3((n + 31) / 32, (R + kSampleR - 1) / kSampleR), 32, 0, s>>>(m->zb, n, R, key, init_bits, Wstride);
+  e = cudaGetLastError();
+  return e == cudaSuccess ? cudaEventRecord(m->busy, s) : e;
 }
 int mlp_max_n(const qis_mlp* m) { return m->max_n; }
 }  // namespace qis
