@@ -48,7 +48,9 @@ extern "C" {
  * exact modes are historical (a BF16 hi/lo split and an FP8 digit were planned); what they do on
  * this GPU is stated beside each. */
 #define QIS_FP64 0        /* plain form: FP64 fields, energies and comparisons, in one fixed
-                             evaluation order (f_i summed with j ascending, E' = E_p + dE) */
+                             evaluation order (f_i summed with j ascending, E' = E_p + dE); the
+                             candidates that can enter a list are found with an FP32 filter with a
+                             rigorous error band where it applies (see pair_scan) */
 #define QIS_SPLIT_BF16 1  /* exact fixed point: J and h on the grid 2^-q (Jq = J 2^q, int64);
                              Jq written in balanced base-4096 digits (12-bit, |d| <= 2048; 11-bit
                              digits, base 2048, above a padded n of 8192), each an exact FP16
@@ -101,7 +103,7 @@ const char* qis_last_error(const qis_ctx* ctx);
 /* Add one Ising instance H0 (Eq. (1)).
  *   n: number of spins, 2 <= n <= cfg.max_n.
  *   J: n*n FP64 row-major, symmetric (bitwise J_ij == J_ji), zero diagonal, finite; host
- *      memory (not retained). In the split modes a page-locked J (cudaHostAlloc /
+ *      memory (not retained). A page-locked J (cudaHostAlloc /
  *      cudaHostRegister) is read by the device directly, without a staging copy.
  *   h: n FP64 finite, host memory.
  * Instances get consecutive ids from 0. In QIS_SPLIT_BF16 the values are represented on
@@ -259,8 +261,11 @@ int qis_candidate_count(qis_ctx* ctx, uint64_t* pairs, uint64_t* singles);
  *                  QIS_FLIPS_SINGLE has no pairs to scan: its search kernel runs every iteration
  *                  of a call in one block per search at any n (K+1 <= 256, fields by update), 3
  *                  (where it is allowed) and QIS_FUSED=0 the per-kernel form.
- *                  Every form gives the same kept lists. QIS_FP64 scans every pair in its plain
- *                  FP64 form whatever this says; qis_get_tuning reports 2 there. */
+ *                  Every form gives the same kept lists. QIS_FP64 ignores this: up to a
+ *                  padded n of 1024 and K+1 <= 256 the fused kernel decides the pairs with the
+ *                  split modes' filter and evaluates the survivors in the defining FP64
+ *                  arithmetic, else (or with QIS_FUSED=0, or magnitudes outside 2^-60 .. 2^60) every
+ *                  pair is evaluated in FP64; qis_get_tuning reports 2 there. */
 typedef struct {
   int scan_chunk_nc;
   int scan_search_group;
@@ -296,7 +301,7 @@ int qis_set_incremental_fields(qis_ctx* ctx, int on);
 /* Pair terms the candidate scan evaluated one by one since the context was created: in the
  * split modes the scan skips every row whose bound c_i = thr - a_i lies below a lower bound
  * of all its pair terms, and counts (rows evaluated) x (chunk width, masked entries
- * included); in QIS_FP64 every pair is evaluated (the qis_candidate_count pairs). The pairs
+ * included); in QIS_FP64 it is the qis_candidate_count pairs. The pairs
  * of qis_candidate_count are all decided exactly either way. The output-sensitive scan
  * (pair_scan 1) counts the pairs it tests one by one (those in the live rows' prefixes, each
  * once). Synchronises the stream. */

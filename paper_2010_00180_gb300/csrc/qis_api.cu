@@ -46,7 +46,9 @@ struct qis_ctx {
   long long* hq = nullptr;
   uint64_t* zob = nullptr;
   double* stats = nullptr;
-  double* jstage = nullptr;   // [max_n * max_n] one instance's J as copied from the host (FP64 mode)
+  double* jstage = nullptr;   // [max_inst][NP * NP] couplings as copied from the host (FP64 mode)
+  bool f64_filter = false;    // FP64 mode: the context holds the filter's fixed-point and FP32 couplings
+  int f64_wild = 0;           // FP64 mode: instances whose magnitudes the FP32 filter does not cover
   LayoutItem* items_d = nullptr;   // [max_inst] staging places of a creation batch
   uint64_t* all_bits = nullptr;   // [max_inst][K1][Wmax] every instance's merged states
   double* all_E = nullptr;        // [max_inst][K1]
@@ -236,7 +238,10 @@ static bool sparse_scan(const qis_ctx* ctx) { return sparse_allowed(ctx) && ctx-
 // per-kernel form) is read.
 static bool fused_search(const qis_ctx* ctx) {
   if (ctx->cfg.flips == QIS_FLIPS_SINGLE)
-    return ctx->P.pw_n > 0 && ctx->tune.pair_scan != 3 && ctx->P.inc_on && !ctx->fields_simt && !ctx->no_fused;
+    return ctx->mode != QIS_FP64 && ctx->P.pw_n > 0 && ctx->tune.pair_scan != 3 && ctx->P.inc_on && !ctx->fields_simt && !ctx->no_fused;
+  // FP64 mode: the same kernel with the defining FP64 fields and energies (any pair_scan: its own
+  // form scans every pair); the FP32 filter needs magnitudes well inside FP32's range
+  if (ctx->mode == QIS_FP64) return ctx->f64_filter && ctx->f64_wild == 0 && !ctx->no_fused;
   return sparse_scan(ctx) && ctx->tune.pair_scan != 3 && ctx->NP <= kSearchMaxNP && ctx->K1 <= kSearchMaxK1 &&
          ctx->P.inc_on && !ctx->fields_simt && !ctx->no_fused;
 }
@@ -248,6 +253,12 @@ static bool fused_search(const qis_ctx* ctx) {
 int launch_iterations_fused(qis_ctx* ctx, int n, cudaStream_t s) {
   ctx->P.dense_ctl = 0;
   const DevPtrs& P = ctx->P;
+  if (ctx->mode == QIS_FP64) {   // picks and computes the fields of every iteration itself
+    CK(prof_begin(ctx, 5));
+    LAUNCH(launch_search(P, n, s));
+    CK(prof_end(ctx, 5));
+    return 0;
+  }
   CK(prof_begin(ctx, 0));
   LAUNCH(launch_pick(P, s));
   CK(prof_end(ctx, 0));
@@ -309,7 +320,7 @@ int build_work(qis_ctx* ctx) {
   ctx->P.gemm_nt = ctx->tune.gemm_tile_searches > 0 ? ctx->tune.gemm_tile_searches
                                                       : gemm_tile_n(ctx->R, ctx->digits_used);
   std::vector<int4> w;
-  for (int id = 0; id < (int)ctx->inst.size() && ctx->mode == QIS_FP64; ++id) {   // the FP64 scan's tiles
+  for (int id = 0; id < (int)ctx->inst.size() && ctx->mode == QIS_FP64 && !fused_search(ctx); ++id) {   // the FP64 scan's tiles
     const int nb = (ctx->inst[id].n + kTile - 1) / kTile;
     for (int bi = 0; bi < nb; ++bi)
       for (int bj = bi; bj < nb; ++bj)
@@ -407,7 +418,14 @@ int qis_create(const qis_config* cfg, qis_ctx** out) {
     ALLOC(ctx->zob, kMaxN);
     ALLOC(ctx->stats, (size_t)ctx->max_inst * (NP + 8));   // validation statistics of every instance
     ALLOC(ctx->items_d, (size_t)ctx->max_inst);
-    if (ctx->mode == QIS_FP64) ALLOC(ctx->jstage, (size_t)cfg->max_n * cfg->max_n);   // the split modes stage in Jq
+    if (ctx->mode == QIS_FP64) ALLOC(ctx->jstage, (size_t)ctx->pool_mat);   // the split modes stage in Jq
+    ctx->f64_filter = ctx->mode == QIS_FP64 && ctx->cfg.flips != QIS_FLIPS_SINGLE && ctx->NP <= kSearchMaxNP &&
+                      ctx->K1 <= kSearchMaxK1;
+    if (ctx->f64_filter) {   // the fixed-point fields and FP32 couplings of the fused search's filter
+      ALLOC(ctx->Jq, ctx->pool_mat);
+      ALLOC(ctx->J4, ctx->pool_mat);
+      ALLOC(ctx->hq, ctx->pool_vec);
+    }
     ALLOC(ctx->all_bits, (size_t)ctx->max_inst * K1 * W);
     ALLOC(ctx->all_E, (size_t)ctx->max_inst * K1);
     ALLOC(ctx->work, (size_t)ctx->max_inst * ((NP / kTile) * (NP / kTile + 1) / 2) *
@@ -461,7 +479,7 @@ int qis_create(const qis_config* cfg, qis_ctx** out) {
     ALLOC(P.full_tile, (size_t)ctx->max_inst * ((ctx->R + 15) / 16));
     P.ring_n = 1;
     P.ring_slot = (long long)B * NP;
-    if (ctx->mode != QIS_FP64) {
+    if (ctx->mode != QIS_FP64 || ctx->f64_filter) {
       // the exact fields of the last ring_n parents of every search (fields by update): as many
       // iterations as fit in 4 GiB, 2 .. 128 (QIS_FIELD_RING overrides)
       const size_t slot = (size_t)B * NP * sizeof(long long);
@@ -469,8 +487,10 @@ int qis_create(const qis_config* cfg, qis_ctx** out) {
       const char* e = getenv("QIS_FIELD_RING");
       if (e && atoi(e) >= 2) rn = atoi(e);
       P.ring_n = rn;
-      P.inc_on = ctx->fields_simt ? 0 : 1;
       ALLOC(P.aq, (size_t)rn * B * NP);
+    }
+    if (ctx->mode != QIS_FP64) {
+      P.inc_on = ctx->fields_simt ? 0 : 1;
       ALLOC(P.as32, B * NP);
       P.s16_stride = (long long)(ctx->R + 255) * NP;   // room for ceil(R / NT) tiles of any NT <= 256
       ALLOC(P.S16, (size_t)ctx->max_inst * P.s16_stride);
@@ -480,7 +500,7 @@ int qis_create(const qis_config* cfg, qis_ctx** out) {
     }
     ALLOC(P.thr32, B);
     ALLOC(P.amin32, B);
-    if (ctx->mode != QIS_FP64) ALLOC(P.rm4, (size_t)ctx->pool_vec);
+    if (ctx->mode != QIS_FP64 || ctx->f64_filter) ALLOC(P.rm4, (size_t)ctx->pool_vec);
     if (ctx->mode != QIS_FP64) {
       ALLOC(P.sctl, B * (size_t)(NP / 32));
     }
@@ -597,15 +617,6 @@ int copy_fields_h(qis_ctx* ctx, int first, int count, const int* n, const double
   return 0;
 }
 
-// The padded layout of instance id's J from `stage`, and its validation into stats slot `slot`.
-int lay_out_instance(qis_ctx* ctx, int id, int slot, int n, const double* stage) {
-  const long long off_mat = (long long)id * ctx->NP * ctx->NP, off_vec = (long long)id * ctx->NP;
-  cudaStream_t s = ctx->stream;
-  LAUNCH(launch_restride(stage, n, pad_of(n), ctx->J64 + off_mat, s));
-  LAUNCH(launch_validate(ctx->P, id, n, off_mat, off_vec, ctx->stats + (size_t)slot * (ctx->NP + 8), s));
-  return 0;
-}
-
 // The descriptor of instance id from its validation statistics (host): the checks of J and
 // h, the fixed-point grid 2^-q and the number of base-4096 digits.
 int describe_instance(qis_ctx* ctx, int id, int n, const double* st, InstDesc& d) {
@@ -633,17 +644,26 @@ int describe_instance(qis_ctx* ctx, int id, int n, const double* st, InstDesc& d
   d.digits = 0;
   d.inv_scale = 1.0;
   d.rounded = 0;
-  d.j4max = 0.f;
+  d.j4max = (float)(4.0 * maxJ) * (1.0f + 1e-6f);   // FP64 mode (the split modes: below, from Jq)
   d.j4max64 = 4.0 * maxJ;   // exact (power-of-two scaling)
   // energies from scratch: integers J 2^eq, exact where 58 bits hold every coupling
   frexp(std::max(maxJ, maxh), &d.etop);
   d.eq = std::min(maxfrac, 58 - d.etop);
+  double S = 0.0;
+  for (int i = 0; i < n; ++i) S += st[4 + i];
+  S += st[4 + n];
+  int qmax = 51;
+  if (S > 0) qmax = 51 - (int)floor(log2(S));
+  if (ctx->f64_filter) {
+    // the filter's grid; q = -1 (no filter) where a_i, 4 J_ij and the energy changes are not well
+    // within FP32's normal range
+    if (d.etop >= -60 && d.etop <= 60 && std::isfinite(S) && qmax >= 0) {
+      d.q = std::min(maxfrac, qmax);
+      d.rounded = maxfrac > qmax;
+      d.inv_scale = ldexp(1.0, -d.q);
+    }
+  }
   if (ctx->mode != QIS_FP64) {
-    double S = 0.0;
-    for (int i = 0; i < n; ++i) S += st[4 + i];
-    S += st[4 + n];
-    int qmax = 51;
-    if (S > 0) qmax = 51 - (int)floor(log2(S));
     int q = maxfrac;
     if (ctx->mode == QIS_PM1_FP8) {
       if (maxfrac != 0 || maxJ > 15.0)
@@ -674,15 +694,16 @@ int describe_instance(qis_ctx* ctx, int id, int n, const double* st, InstDesc& d
 // fixed-point planes, the host tables (asynchronous on the library stream).
 int register_instances(qis_ctx* ctx, int first, const std::vector<InstDesc>& ds) {
   cudaStream_t s = ctx->stream;
+  int max_pad = 0;
+  for (const InstDesc& d : ds) max_pad = std::max(max_pad, d.n_pad);
   CK(cudaMemcpyAsync(ctx->inst_d + first, ds.data(), sizeof(InstDesc) * ds.size(), cudaMemcpyHostToDevice, s));
-  if (ctx->mode != QIS_FP64 && !ds.empty()) {
+  if ((ctx->mode != QIS_FP64 || ctx->f64_filter) && !ds.empty()) {
     // fixed-point planes, digits and row maxima of the whole batch: two launches
-    int max_pad = 0;
-    for (const InstDesc& d : ds) max_pad = std::max(max_pad, d.n_pad);
     LAUNCH(launch_prepare_batch(ctx->P, first, (int)ds.size(), max_pad, ctx->D16, ctx->Jq, ctx->J4, ctx->hq, s));
   }
   for (size_t k = 0; k < ds.size(); ++k) {
     const InstDesc& d = ds[k];
+    if (ctx->f64_filter && d.q < 0) ++ctx->f64_wild;
     ctx->inst.push_back(d);
     if (d.digits > ctx->digits_used) ctx->digits_used = d.digits;
     ctx->inst_ready.push_back(0);
@@ -740,8 +761,7 @@ int flush_init(qis_ctx* ctx, bool defer) {
                          cudaMemcpyHostToDevice, ctx->stream));
       x = y;
     }
-    // split modes: the initial energies of the range in groups of states per block first
-    // (unless they are known or deferred); FP64 mode: formed by k_init_search itself
+    // the initial energies of the range first, unless they are known or (split modes) deferred
     const bool grouped = ctx->mode != QIS_FP64;
     bool known = true;
     for (int x = a; x < e; ++x) known = known && ctx->e0_valid[x];
@@ -749,15 +769,16 @@ int flush_init(qis_ctx* ctx, bool defer) {
     if (deferred) {
       for (int x = a; x < e; ++x) ctx->e0_deferred[x] = 1;
       ctx->e0_unresolved = true;
-    } else if (grouped && !known) {
+    } else if (!grouped && !known) {
+      LAUNCH(launch_init_energy_f64(ctx->P, a, e - a, ctx->stream));
+    } else if (!known) {
       int max_n = 0;
       for (int x = a; x < e; ++x) max_n = std::max(max_n, ctx->inst[x].n);
       int dg = 1;
       for (int x = a; x < e; ++x) dg = std::max(dg, energy_digits(ctx->inst[x].etop, ctx->inst[x].q));
       LAUNCH(launch_init_energy(ctx->P, a, e - a, max_n, dg, ctx->stream));
     }
-    LAUNCH(launch_init_search(ctx->P, ctx->inst[a].first_search, (e - a) * ctx->R, ctx->stream,
-                              known || (grouped && !deferred), deferred));
+    LAUNCH(launch_init_search(ctx->P, ctx->inst[a].first_search, (e - a) * ctx->R, ctx->stream, deferred));
     if (!deferred)
       for (int x = a; x < e; ++x) ctx->e0_valid[x] = 1;
     a = e;
@@ -790,22 +811,22 @@ int qis_create_instances(qis_ctx* ctx, int count, const int* n, const double* co
     if (rc) return rc;
   }
   CK(cudaSetDevice(ctx->cfg.device));
-  // every copy, then every layout and validation, then one read-back of all statistics. In the
-  // split modes each instance is staged in its own region of the fixed-point pool (written
-  // from J64 later), so the copies run back to back; the FP64 mode stages one instance at a
-  // time (a copy from pageable memory first waits for the stream, so the buffer is free again).
+  // every copy, then every layout and validation, then one read-back of all statistics. Each
+  // instance is staged in its own region (split modes: of the fixed-point pool, written from J64
+  // later), so the copies run back to back.
   {
     const int rc = copy_fields_h(ctx, first, count, n, h);
     if (rc) return rc;
   }
-  if (ctx->mode != QIS_FP64) {
+  {
     // a page-locked J is read by the layout kernel itself (one pass over the host memory);
     // any other J is staged with a copy first
     std::vector<const double*> src(count);
     for (int k = 0; k < count; ++k) {
       src[k] = pinned_view(J[k]);
       if (src[k]) continue;
-      double* stage = reinterpret_cast<double*>(ctx->Jq + (long long)(first + k) * ctx->NP * ctx->NP);
+      double* stage = (ctx->mode == QIS_FP64 ? ctx->jstage : reinterpret_cast<double*>(ctx->Jq)) +
+                      (long long)(first + k) * ctx->NP * ctx->NP;
       const int rc = copy_instance(ctx, n[k], J[k], stage);
       if (rc) return rc;
       src[k] = stage;
@@ -826,12 +847,6 @@ int qis_create_instances(qis_ctx* ctx, int count, const int* n, const double* co
     CK(cudaMemsetAsync(ctx->stats, 0, sizeof(double) * (size_t)count * (ctx->NP + 8), ctx->stream));
     CK(cudaMemcpyAsync(ctx->items_d, items.data(), sizeof(LayoutItem) * count, cudaMemcpyHostToDevice, ctx->stream));
     LAUNCH(launch_layout_batch(ctx->P, ctx->items_d, count, max_pad, ctx->J64, ctx->stream));
-  } else {
-    for (int k = 0; k < count; ++k) {
-      int rc = copy_instance(ctx, n[k], J[k], ctx->jstage);
-      if (!rc) rc = lay_out_instance(ctx, first + k, k, n[k], ctx->jstage);
-      if (rc) return rc;
-    }
   }
   const size_t stride = (size_t)ctx->NP + 8;
   std::vector<double> st(stride * count);
@@ -866,6 +881,7 @@ int qis_clear_instances(qis_ctx* ctx) {
   }
   CK(cudaMemset(ctx->P.status, 0, sizeof(int)));   // device flags of the removed searches
   ctx->inst.clear();
+  ctx->f64_wild = 0;
   ctx->inst_ready.clear();
   ctx->init_pending.clear();
   ctx->init_from_host.clear();
@@ -884,9 +900,10 @@ int qis_instance_info(qis_ctx* ctx, int instance_id, int* q, int* digits, int* r
   if (!ctx) return fail(nullptr, QIS_ERR_INVALID_ARG, "ctx is NULL");
   if (instance_id < 0 || instance_id >= (int)ctx->inst.size()) return fail(ctx, QIS_ERR_INVALID_ARG, "bad instance id");
   const InstDesc& d = ctx->inst[instance_id];
-  if (q) *q = d.q;
+  const bool f64 = ctx->mode == QIS_FP64;   // (its filter's grid is no property of the instance)
+  if (q) *q = f64 ? -1 : d.q;
   if (digits) *digits = d.digits;
-  if (rounded) *rounded = d.rounded;
+  if (rounded) *rounded = f64 ? 0 : d.rounded;
   return 0;
 }
 

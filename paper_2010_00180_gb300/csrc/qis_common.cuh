@@ -27,7 +27,7 @@ struct InstDesc {
   int n;            // spins
   int n_pad;        // n rounded up to kPad
   int W;            // words per state
-  int q;            // fixed-point exponent: Jq = J * 2^q  (-1 in FP64 mode)
+  int q;            // fixed-point exponent: Jq = J * 2^q (FP64 mode: of the filter's couplings, or -1)
   int digits;       // number of balanced base-2^dbits digits of Jq
   int dbits;        // digit width: 12 bits, 11 above n_pad = 8192 (FP32 partial sums of the digit
                     // GEMM stay below 2^24: |digit| <= 2^(dbits-1), n_pad terms)
@@ -333,7 +333,6 @@ cudaError_t mlp_propose_states(qis_mlp* m, const double* J64, long long stride, 
 int mlp_max_n(const qis_mlp* m);
 
 // Kernel launchers (defined in the .cu files); each returns the cudaError_t of the launch.
-cudaError_t launch_restride(const double* src, int n, int n_pad, double* dst, cudaStream_t s);
 // Where one instance of a creation batch was staged and where its layout and statistics go.
 struct LayoutItem {
   const double* src;   // n x n FP64, contiguous, as copied from the host
@@ -345,7 +344,6 @@ cudaError_t launch_layout_batch(const DevPtrs& P, const LayoutItem* items, int c
                                 cudaStream_t s);
 cudaError_t launch_prepare_batch(const DevPtrs& P, int first, int count, int max_n_pad, __half* D16, long long* Jq,
                                  float* J4, long long* hq, cudaStream_t s);
-cudaError_t launch_rowmax4(const DevPtrs& P, const InstDesc& d, cudaStream_t s);
 cudaError_t launch_scan_sparse(const DevPtrs& P, cudaStream_t s);
 constexpr int kSparseMaxNP = 4096;   // the sparse pair scan's largest padded n (shared-memory lists)
 // The fused search kernel (every iteration of a search in one block): its largest padded n and
@@ -355,16 +353,11 @@ constexpr int kSearchMaxK1 = 256;
 cudaError_t launch_search(const DevPtrs& P, int n_iters, cudaStream_t s);
 // Single flips: any padded n, at most P.pw_n iterations per launch.
 cudaError_t launch_single(const DevPtrs& P, int n_iters, int ext, cudaStream_t s);
-size_t search_smem(const DevPtrs& P);
-cudaError_t launch_validate(const DevPtrs& P, int inst, int n, long long off_mat, long long off_vec,
-                            double* stats, cudaStream_t s);
 cudaError_t launch_fields_tc(const DevPtrs& P, const void* D16, const void* S16, int max_inst, int digits_max,
                              int nt, cudaStream_t s);
 int gemm_tile_n(int R, int digits);
-cudaError_t launch_quantize(const DevPtrs& P, const InstDesc& d, int inst, __half* D16, long long* Jq,
-                            float* J4, long long* hq, cudaStream_t s);
-cudaError_t launch_init_search(const DevPtrs& P, int b0, int nb, cudaStream_t s, bool cached = false,
-                               bool deferred = false);
+cudaError_t launch_init_search(const DevPtrs& P, int b0, int nb, cudaStream_t s, bool deferred = false);
+cudaError_t launch_init_energy_f64(const DevPtrs& P, int inst0, int n_inst, cudaStream_t s);
 cudaError_t launch_hash_list(const DevPtrs& P, int b, int count, cudaStream_t s);
 cudaError_t launch_pick(const DevPtrs& P, cudaStream_t s);
 cudaError_t launch_fields_exact(const DevPtrs& P, cudaStream_t s);

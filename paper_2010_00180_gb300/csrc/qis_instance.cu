@@ -75,12 +75,6 @@ __device__ __forceinline__ void validate_row(const double* J64, const double* h6
   }
 }
 
-__global__ void __launch_bounds__(256) k_validate(const double* J64, const double* h64, int n, int n_pad, double* stats) {
-  const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (i >= n) return;   // warp-uniform
-  validate_row(J64, h64, n, n_pad, stats, i);
-}
-
 // A batch of instances at once: blockIdx.y is the instance of the batch (its layout item).
 __global__ void __launch_bounds__(256) k_validate_batch(const LayoutItem* items, const double* J64, const double* h64) {
   const LayoutItem L = items[blockIdx.y];
@@ -89,26 +83,8 @@ __global__ void __launch_bounds__(256) k_validate_batch(const LayoutItem* items,
   validate_row(J64 + L.off_mat, h64 + L.off_vec, L.n, L.n_pad, L.stats, i);
 }
 
-cudaError_t launch_validate(const DevPtrs& P, int inst, int n, long long off_mat, long long off_vec,
-                            double* stats, cudaStream_t s) {
-  (void)inst;
-  cudaMemsetAsync(stats, 0, 4 * sizeof(double), s);
-  const int np = pad_of(n);
-  k_validate<<<(n + 7) / 8, 256, 0, s>>>(P.J64 + off_mat, P.h64 + off_vec, n, np, stats);
-  return cudaGetLastError();
-}
-
 // ---------------------------------------------------------------- padded layout
-// J (n x n, contiguous, as copied from the host) into the padded n_pad x n_pad plane; zeros
-// past n.
-__global__ void k_restride(const double* src, int n, int n_pad, double* dst) {
-  const long long total = (long long)n_pad * n_pad;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(e / n_pad), j = (int)(e % n_pad);
-    dst[e] = (i < n && j < n) ? src[(long long)i * n + j] : 0.0;
-  }
-}
-
+// J (n x n, contiguous, as given by the host) into the padded n_pad x n_pad plane; zeros past n.
 // Rows i = blockIdx.x, blockIdx.x + gridDim.x, ... of every instance (blockIdx.y), the threads
 // over the columns: coalesced reads of the caller's rows (page-locked host memory read in place
 // where it is), no index division.
@@ -131,37 +107,8 @@ cudaError_t launch_layout_batch(const DevPtrs& P, const LayoutItem* items, int c
   return cudaGetLastError();
 }
 
-cudaError_t launch_restride(const double* src, int n, int n_pad, double* dst, cudaStream_t s) {
-  const long long total = (long long)n_pad * n_pad;
-  const int blocks = (int)std::min<long long>((total + 255) / 256, 4096);
-  k_restride<<<blocks, 256, 0, s>>>(src, n, n_pad, dst);
-  return cudaGetLastError();
-}
-
 // ---------------------------------------------------------------- fixed point + digits
 // D16 holds, per digit and instance, an NP x NP plane in the tiled layout of d16_offset.
-__global__ void k_quantize(const double* J64, const double* h64, int n, int n_pad, int NP, int q, int digits,
-                           int dbits, long long plane, __half* D16, long long* Jq, float* J4, long long* hq) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long tot = (long long)n_pad * n_pad;
-  if (e < tot) {
-    const int i = (int)(e / n_pad), j = (int)(e % n_pad);
-    long long v = 0;
-    if (i < n && j < n) v = __double2ll_rn(ldexp(J64[e], q));
-    Jq[e] = v;
-    J4[e] = (float)(4.0 * ldexp((double)v, -q));
-    long long x = v;
-    const long long base = 1ll << dbits;
-    for (int d = 0; d < digits; ++d) {
-      long long r = x & (base - 1);           // x mod base
-      if (r >= base / 2) r -= base;           // balanced digit in [-base/2, base/2)
-      D16[d * plane + d16_offset(i, j, NP)] = __float2half_rn((float)r);
-      x = (x - r) >> dbits;                   // exact
-    }
-  }
-  if (e < n_pad) hq[e] = (e < n) ? __double2ll_rn(ldexp(h64[e], q)) : 0;
-}
-
 // Instances first .. first+count-1 at once (blockIdx.y), descriptors read on the device; rows
 // i = blockIdx.x, blockIdx.x + gridDim.x, ..., the threads over the columns (no index division).
 // Jq = rn(J 2^q), J4 = fl32(4 Jq 2^-q) (= fl32(Jq) 2^(2-q): scaling by a power of two commutes
@@ -217,71 +164,56 @@ cudaError_t launch_prepare_batch(const DevPtrs& P, int first, int count, int max
   return cudaGetLastError();
 }
 
-cudaError_t launch_quantize(const DevPtrs& P, const InstDesc& d, int inst, __half* D16, long long* Jq,
-                            float* J4, long long* hq, cudaStream_t s) {
-  const long long tot = (long long)d.n_pad * d.n_pad;
-  k_quantize<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(
-      P.J64 + d.off_mat, P.h64 + d.off_vec, d.n, d.n_pad, P.NP, d.q, d.digits, d.dbits, P.pool_mat,
-      D16 + (long long)inst * P.NP * P.NP, Jq + d.off_mat, J4 + d.off_mat, hq + d.off_vec);
-  return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------- row maxima of the filter couplings
-// rm4_i = max_j |4J~_ij| (the FP32 couplings of the scan), a warp per row.
-__global__ void __launch_bounds__(256) k_rowmax4(const float* J4, int n, int n_pad, float* rm4) {
-  const int lane = threadIdx.x & 31;
-  const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (i >= n_pad) return;   // warp-uniform
-  float m = 0.f;
-  if (i < n)
-    for (int j = lane; j < n; j += 32) m = fmaxf(m, fabsf(J4[(long long)i * n_pad + j]));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (lane == 0) rm4[i] = m;
-}
-
-cudaError_t launch_rowmax4(const DevPtrs& P, const InstDesc& d, cudaStream_t s) {
-  k_rowmax4<<<(d.n_pad + 7) / 8, 256, 0, s>>>(P.J4 + d.off_mat, d.n, d.n_pad, P.rm4 + d.off_vec);
-  return cudaGetLastError();
-}
-
 // ---------------------------------------------------------------- search initialisation
-// Alg. 3 initial list: [psi0, K placeholders], E(psi0) from Eq. (1), nothing used.
-// mode 1 (cached): E(psi0) is taken from init_E / init_q, written by launch_init_energy (split modes:
-// exact int64 E 2^q) or by an earlier launch for the same initial
-// states. Mode 2 (deferred, split modes): E(psi0) is left to the first iteration of the fused
-// search kernel, which forms it from the exact fields of psi0 that the iteration computes anyway;
-// the entry holds 0 until then and e0_pend marks the search. Mode 0 (FP64 mode): one thread adds
-// the pair terms i-major, j ascending, then the field terms.
-__global__ void __launch_bounds__(256) k_init_search(DevPtrs P, int b0, int mode) {
-  const bool cached = mode == 1;
+// FP64 mode: E(psi0) of the initial states of instances inst0, inst0 + 1, ... into init_E, the pair
+// terms added i-major, j ascending, then the field terms. A lane per search, 32 searches of an
+// instance per block: the lanes share every coupling's load, and the chain of n^2 / 2 dependent
+// additions is what it costs (one search per block took as long for each: 1.5 ms for 3840 searches
+// of n = 100).
+__global__ void __launch_bounds__(32) k_init_energy_f64(DevPtrs P, int inst0) {
+  const int inst = inst0 + blockIdx.y, r = blockIdx.x * 32 + (int)threadIdx.x;
+  const InstDesc d = P.inst[inst];
+  const int n = d.n;
+  const long long b = (long long)d.first_search + min(r, P.R - 1);
+  const uint64_t* bits = P.init_bits + b * P.Wmax;
+  const double* J = P.J64 + d.off_mat;
+  double Pp = 0.0, F = 0.0;
+  for (int i = 0; i < n; ++i) {
+    const uint64_t si = 0ull - (uint64_t)sigma_of(bits, i);   // all ones where s_i = -1
+    const double* row = J + (long long)i * d.n_pad;
+    for (int j0 = (i + 1) & ~63; j0 < n; j0 += 64) {
+      const uint64_t w = bits[j0 >> 6] ^ si;
+      const int u1 = min(64, n - j0);
+#pragma unroll 8
+      for (int u = max(0, i + 1 - j0); u < u1; ++u)
+        Pp = __dadd_rn(Pp, __longlong_as_double(__double_as_longlong(row[j0 + u]) ^ (long long)((w >> u) << 63)));
+    }
+  }
+  for (int i = 0; i < n; ++i) F = __dadd_rn(F, P.h64[d.off_vec + i] * (sigma_of(bits, i) ? -1.0 : 1.0));
+  if (r < P.R) P.init_E[b] = __dadd_rn(Pp, F);
+}
+
+cudaError_t launch_init_energy_f64(const DevPtrs& P, int inst0, int n_inst, cudaStream_t s) {
+  for (int y = 0; y < n_inst; y += 65535)   // (the grid's second dimension)
+    k_init_energy_f64<<<dim3((P.R + 31) / 32, std::min(n_inst - y, 65535)), 32, 0, s>>>(P, inst0 + y);
+  return cudaGetLastError();
+}
+
+// Alg. 3 initial list: [psi0, K placeholders], E(psi0) from Eq. (1), nothing used. E(psi0) is taken
+// from init_E / init_q, written by launch_init_energy (split modes: exact int64 E 2^q),
+// launch_init_energy_f64 or an earlier start from the same initial states; or (deferred, split
+// modes) it is left to the first iteration of the fused search kernel, which forms it from the
+// exact fields of psi0 that the iteration computes anyway: the entry holds 0 until then and
+// e0_pend marks the search.
+__global__ void __launch_bounds__(256) k_init_search(DevPtrs P, int b0, int deferred) {
   const int b = b0 + blockIdx.x;
   const InstDesc d = P.inst[b / P.R];
-  const int n = d.n, np = d.n_pad, W = d.W;
+  const int n = d.n, W = d.W;
   __shared__ uint64_t bits[kMaxN / 64];
-  __shared__ long long red[1];
   for (int w = threadIdx.x; w < W; w += blockDim.x) bits[w] = P.init_bits[(long long)b * P.Wmax + w];
   __syncthreads();
-  double E0 = 0.0;
-  if (cached) {
-    E0 = P.init_E[b];
-    if (threadIdx.x == 0) red[0] = P.init_q[b];
-  } else if (mode == 2) {
-    if (threadIdx.x == 0) red[0] = 0;
-  } else if (threadIdx.x == 0) {
-    double Pp = 0.0, F = 0.0;
-    const double* J = P.J64 + d.off_mat;
-    for (int i = 0; i < n; ++i) {
-      const double si = sigma_of(bits, i) ? -1.0 : 1.0;
-      for (int j = i + 1; j < n; ++j) {
-        const double sj = sigma_of(bits, j) ? -1.0 : 1.0;
-        Pp = __dadd_rn(Pp, J[(long long)i * np + j] * si * sj);
-      }
-    }
-    for (int i = 0; i < n; ++i) F = __dadd_rn(F, P.h64[d.off_vec + i] * (sigma_of(bits, i) ? -1.0 : 1.0));
-    E0 = __dadd_rn(Pp, F);
-    red[0] = 0;
-  }
+  const double E0 = deferred ? 0.0 : P.init_E[b];
+  const long long q0 = deferred || P.mode == QIS_FP64 ? 0 : P.init_q[b];
   // Zobrist hash of psi0: XOR over the threads' sites, then over the warps
   __shared__ uint64_t s_h[8];
   uint64_t hsh = 0;
@@ -300,10 +232,10 @@ __global__ void __launch_bounds__(256) k_init_search(DevPtrs P, int b0, int mode
   if (threadIdx.x == 0) {
     for (int w = 1; w < (int)(blockDim.x >> 5); ++w) hsh ^= s_h[w];
     P.init_E[b] = E0;
-    P.init_q[b] = (P.mode != QIS_FP64) ? red[0] : 0;
+    P.init_q[b] = q0;
     P.lst_E[base] = E0;
-    if (P.mode != QIS_FP64) P.lst_q[base] = red[0];
-    P.lst_key[base] = (P.mode != QIS_FP64) ? qkey(red[0]) : dkey(E0);
+    if (P.mode != QIS_FP64) P.lst_q[base] = q0;
+    P.lst_key[base] = (P.mode != QIS_FP64) ? qkey(q0) : dkey(E0);
     P.lst_stamp[base] = 0;
     P.lst_hash[base] = hsh;
     P.lst_count[b] = 1;
@@ -311,13 +243,13 @@ __global__ void __launch_bounds__(256) k_init_search(DevPtrs P, int b0, int mode
     P.iter_t[b] = 0;
     if (P.ring_t0) P.ring_t0[b] = 0;
     P.surv_cnt[b] = 0;
-    P.e0_pend[b] = mode == 2;
+    P.e0_pend[b] = deferred;
   }
 }
 
-cudaError_t launch_init_search(const DevPtrs& P, int b0, int nb, cudaStream_t s, bool cached, bool deferred) {
+cudaError_t launch_init_search(const DevPtrs& P, int b0, int nb, cudaStream_t s, bool deferred) {
   if (nb <= 0) return cudaSuccess;
-  k_init_search<<<nb, 256, 0, s>>>(P, b0, deferred ? 2 : cached ? 1 : 0);
+  k_init_search<<<nb, 256, 0, s>>>(P, b0, deferred ? 1 : 0);
   return cudaGetLastError();
 }
 

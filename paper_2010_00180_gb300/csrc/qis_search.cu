@@ -1,5 +1,5 @@
 // qis_search.cu -- every iteration of one search in one thread block (the fused, persistent
-// form of the iteration of Alg. 3 in the split precision modes; single flips alone: qis_single.cu).
+// form of the iteration of Alg. 3; single flips alone: qis_single.cu).
 //
 // The R searches of an instance, and the instances, share nothing until the Alg. 4 merge, so
 // one block can take one search through all the iterations of a qis_iterate call without ever
@@ -18,8 +18,9 @@
 // The kept list's order, keys, stamps and used flags, the parent's spins and {a_i, s_i} stay in
 // shared memory across the iterations; the kept states' bits, the aq ring and the survivor
 // buffer are in global memory (written and read by this block only, within the L2 cache).
-// The first iteration's parent is picked, and its fields computed (update, or the tensor-core
-// GEMM for a parent without a stored generator), by the kernels launched before this one.
+// Split modes: the first iteration's parent is picked, and its fields computed (update, or the
+// tensor-core GEMM for a parent without a stored generator), by the kernels launched before this one.
+// FP64 mode: the same filter, the survivors' energies in the defining FP64 arithmetic.
 // The arithmetic of every phase is that of the per-kernel form (k_bound, k_scan_sparse,
 // k_merge), so the kept lists are identical bit for bit.
 #include "qis_block.cuh"
@@ -37,13 +38,13 @@ __host__ __device__ inline int search_pcs(int cap, int merge_cand) {
 
 // Byte offsets of the dynamic shared memory of a search block.
 struct SearchLayout {
-  int as, pb, okey0, okey1, ostamp, oslot0, oslot1, htab, ssv, oused, scratch, total;
+  int as, ad, pb, okey0, okey1, ostamp, oslot0, oslot1, htab, ssv, oused, scratch, total;
   int sc;   // bytes of the scratch region
 };
 
 constexpr int kSSV = 512;   // survivors held in shared memory (more go to the global buffer)
 
-__host__ __device__ inline SearchLayout search_layout(int NP, int Wmax, int K1, int cap, int merge_cand) {
+__host__ __device__ inline SearchLayout search_layout(int NP, int Wmax, int K1, int cap, int merge_cand, bool f64) {
   SearchLayout L;
   int o = 0;
   auto take = [&](int bytes) {
@@ -53,6 +54,7 @@ __host__ __device__ inline SearchLayout search_layout(int NP, int Wmax, int K1, 
     return r;
   };
   L.as = take(NP * 8);
+  L.ad = take(f64 ? NP * 8 : 0);
   L.pb = take(Wmax * 8);
   L.okey0 = take(K1 * 8);
   L.okey1 = take(K1 * 8);
@@ -105,9 +107,44 @@ static __device__ __noinline__ void fields_full(const DevPtrs& P, const InstDesc
   }
 }
 
+// FP64 mode: a_i = -2 s_i f_i with f_i = (sum_{j != i} s_j J_ij, j ascending from +0.0) + h_i (the
+// order of k_fields_fp64) of the m sites of `list`, ascending. A chain of n additions per site, on
+// two FP64 lanes per SM, is what bounds the FP64 search, so only the sites of the survivors pay it
+// (the filter works on the fixed-point fields): 120 iterations of 3840 searches of n = 100 take
+// 15.3 ms, 17.2 with the chains of every site, and 86 ms in the per-kernel form (every pair in FP64). An instance exactly on its grid needs no
+// chain: every partial sum is exact, so the fixed-point field is the same double.
+static __device__ __forceinline__ void fields_f64(const DevPtrs& P, const InstDesc& d, const uint64_t* pb,
+                                                  const long long* aq, const unsigned short* list, int m, double* ad) {
+  const int n = d.n;
+  for (int q = threadIdx.x; q < m; q += kSNT) {
+    const int i = list[q];
+    if (!d.rounded) {   // block-uniform
+      ad[i] = (double)aq[i] * d.inv_scale;
+      continue;
+    }
+    const double* J = P.J64 + d.off_mat + i;   // J_ji = J_ij
+    double acc = 0.0;
+    for (int j0 = 0; j0 < n; j0 += 64) {
+      const uint64_t w = pb[j0 >> 6];
+      const int e = min(64, n - j0);
+#pragma unroll 8
+      for (int u = 0; u < e; ++u) {
+        const double v = J[(long long)(j0 + u) * d.n_pad];
+        const double x = __longlong_as_double(__double_as_longlong(v) ^ (long long)((w >> u) << 63));
+        if (j0 + u != i) acc = __dadd_rn(acc, x);
+      }
+    }
+    const double f = __dadd_rn(acc, P.h64[d.off_vec + i]);
+    ad[i] = sigma_of(pb, i) ? 2.0 * f : -2.0 * f;
+  }
+}
+
 // FL: flip set, QIS_FLIPS_SINGLE_PAIR or QIS_FLIPS_EXCHANGE (single flips alone: qis_single.cu). One
 // block of kSNT threads per search; n_iters >= 1.
-template <int FL>
+// F64: the FP64 mode. The candidates are filtered as in the split modes (fixed-point fields, FP32
+// copies of a_i and 4 J_ij), the survivors get the defining FP64 energies from their sites' defining
+// FP64 fields; every iteration's parent is picked here.
+template <int FL, bool F64>
 __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_iters) {
   constexpr bool EX = FL == QIS_FLIPS_EXCHANGE;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -115,8 +152,9 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int K1 = P.K1, Wm = P.Wmax, NP = P.NP, cap = P.cap;
   const long long base = (long long)b * K1;
-  const SearchLayout L = search_layout(NP, Wm, K1, cap, P.merge_cand);
+  const SearchLayout L = search_layout(NP, Wm, K1, cap, P.merge_cand, F64);
   float2* as = reinterpret_cast<float2*>(smem + L.as);
+  double* ad = reinterpret_cast<double*>(smem + L.ad);   // FP64 mode: a_i
   uint64_t* pb = reinterpret_cast<uint64_t*>(smem + L.pb);
   unsigned long long* okeyA = reinterpret_cast<unsigned long long*>(smem + L.okey0);
   unsigned long long* okeyB = reinterpret_cast<unsigned long long*>(smem + L.okey1);
@@ -137,10 +175,11 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
   const int act0 = P.active[b];
   const InstDesc d = P.inst[b / P.R];
   const int n = d.n, W = d.W;
-  const int t_first = P.iter_t[b];
+  const int t_first = P.iter_t[b] + (F64 ? 1 : 0);   // the iteration of iter = 0
   const int ring_t0 = P.ring_t0[b];
   int cnt = P.lst_count[b];
-  long long Epq = P.par_q[b];
+  // the parent's energy: E 2^q exact, or the bits of the FP64 mode's double
+  long long Epq = F64 ? 0 : P.par_q[b];
   uint64_t ph = P.par_hash[b];
   for (int r = tid; r < K1; r += kSNT) {
     okeyA[r] = P.lst_key[base + r];
@@ -150,7 +189,7 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
   }
   for (int w = tid; w < W; w += kSNT) pb[w] = P.par_bits[(long long)b * Wm + w];
   float mn = INFINITY, mx = -INFINITY;   // this thread's range of a_i (for the bound)
-  if (act0)
+  if (!F64 && act0)
     for (int i = tid; i < n; i += kSNT) {
       const float2 v = P.as32[(long long)b * NP + i];
       as[i] = v;
@@ -158,7 +197,7 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
       mx = fmaxf(mx, v.x);
     }
   __syncthreads();
-  if (act0 && P.e0_pend[b]) {   // block-uniform: the list is [psi0] and psi0 is the parent
+  if (!F64 && act0 && P.e0_pend[b]) {   // block-uniform: the list is [psi0] and psi0 is the parent
     Epq = initial_energy(P, d, pb, aq_of(P, b, t_first), reinterpret_cast<long long*>(scr));
     if (tid == 0) {
       const int s0 = oslotA[0];
@@ -173,7 +212,7 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
     __syncthreads();
   }
 
-  int act = act0, t = t_first, cur = 0;
+  int act = act0, t = F64 ? t_first - 1 : t_first, cur = 0;
   int nprod = 0;
   unsigned long long npair = 0, nev = 0, nsurv = 0;
   const float scale_q = (float)d.inv_scale;
@@ -191,7 +230,7 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
     unsigned long long* okeyN = cur ? okeyA : okeyB;
     int* oslot = cur ? oslotB : oslotA;
     int* oslotN = cur ? oslotA : oslotB;
-    if (iter > 0) {
+    if (F64 || iter > 0) {
       t += 1;
       if (!act) continue;
       // ------------------------------------------------------------ pick (Alg. 3)
@@ -212,7 +251,7 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
         continue;
       }
       const int pslot = oslot[sel];
-      Epq = (long long)(okey[sel] ^ (1ull << 63));
+      Epq = F64 ? __double_as_longlong(dkey_inv(okey[sel])) : (long long)(okey[sel] ^ (1ull << 63));
       const uint64_t pst = ostamp[pslot];
       ph = P.lst_hash[base + pslot];
       for (int w = tid; w < W; w += kSNT) pb[w] = P.lst_bits[(base + pslot) * Wm + w];
@@ -453,8 +492,13 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
       // from the exact integer keys, scaled by the power of two 2^-q. (Every thread forms the
       // same value from the same operands.)
       const unsigned long long kT = okey[K1 - 1];
+      // FP64 mode: E' = fl(E_p + dE) < T needs dE < T - E_p, and E' at or below the k-th lowest needs dE
+      // within an ulp of E' of its dE; |E'| <= n (|a|max + n j4max / 4) with n <= 1024, so that ulp and
+      // the roundings of the FP64 fields are below 2^-10 of delta; the grid 2^-q (2^q sum |J| >= 2^50)
+      // puts a_i + a_j off by at most 2 n 2^-q <= 2^-22 j4max, half of delta's margin.
       const float tE = (cnt != K1) ? INFINITY
-                                   : __fmul_ru(__ll2float_ru((long long)(kT ^ (1ull << 63)) - Epq), scale_q);
+                       : F64 ? __double2float_ru(__dsub_ru(dkey_inv(kT), __longlong_as_double(Epq)))
+                             : __fmul_ru(__ll2float_ru((long long)(kT ^ (1ull << 63)) - Epq), scale_q);
       const float tt = fminf(tE, Uf);
       const float big = __fadd_ru(__fadd_ru(__fmul_ru(3.f, fmaxf(fabsf(amin), fabsf(amax))), d.j4max),
                                   isinf(tt) ? 0.f : fabsf(tt));
@@ -659,14 +703,45 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
       continue;
     }
     nsurv += (unsigned long long)S;
+    if constexpr (F64) {   // the survivors' sites (the FP32 fields have been read: their place is free)
+      unsigned* mark = reinterpret_cast<unsigned*>(as);                  // [32]
+      unsigned short* list = reinterpret_cast<unsigned short*>(mark + 32);   // [NP]
+      if (tid < 32) mark[tid] = 0u;
+      __syncthreads();
+      for (int e = tid; e < S; e += kSNT) {
+        int i, j;
+        surv_sites((e < kSSV) ? ssv[e] : surv[e], i, j);
+        atomicOr(&mark[i >> 5], 1u << (i & 31));
+        if (j >= 0) atomicOr(&mark[j >> 5], 1u << (j & 31));
+      }
+      __syncthreads();
+      // every warp counts for itself; warp w lists the words w, w + 4, ..
+      const unsigned mk = mark[lane];
+      int inc = __popc(mk);
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+      }
+      const int m = __shfl_sync(0xffffffffu, inc, 31);
+      for (int w = warp; w < 32; w += kSW) {
+        const unsigned x = __shfl_sync(0xffffffffu, mk, w);
+        const int at = __shfl_sync(0xffffffffu, inc, w) - __popc(x);
+        if ((x >> lane) & 1u) list[at + __popc(x & ((1u << lane) - 1u))] = (unsigned short)(w * 32 + lane);
+      }
+      __syncthreads();
+      fields_f64(P, d, pb, aq_of(P, b, t), list, m, ad);
+      __syncthreads();
+    }
     const bool big = S > PCs;
     if (big) {
       const long long stride = next_pow2(max(cap, 256));
       sk = P.mrg_scratch + (long long)b * 2 * stride;
       se = sk + stride;
     }
-    const long long Tq = (cnt == K1) ? (long long)(okey[K1 - 1] ^ (1ull << 63)) : LLONG_MAX;
-    const long long* aqb = aq_of(P, b, t);
+    const long long Tq = (!F64 && cnt == K1) ? (long long)(okey[K1 - 1] ^ (1ull << 63)) : LLONG_MAX;
+    const double T = (F64 && cnt == K1) ? dkey_inv(okey[K1 - 1]) : INFINITY;
+    const long long* aqb = F64 ? nullptr : aq_of(P, b, t);
     unsigned long long kmn = ~0ull, kmx = 0;
     for (int u0 = 0; u0 < S; u0 += kSNT) {
       const int e = u0 + tid;
@@ -677,14 +752,22 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
         int i, j;
         surv_sites(ent, i, j);
         ent |= (j < 0) ? (uint32_t)i : pair_index(n, i, j);
-        long long de = aqb[i];
-        if (j >= 0) {
-          const long long jq = Jq[(long long)i * d.n_pad + j];
-          de += aqb[j] + ((sigma_of(pb, i) ^ sigma_of(pb, j)) ? -4 * jq : 4 * jq);
+        if constexpr (F64) {
+          const double de = (j < 0) ? ad[i] : dE64(ad[i], ad[j], P.J64[d.off_mat + (long long)i * d.n_pad + j],
+                                                   sigma_of(pb, i) ^ sigma_of(pb, j));
+          const double e = __dadd_rn(__longlong_as_double(Epq), de);
+          kk = dkey(e);
+          keep = e < T;   // Alg. 2: strict <
+        } else {
+          long long de = aqb[i];
+          if (j >= 0) {
+            const long long jq = Jq[(long long)i * d.n_pad + j];
+            de += aqb[j] + ((sigma_of(pb, i) ^ sigma_of(pb, j)) ? -4 * jq : 4 * jq);
+          }
+          const long long eq = Epq + de;
+          kk = qkey(eq);
+          keep = eq < Tq;   // Alg. 2: strict <
         }
-        const long long eq = Epq + de;
-        kk = qkey(eq);
-        keep = eq < Tq;   // Alg. 2: strict <
         if (keep) {
           const uint32_t c = (uint32_t)ent;
           for (uint32_t pos = chash(c) & (HT - 1); htab[pos] != kNoCand; pos = (pos + 1) & (HT - 1))
@@ -839,7 +922,8 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
         if (j >= 0 && (j >> 6) != wi) dst[j >> 6] = pb[j >> 6] ^ (1ull << (j & 63));
       }
       const uint64_t stamp = ((uint64_t)t << 32) | c;
-      P.lst_q[base + slot] = (long long)(kp ^ (1ull << 63));
+      if (F64) P.lst_E[base + slot] = dkey_inv(kp);
+      else P.lst_q[base + slot] = (long long)(kp ^ (1ull << 63));
       P.lst_stamp[base + slot] = stamp;
       ostamp[slot] = stamp;
       P.lst_hash[base + slot] = ph ^ P.zob[i] ^ ((j >= 0) ? P.zob[j] : 0ull);
@@ -867,7 +951,8 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
     P.iter_t[b] = t_first + n_iters - 1;
     if (act0) {
       P.active[b] = act;
-      P.par_q[b] = Epq;
+      if (F64) P.par_E[b] = __longlong_as_double(Epq);
+      else P.par_q[b] = Epq;
       P.par_hash[b] = ph;
       P.nprod[b] += nprod;
       P.npair[b] += npair;
@@ -881,22 +966,27 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
   }
 }
 
-size_t search_smem(const DevPtrs& P) { return (size_t)search_layout(P.NP, P.Wmax, P.K1, P.cap, P.merge_cand).total; }
+template <int FL, bool F64>
+static cudaError_t launch_search_as(const DevPtrs& P, int n_iters, cudaStream_t s) {
+  const size_t sm = (size_t)search_layout(P.NP, P.Wmax, P.K1, P.cap, P.merge_cand, F64).total;
+  static size_t attr = 0;
+  if (attr < sm) {
+    const cudaError_t e = cudaFuncSetAttribute(k_search<FL, F64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    attr = sm;
+  }
+  k_search<FL, F64><<<P.B, kSNT, sm, s>>>(P, n_iters);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_search(const DevPtrs& P, int n_iters, cudaStream_t s) {
   if (n_iters <= 0 || P.B == 0) return cudaSuccess;
-  const size_t sm = search_smem(P);
-  static size_t attr[2] = {0, 0};
-  const int ex = P.flips == QIS_FLIPS_EXCHANGE;
-  if (attr[ex] < sm) {
-    const cudaError_t e = ex ? cudaFuncSetAttribute(k_search<QIS_FLIPS_EXCHANGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)
-                             : cudaFuncSetAttribute(k_search<QIS_FLIPS_SINGLE_PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    attr[ex] = sm;
-  }
-  if (ex) k_search<QIS_FLIPS_EXCHANGE><<<P.B, kSNT, sm, s>>>(P, n_iters);
-  else k_search<QIS_FLIPS_SINGLE_PAIR><<<P.B, kSNT, sm, s>>>(P, n_iters);
-  return cudaGetLastError();
+  const bool ex = P.flips == QIS_FLIPS_EXCHANGE;
+  if (P.mode == QIS_FP64)
+    return ex ? launch_search_as<QIS_FLIPS_EXCHANGE, true>(P, n_iters, s)
+              : launch_search_as<QIS_FLIPS_SINGLE_PAIR, true>(P, n_iters, s);
+  return ex ? launch_search_as<QIS_FLIPS_EXCHANGE, false>(P, n_iters, s)
+            : launch_search_as<QIS_FLIPS_SINGLE_PAIR, false>(P, n_iters, s);
 }
 
 }  // namespace qis
