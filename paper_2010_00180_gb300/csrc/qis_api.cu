@@ -255,7 +255,7 @@ int launch_iterations_fused(qis_ctx* ctx, int n, cudaStream_t s) {
   const DevPtrs& P = ctx->P;
   if (ctx->mode == QIS_FP64) {   // picks and computes the fields of every iteration itself
     CK(prof_begin(ctx, 5));
-    LAUNCH(launch_search(P, n, s));
+    for (int i = 0; i < n; i += P.pw_n) LAUNCH(launch_search(P, std::min(n - i, P.pw_n), 0, s));
     CK(prof_end(ctx, 5));
     return 0;
   }
@@ -270,7 +270,7 @@ int launch_iterations_fused(qis_ctx* ctx, int n, cudaStream_t s) {
   if (ctx->cfg.flips == QIS_FLIPS_SINGLE) {
     for (int i = 0; i < n; i += P.pw_n) LAUNCH(launch_single(P, std::min(n - i, P.pw_n), i == 0, s));
   } else {
-    LAUNCH(launch_search(P, n, s));
+    for (int i = 0; i < n; i += P.pw_n) LAUNCH(launch_search(P, std::min(n - i, P.pw_n), i == 0, s));
   }
   CK(prof_end(ctx, 5));
   return 0;
@@ -348,6 +348,24 @@ int build_work(qis_ctx* ctx) {
 }
 
 }  // namespace
+
+void qis::gf_tables(GfTables& g) {
+  const int N = kGfSites - 1;
+  memset(&g, 0, sizeof(g));
+  for (int e = 0, x = 1; e < N; ++e) {
+    g.exp[e] = g.exp[e + N] = (uint16_t)x;
+    g.log[x] = (uint32_t)e | ((uint32_t)(3 * (N - e) % N) << 16);
+    x <<= 1;
+    if (x & kGfSites) x ^= kGfSites | 9;
+  }
+  std::vector<uint16_t> sol(kGfSites, (uint16_t)kGfNone);
+  for (int y = 0; y < kGfSites; y += 2) {   // y and y + 1 solve for the same c
+    const int c = (y ? g.exp[2 * (int)(g.log[y] & 0xffffu)] : 0) ^ y;
+    sol[c] = y ? (uint16_t)(g.log[y] & 0xffffu) : (uint16_t)kGfZero;
+  }
+  for (int e = 0; e < 2 * N; ++e) g.root[e] = sol[g.exp[e] ^ 1];
+  g.root1 = sol[1];
+}
 
 void qis::set_global_error(const char* msg) { g_create_error = msg; }
 
@@ -463,7 +481,8 @@ int qis_create(const qis_config* cfg, qis_ctx** out) {
     ALLOC(P.lst_ord, B * K1);
     ALLOC(P.lst_count, B);
     P.pw_n = 0;
-    if (ctx->mode != QIS_FP64 && ctx->cfg.flips == QIS_FLIPS_SINGLE && ctx->K1 <= kSearchMaxK1) {
+    if (ctx->K1 <= kSearchMaxK1 && (ctx->mode == QIS_FP64 ? ctx->f64_filter
+                                                          : ctx->cfg.flips == QIS_FLIPS_SINGLE || ctx->NP <= kSearchMaxNP)) {
       // the parents' words of a launch's iterations: as many as fit in 1 GiB, 8 .. 128
       P.pw_n = (int)std::min<size_t>(128, std::max<size_t>(8, (1ull << 30) / (B * W * sizeof(uint64_t))));
       ALLOC(P.pw, B * (size_t)P.pw_n * W);
@@ -546,8 +565,18 @@ int qis_create(const qis_config* cfg, qis_ctx** out) {
     }
     // Zobrist keys of the sites (SplitMix64 stream with a fixed key)
     std::vector<uint64_t> z(kMaxN);
-    for (int i = 0; i < kMaxN; ++i)   // the site itself in the low bits (qis_single.cu reads it there)
+    // the site in the low 14 bits and, for the sites of the pair searches, its cube in the next 10
+    // (near_sites reads the flips between two states from the XOR of their hashes)
+    GfTables gf;
+    gf_tables(gf);
+    GfTables* gf_d = nullptr;
+    ALLOC(gf_d, 1);
+    CK(cudaMemcpy(gf_d, &gf, sizeof(gf), cudaMemcpyHostToDevice));
+    P.gf = gf_d;
+    for (int i = 0; i < kMaxN; ++i) {
       z[i] = (splitmix64(0x2F0A7B6C5D4E3F21ull, (uint64_t)i) & ~(uint64_t)kSiteMask) | (uint64_t)i;
+      if (i < kGfSites) z[i] = (z[i] & ~((uint64_t)(kGfSites - 1) << 14)) | ((uint64_t)gf_cube(gf, i) << 14);
+    }
     CK(cudaMemcpy(ctx->zob, z.data(), kMaxN * sizeof(uint64_t), cudaMemcpyHostToDevice));
     // kernel attributes for the large dynamic shared-memory users
     CK(cudaDeviceSynchronize());

@@ -72,47 +72,55 @@ static __device__ float value_select_upper(const float* v, int cnt, int rank, in
   return mx;
 }
 
-// Candidate index of the kept state x if it is one or two flips from the parent p (the single
-// flip of its differing site, or the pair of its two), else -1. The words are compared in
-// order, four loads in flight per step, and the test stops at the third differing bit: most
-// kept states differ in more sites, so most tests read only their first words, while a state
-// that is near (the parent itself among them) costs a round trip per four words instead of one
-// per word (a rolled loop over the four: a small body fetches better than all W in flight).
-static __device__ __forceinline__ long long near_code_sp(const uint64_t* x, const uint64_t* p, int W, int n) {
-  int dist = 0, q0 = 0, q1 = 0;
-#pragma unroll 1
-  for (int w = 0; w < W; w += 4) {
-    const uint64_t x0 = x[w];
-    const uint64_t x1 = (w + 1 < W) ? x[w + 1] : 0ull;
-    const uint64_t x2 = (w + 2 < W) ? x[w + 2] : 0ull;
-    const uint64_t x3 = (w + 3 < W) ? x[w + 3] : 0ull;
-    uint64_t v = x0 ^ p[w];
-    uint64_t v1 = (w + 1 < W) ? (x1 ^ p[w + 1]) : 0ull;
-    uint64_t v2 = (w + 2 < W) ? (x2 ^ p[w + 2]) : 0ull;
-    uint64_t v3 = (w + 3 < W) ? (x3 ^ p[w + 3]) : 0ull;
-#pragma unroll 1
-    for (int u = 0; u < 4; ++u) {   // word w + u in v
-      while (v) {
-        const int pos = (w + u) * 64 + __ffsll((long long)v) - 1;
-        if (dist == 0) q0 = pos; else q1 = pos;
-        ++dist;
-        v &= v - 1;
-        if (dist > 2) return -1;
+// The flips of a state one or two flips from another from the XOR x of their Zobrist hashes (n up to
+// kGfSites): the keys hold the site i in their low 14 bits and i^3 in GF(2^10) in the next 10, so
+// x holds S1 = i + j and S3 = i^3 + j^3, the syndromes of a code that corrects two errors: with
+// i = S1 y, y^2 + y = S3 / S1^3 + 1, read from tables of logarithms and solutions. A state that is not
+// near decodes to nothing or to flips whose keys do not give x (but for a chance of 2^-40: the
+// caller compares the words). gf: GfTables on the device. Sites come with i < j, j = -1 for one flip.
+static __device__ __forceinline__ bool near_sites(uint64_t x, const GfTables* __restrict__ gf,
+                                                  const uint64_t* __restrict__ zob, int n, int& i, int& j) {
+  const int s1 = (int)(x & kSiteMask), s3 = (int)(x >> 14) & (kGfSites - 1);
+  if (x == 0 || s1 >= kGfSites) return false;
+  i = 0;
+  j = s1;   // y = 0: sites 0 and s1, or the one site s1
+  if (s1) {
+    const uint32_t l1 = gf->log[s1];
+    const int ly = s3 ? gf->root[(gf->log[s3] & 0xffffu) + (l1 >> 16)] : gf->root1;   // log y
+    if (ly == kGfNone) return false;
+    if (ly != kGfZero) {
+      i = gf->exp[ly + (int)(l1 & 0xffffu)];
+      j = i ^ s1;
+      if (max(i, j) >= n || (zob[i] ^ zob[j]) != x) return false;
+      if (i > j) {
+        const int tmp = i;
+        i = j;
+        j = tmp;
       }
-      v = v1;
-      v1 = v2;
-      v2 = v3;
-      v3 = 0ull;
+      return true;
     }
   }
-  if (dist == 1) return q0;
-  if (dist == 2) return pair_index(n, q0, q1);
-  return -1;
+  if (s1 >= n) return false;
+  if (zob[s1] == x) {
+    i = s1;
+    j = -1;
+    return true;
+  }
+  return s1 != 0 && (zob[0] ^ zob[s1]) == x;
 }
 
-// The same test for wide states (the per-kernel form, n above 1024): the words are loaded ten at
-// a time (one round trip per ten words) and the test stops after the batch that holds the third
-// differing bit.
+// Minimum / maximum of a 64-bit key over the warp (every lane gets it), in 32-bit reductions.
+static __device__ __forceinline__ unsigned long long warp_min64(unsigned long long x) {
+  const unsigned h = __reduce_min_sync(0xffffffffu, (unsigned)(x >> 32));
+  const unsigned l = __reduce_min_sync(0xffffffffu, (unsigned)(x >> 32) == h ? (unsigned)x : 0xffffffffu);
+  return (unsigned long long)h << 32 | l;
+}
+static __device__ __forceinline__ unsigned long long warp_max64(unsigned long long x) { return ~warp_min64(~x); }
+
+// Candidate index of the kept state x if it is one or two flips from the parent p (the single
+// flip of its differing site, or the pair of its two), else -1 (the per-kernel form): the words are
+// loaded ten at a time (one round trip per ten words) and the test stops after the batch that holds
+// the third differing bit.
 static __device__ __forceinline__ long long near_code_batched(const uint64_t* x, const uint64_t* p, int W, int n) {
   int dist = 0, p0 = 0, p1 = 0;
   for (int w0 = 0; w0 < W; w0 += 10) {

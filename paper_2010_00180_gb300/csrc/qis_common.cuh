@@ -17,6 +17,21 @@ constexpr int kMaxN = 16384;
 constexpr int kSiteMask = kMaxN - 1;   // the low bits of a site's Zobrist key hold the site
 constexpr int kScan64Group = 4;  // searches per block of the FP64 pair scan
 
+// Logarithms and square-equation solutions in GF(2^10) (x^10 + x^3 + 1, generator x): the tables that
+// decode the XOR of two Zobrist hashes into at most two sites (near_sites).
+constexpr int kGfSites = 1024;
+constexpr int kGfNone = 0xffff, kGfZero = 0xfffe;
+struct GfTables {
+  uint32_t log[kGfSites];       // log s | log s^-3 << 16 (s > 0)
+  uint16_t exp[2 * kGfSites];   // of 0 .. 2 (2^10 - 2)
+  uint16_t root[2 * kGfSites];  // by e: log of y with y^2 + y = exp(e) + 1, kGfZero for y = 0, kGfNone
+  uint16_t root1;               // the same for y^2 + y = 1
+};
+void gf_tables(GfTables& g);
+inline int gf_cube(const GfTables& g, int s) {   // s^3
+  return s ? g.exp[3 * (int)(g.log[s] & 0xffffu) % (kGfSites - 1)] : 0;
+}
+
 // Device error flags (bit mask in ctx status word).
 constexpr int kStatCapacity = 1;
 constexpr int kStatTimeout = 2;
@@ -66,8 +81,9 @@ struct DevPtrs {
   uint64_t* lst_stamp;    // [b][K1]
   uint64_t* lst_hash;     // [b][K1]
   uint8_t* lst_used;      // [b][K1]
-  uint64_t* pw;           // [b][pw_n][Wmax] parents' words of the iterations of a launch (single flips)
-  int pw_n;               // iterations per launch of the single-flip search kernel
+  uint64_t* pw;           // [b][pw_n][Wmax] parents' words of the iterations of a launch (fused kernels)
+  int pw_n;               // iterations per launch of the fused search kernels
+  const GfTables* gf;     // near-state decoding
   int* lst_ord;           // [b][K1] slot of rank r
   int* lst_count;         // [b]
   uint64_t* par_bits;     // [b][Wmax]
@@ -150,7 +166,7 @@ __host__ __device__ inline int pad_of(int n) { return (n + kPad - 1) / kPad * kP
 
 // candidate index <-> sites: c < n single i = c; c >= n pair (i, j), i < j, lexicographic
 __host__ __device__ inline uint32_t pair_index(int n, int i, int j) {
-  return (uint32_t)n + (uint32_t)((long long)i * n - (long long)i * (i + 1) / 2 + (j - i - 1));
+  return (uint32_t)(n + i * n - i * (i + 1) / 2 + (j - i - 1));   // (n <= 16384: below 2^28)
 }
 // Survivor entry: bits 32-45 site i, bits 46-59 site j, bit 60 set for a single flip (no j);
 // n <= 16384 keeps i and j in 14 bits. The candidate filters (singles by k_bound, pairs by the
@@ -172,18 +188,18 @@ __host__ __device__ inline void surv_decode(unsigned long long e, uint32_t& c, i
 
 __device__ inline void decode_candidate(int n, uint32_t c, int& i, int& j) {
   if (c < (uint32_t)n) { i = (int)c; j = -1; return; }
-  long long r = (long long)c - n;
+  const int r = (int)c - n;   // (n <= 16384: every product below stays below 2^28)
   // row i holds n-1-i pairs; start(i) = i*n - i*(i+1)/2. The closed form in FP32 lands within
-  // a step or two of the row (r < 2^23); the integer loops below make it exact. (FP64 here
+  // a few steps of the row (r < 2^27); the integer loops below make it exact. (FP64 here
   // would cost every thread a double square root on GB300's narrow FP64 pipe.)
   const float nn = 2.f * n - 1.f;
   int ii = (int)((nn - sqrtf(fmaxf(nn * nn - 8.f * (float)r, 0.f))) * 0.5f);
   if (ii < 0) ii = 0;
   if (ii > n - 2) ii = n - 2;
-  while (ii > 0 && (long long)ii * n - (long long)ii * (ii + 1) / 2 > r) --ii;
-  while (ii < n - 2 && (long long)(ii + 1) * n - (long long)(ii + 1) * (ii + 2) / 2 <= r) ++ii;
+  while (ii > 0 && ii * n - ii * (ii + 1) / 2 > r) --ii;
+  while (ii < n - 2 && (ii + 1) * n - (ii + 1) * (ii + 2) / 2 <= r) ++ii;
   i = ii;
-  j = (int)(r - ((long long)ii * n - (long long)ii * (ii + 1) / 2)) + ii + 1;
+  j = r - (ii * n - ii * (ii + 1) / 2) + ii + 1;
 }
 
 __device__ inline int sigma_of(const uint64_t* bits, int i) { return (int)((bits[i >> 6] >> (i & 63)) & 1ull); }
@@ -251,35 +267,31 @@ __device__ inline double dkey_inv(unsigned long long k) {
   return __longlong_as_double((long long)((k & 0x8000000000000000ull) ? (k & 0x7fffffffffffffffull) : ~k));
 }
 
-// Warp-parallel search of a 256-bin histogram: the bin holding the rank-th element (0-based),
-// and the rank of that element within the bin. Called by one full warp.
+// Warp-parallel search of a 256-bin histogram (16-byte aligned): the bin holding the rank-th element
+// (0-based), and the rank of that element within the bin. Called by one full warp.
 __device__ inline void find_bin(const int* hist, int rank, int& bin, int& within) {
   const int lane = threadIdx.x & 31;
-  int loc[8], s = 0;
+  const int4 x = reinterpret_cast<const int4*>(hist)[2 * lane], y = reinterpret_cast<const int4*>(hist)[2 * lane + 1];
+  const int loc[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+  int s = 0;
 #pragma unroll
-  for (int u = 0; u < 8; ++u) {
-    loc[u] = hist[lane * 8 + u];
-    s += loc[u];
-  }
+  for (int u = 0; u < 8; ++u) s += loc[u];
   int incl = s;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
+    const int z = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += z;
   }
   const unsigned m = __ballot_sync(0xffffffffu, incl > rank);
   const int L = m ? __ffs(m) - 1 : 31;
-  int r = rank - __shfl_sync(0xffffffffu, incl - s, L);
-  int bb = 255;
-  if (lane == L) {
-    int u = 0;
-    for (; u < 7; ++u) {
-      if (r < loc[u]) break;
-      r -= loc[u];
+  int r = rank - (incl - s), u = 0;   // meaningful on lane L
+#pragma unroll
+  for (int v = 0; v < 7; ++v)
+    if (u == v && r >= loc[v]) {
+      r -= loc[v];
+      ++u;
     }
-    bb = L * 8 + u;
-  }
-  bin = __shfl_sync(0xffffffffu, bb, L);
+  bin = __shfl_sync(0xffffffffu, lane * 8 + u, L);
   within = __shfl_sync(0xffffffffu, r, L);
 }
 
@@ -350,8 +362,9 @@ constexpr int kSparseMaxNP = 4096;   // the sparse pair scan's largest padded n 
 // list length (per-search arrays in shared memory).
 constexpr int kSearchMaxNP = 1024;
 constexpr int kSearchMaxK1 = 256;
-cudaError_t launch_search(const DevPtrs& P, int n_iters, cudaStream_t s);
-// Single flips: any padded n, at most P.pw_n iterations per launch.
+// At most P.pw_n iterations per launch; ext: the first one's parent and fields are in place.
+cudaError_t launch_search(const DevPtrs& P, int n_iters, int ext, cudaStream_t s);
+// Single flips: any padded n.
 cudaError_t launch_single(const DevPtrs& P, int n_iters, int ext, cudaStream_t s);
 cudaError_t launch_fields_tc(const DevPtrs& P, const void* D16, const void* S16, int max_inst, int digits_max,
                              int nt, cudaStream_t s);

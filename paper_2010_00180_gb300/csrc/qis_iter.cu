@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(128, 10) k_bound(DevPtrs P) {
   const int n = d.n;
   const bool fp64 = P.mode == QIS_FP64;
   extern __shared__ unsigned long long subkey[];     // [kSubMax] (u32 keys reuse the front)
-  __shared__ int hist[256], hist2[256];
+  __shared__ __align__(16) int hist[256], hist2[256];
   __shared__ int sites[kSubSites];
   __shared__ int s_nsites, s_n2, s_bin, s_bin2, s_near, s_ns;
   __shared__ float s_thr;

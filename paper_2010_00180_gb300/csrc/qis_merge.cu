@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(kMergeThreads, 8) k_merge(DevPtrs P) {
   //          (each later one has K+1 new states below it), so keep the keys up to the (K+1)-th
   //          smallest (ties included) before sorting; compaction in place, chunk by chunk
   if (nv > (int)blockDim.x && nv > K1) {
-    __shared__ int hist[256];
+    __shared__ __align__(16) int hist[256];
     const unsigned long long x = radix_select<unsigned long long>(sk, nv, K1 - 1, hist);
     int kept = 0;
     for (int t0 = 0; t0 < nv; t0 += blockDim.x) {

@@ -118,7 +118,8 @@ __global__ void __launch_bounds__(256) k_na_select(int n, const double* J, const
   float* sub = reinterpret_cast<float*>(na_smem);                             // [kSubMax], before the candidates
   __shared__ double a[kNaMaxN];
   __shared__ uint64_t pb[kNaMaxN / 64];
-  __shared__ int hist[256], sites[kSubSites], off[kNaBlocks + 1];
+  __shared__ __align__(16) int hist[256];
+  __shared__ int sites[kSubSites], off[kNaBlocks + 1];
   __shared__ int s_ns, s_bin, s_cnt, s_last;
   __shared__ double s_e[8];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;

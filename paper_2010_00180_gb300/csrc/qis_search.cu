@@ -8,43 +8,56 @@
 //   fields  its exact integer fields from its generating parent's, held in the aq ring, minus
 //           the flipped sites' coupling columns (the Sec. III energy algebra; a parent whose
 //           generator is no longer in the ring gets them from a full row sum instead);
-//           a_i = -2 s_i f_i
-//   bound   filter threshold (the last kept energy and an order-statistic bound), the kept
-//           states one or two flips from the parent (the only possible duplicates), singles
-//   scan    pair flips dE_ij = a_i + a_j + 4 s_i s_j J_ij decided by the output-sensitive scan
+//           a_i = -2 s_i f_i. The sites with a_i up to a cut, guessed from the last iteration, are
+//           listed on the way: only they can be flipped by a candidate that enters the list, and
+//           what follows works on this list (a fifth of the sites at n = 600) in a bucket order of a_i
+//   near    the kept states one or two flips from the parent (the only possible duplicates), from
+//           the flips of its own generation and from the hashes of the others (near_sites)
+//   bound   filter threshold: the last kept energy and an order-statistic bound from the flips of
+//           the lowest listed sites; a list that does not reach what the threshold needs is
+//           taken again
+//   scan    pair flips dE_ij = a_i + a_j + 4 s_i s_j J_ij decided by the output-sensitive scan: a
+//           live row's partners are the sites after it in the order, up to the bucket of its bound
 //   merge   exact integer keys of the survivors, duplicates dropped, the new states ranked by
 //           a counting sort over buckets of their keys (no sort), first K+1 of the old list and
 //           the new states by (E, stamp)
-// The kept list's order, keys, stamps and used flags, the parent's spins and {a_i, s_i} stay in
-// shared memory across the iterations; the kept states' bits, the aq ring and the survivor
-// buffer are in global memory (written and read by this block only, within the L2 cache).
+// The kept list's order, keys, flips, hashes and used flags and the parent's spins stay in shared
+// memory across the iterations; a new state is kept as (iteration, flips), its words being its
+// parent's (stored per iteration) with at most two bits flipped, and the words are written into
+// the list once, at the end of the launch. The aq ring and the survivors past 512 are in global
+// memory (written and read by this block only, within the L2 cache).
 // Split modes: the first iteration's parent is picked, and its fields computed (update, or the
 // tensor-core GEMM for a parent without a stored generator), by the kernels launched before this one.
 // FP64 mode: the same filter, the survivors' energies in the defining FP64 arithmetic.
-// The arithmetic of every phase is that of the per-kernel form (k_bound, k_scan_sparse,
-// k_merge), so the kept lists are identical bit for bit.
+// Every decision is that of the per-kernel form (k_bound, k_scan_sparse, k_merge), so the kept
+// lists are identical bit for bit.
+//
+// What bounds it: the latency and issue of many short dependent steps (32 warps per SM at 64
+// registers, about 2 instructions per SM cycle); no phase takes more than a sixth of the time. 7680
+// searches of n = 600, 120 iterations: 31.9 ms with passes over all sites for each of histogram,
+// selection, rows, bucket counts and order, with the near states found by comparing words, and with
+// every new state's words written in every iteration; 26.6 ms with the listed sites, hashes and
+// words at the end; 21.7 ms with the own generation's near states from their flips alone.
 #include "qis_block.cuh"
 
 namespace qis {
 
-constexpr int kSNT = 128;          // threads of a search block
-constexpr int kSW = kSNT / 32;      // its warps
-constexpr int kSMinBlocks = 8;      // resident blocks per SM the register budget is set for
+constexpr int kSSV = 512;   // survivors held in shared memory (more go to the global buffer)
 
 __host__ __device__ inline int search_pcs(int cap, int merge_cand) {
   const int pc = next_pow2(cap > 256 ? cap : 256);
   return pc < merge_cand ? pc : merge_cand;
 }
 
-// Byte offsets of the dynamic shared memory of a search block.
+// Byte offsets of the dynamic shared memory of a search block of `warps` warps.
 struct SearchLayout {
-  int as, ad, pb, okey0, okey1, ostamp, oslot0, oslot1, htab, ssv, oused, scratch, total;
-  int sc;   // bytes of the scratch region
+  int pb, okey0, okey1, oflip, ohash, oslot0, oslot1, htab, ssv, oused, ogen, ad, scratch, total;
+  // the scratch region while candidates are found (later the merge's): the low sites as taken and in
+  // order, the rows' list offsets (the bound's histogram before), the buckets
+  int oa, orm, os, ua, us, pc, bs, bcur;
 };
 
-constexpr int kSSV = 512;   // survivors held in shared memory (more go to the global buffer)
-
-__host__ __device__ inline SearchLayout search_layout(int NP, int Wmax, int K1, int cap, int merge_cand, bool f64) {
+__host__ __device__ inline SearchLayout search_layout(int NP, int Wmax, int K1, int cap, int merge_cand, int warps, bool f64) {
   SearchLayout L;
   int o = 0;
   auto take = [&](int bytes) {
@@ -53,26 +66,30 @@ __host__ __device__ inline SearchLayout search_layout(int NP, int Wmax, int K1, 
     o += bytes;
     return r;
   };
-  L.as = take(NP * 8);
-  L.ad = take(f64 ? NP * 8 : 0);
   L.pb = take(Wmax * 8);
   L.okey0 = take(K1 * 8);
   L.okey1 = take(K1 * 8);
-  L.ostamp = take(K1 * 8);
+  L.ohash = take(K1 * 8);
+  L.oflip = take(K1 * 4);
   L.oslot0 = take(K1 * 4);
   L.oslot1 = take(K1 * 4);
   L.htab = take(next_pow2(2 * K1) * 4);
   L.ssv = take(kSSV * 8);
   L.oused = take(K1);
-  // scratch: the phases' working arrays, one phase at a time
-  const int bound = 4 * 256 * 4 + kSubSites * 4;
-  const int scan = 3 * NP * 4 + (2 * kSparseNB + 1) * 4;
-  const int merge = search_pcs(cap, merge_cand) * 16 + (512 + kMB + kSW * (kMB + 4)) * 4;
-  int sc = bound > scan ? bound : scan;
-  sc = sc > merge ? sc : merge;
-  L.scratch = take(sc);
-  L.sc = sc;
-  L.total = align_up(o, 16);
+  L.ogen = take(K1);
+  L.ad = take(f64 ? NP * 8 : 0);
+  o = align_up(o, 16);
+  L.scratch = o;
+  L.oa = take(NP * 4);
+  L.orm = take(NP * 4);
+  L.os = take(NP * 2);
+  L.ua = take(NP * 4);
+  L.us = take(NP * 2);
+  L.pc = take(NP * 4 > 2048 ? NP * 4 : 2048);
+  L.bs = take((kSparseNB + 1) * 4);
+  L.bcur = take(kSparseNB * 4);
+  const int merge = search_pcs(cap, merge_cand) * 16 + (512 + kMB + warps * (kMB + 4)) * 4;
+  L.total = align_up(o - L.scratch > merge ? o : L.scratch + merge, 16);
   return L;
 }
 
@@ -88,22 +105,15 @@ __device__ __forceinline__ float fkey_inv(unsigned k) {
 // Fields of a parent without a stored generator, from scratch: fq_k = hq_k + sum_j s_j Jq_jk
 // (columns coalesced), aq_k = -2 s_k fq_k. Rarely taken (out of line: the hot loop stays small).
 static __device__ __noinline__ void fields_full(const DevPtrs& P, const InstDesc& d, const uint64_t* pb,
-                                                long long* ax, float2* as, float& mn, float& mx) {
+                                                long long* ax) {
   const long long* Jq = P.Jq + d.off_mat;
-  const float scale_q = (float)d.inv_scale;
   for (int k = threadIdx.x; k < d.n; k += blockDim.x) {
     long long acc = P.hq[d.off_vec + k];
     for (int jj = 0; jj < d.n; ++jj) {
       const long long v = Jq[(long long)jj * d.n_pad + k];
       acc += sigma_of(pb, jj) ? -v : v;
     }
-    const int sx = sigma_of(pb, k);
-    const long long aq = sx ? 2 * acc : -2 * acc;
-    const float a = __ll2float_rn(aq) * scale_q;
-    ax[k] = aq;
-    as[k] = make_float2(a, sx ? -1.f : 1.f);
-    mn = fminf(mn, a);
-    mx = fmaxf(mx, a);
+    ax[k] = sigma_of(pb, k) ? 2 * acc : -2 * acc;
   }
 }
 
@@ -116,7 +126,7 @@ static __device__ __noinline__ void fields_full(const DevPtrs& P, const InstDesc
 static __device__ __forceinline__ void fields_f64(const DevPtrs& P, const InstDesc& d, const uint64_t* pb,
                                                   const long long* aq, const unsigned short* list, int m, double* ad) {
   const int n = d.n;
-  for (int q = threadIdx.x; q < m; q += kSNT) {
+  for (int q = threadIdx.x; q < m; q += blockDim.x) {
     const int i = list[q];
     if (!d.rounded) {   // block-uniform
       ad[i] = (double)aq[i] * d.inv_scale;
@@ -139,65 +149,162 @@ static __device__ __forceinline__ void fields_f64(const DevPtrs& P, const InstDe
   }
 }
 
+// The candidate sites of an iteration, from scratch (out of line: the first iteration of a launch, or
+// when the cut guessed from the last one does not reach far enough): the sites with a_i <= cut (inf:
+// every site) in a monotone bucket order of a_i. Returns their number; lo and inv are the buckets'.
+// amin, amax: the range of a_i (known = false: found here).
+struct LowSites {
+  float *oa, *orm, *ua;
+  unsigned short *os, *us;
+  int *bs, *bcur;
+};
+
+static __device__ __forceinline__ void set_buckets(float amin, float amax, float cut, float& lo, float& inv) {
+  const float span = __fsub_ru(fminf(cut, amax), amin);
+  lo = amin;
+  inv = (span > 0.f && span < INFINITY) ? __fdiv_rn((float)kSparseNB, span) : 0.f;
+}
+
+// Exclusive starts of the bucket counts in cur, into bs (kSparseNB + 1) and cur. One warp.
+static __device__ __forceinline__ void bucket_starts(int* cur, int* bs) {
+  const int lane = threadIdx.x & 31;
+  int x[kSparseNB / 32], s = 0;
+#pragma unroll
+  for (int q = 0; q < kSparseNB / 32; ++q) {
+    x[q] = cur[lane * (kSparseNB / 32) + q];
+    s += x[q];
+  }
+  int inc = s;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  int acc = inc - s;
+#pragma unroll
+  for (int q = 0; q < kSparseNB / 32; ++q) {
+    bs[lane * (kSparseNB / 32) + q] = acc;
+    cur[lane * (kSparseNB / 32) + q] = acc;
+    acc += x[q];
+  }
+  if (lane == 31) bs[kSparseNB] = acc;
+}
+
+static __device__ __noinline__ int low_sites_again(const long long* ax, const float* rm, int n, float scale_q,
+                                                   const uint64_t* pb, const LowSites& S, int* s_cn, bool known,
+                                                   float& amin, float& amax, float cut, float& lo, float& inv) {
+  if (!known) {
+    float mn = INFINITY, mx = -INFINITY;
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+      const float v = __ll2float_rn(ax[k]) * scale_q;
+      mn = fminf(mn, v);
+      mx = fmaxf(mx, v);
+    }
+    block_min_max(mn, mx);
+    amin = mn;
+    amax = mx;
+  }
+  set_buckets(amin, amax, cut, lo, inv);
+  __syncthreads();
+  if (threadIdx.x == 0) *s_cn = 0;
+  for (int x = threadIdx.x; x < kSparseNB; x += blockDim.x) S.bcur[x] = 0;
+  __syncthreads();
+  for (int k = threadIdx.x; k < n; k += blockDim.x) {
+    const float v = __ll2float_rn(ax[k]) * scale_q;
+    if (v <= cut) {
+      const int e = atomicAdd(s_cn, 1);
+      S.ua[e] = v;
+      S.us[e] = (unsigned short)(k | (sigma_of(pb, k) << 15));
+      atomicAdd(&S.bcur[sparse_bucket(v, lo, inv)], 1);
+    }
+  }
+  __syncthreads();
+  const int cn = *s_cn;
+  if (threadIdx.x < 32) bucket_starts(S.bcur, S.bs);
+  __syncthreads();
+  for (int e = threadIdx.x; e < cn; e += blockDim.x) {
+    const float v = S.ua[e];
+    const unsigned short s = S.us[e];
+    const int q = atomicAdd(&S.bcur[sparse_bucket(v, lo, inv)], 1);
+    S.oa[q] = v;
+    S.os[q] = s;
+    S.orm[q] = rm[s & 0x7fff];
+  }
+  __syncthreads();
+  return cn;
+}
+
 // FL: flip set, QIS_FLIPS_SINGLE_PAIR or QIS_FLIPS_EXCHANGE (single flips alone: qis_single.cu). One
-// block of kSNT threads per search; n_iters >= 1.
+// block of NT threads per search; 1 <= n_iters <= P.pw_n. ext: the first iteration's parent was
+// picked and its fields computed by the kernels launched before this one (split modes).
 // F64: the FP64 mode. The candidates are filtered as in the split modes (fixed-point fields, FP32
 // copies of a_i and 4 J_ij), the survivors get the defining FP64 energies from their sites' defining
-// FP64 fields; every iteration's parent is picked here.
-template <int FL, bool F64>
-__global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_iters) {
+// FP64 fields.
+template <int FL, bool F64, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters, int ext) {
   constexpr bool EX = FL == QIS_FLIPS_EXCHANGE;
+  constexpr int NW = NT / 32;
   extern __shared__ __align__(16) unsigned char smem[];
   const int b = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int K1 = P.K1, Wm = P.Wmax, NP = P.NP, cap = P.cap;
+  const int K1 = P.K1, Wm = P.Wmax, cap = P.cap;
   const long long base = (long long)b * K1;
-  const SearchLayout L = search_layout(NP, Wm, K1, cap, P.merge_cand, F64);
-  float2* as = reinterpret_cast<float2*>(smem + L.as);
-  double* ad = reinterpret_cast<double*>(smem + L.ad);   // FP64 mode: a_i
+  const SearchLayout L = search_layout(P.NP, Wm, K1, cap, P.merge_cand, NW, F64);
   uint64_t* pb = reinterpret_cast<uint64_t*>(smem + L.pb);
   unsigned long long* okeyA = reinterpret_cast<unsigned long long*>(smem + L.okey0);
   unsigned long long* okeyB = reinterpret_cast<unsigned long long*>(smem + L.okey1);
-  uint64_t* ostamp = reinterpret_cast<uint64_t*>(smem + L.ostamp);
+  uint32_t* oflip = reinterpret_cast<uint32_t*>(smem + L.oflip);   // of a state of this launch: i | j << 16 (j = 0xffff: none)
+  uint64_t* ohash = reinterpret_cast<uint64_t*>(smem + L.ohash);
   int* oslotA = reinterpret_cast<int*>(smem + L.oslot0);
   int* oslotB = reinterpret_cast<int*>(smem + L.oslot1);
   uint32_t* htab = reinterpret_cast<uint32_t*>(smem + L.htab);
   unsigned long long* ssv = reinterpret_cast<unsigned long long*>(smem + L.ssv);
   const int HT = next_pow2(2 * K1);
   uint8_t* oused = reinterpret_cast<uint8_t*>(smem + L.oused);
+  uint8_t* ogen = reinterpret_cast<uint8_t*>(smem + L.ogen);
+  double* ad = reinterpret_cast<double*>(smem + L.ad);   // FP64 mode: a_i of the survivors' sites
   unsigned char* scr = smem + L.scratch;
+  const LowSites LS = {reinterpret_cast<float*>(smem + L.oa), reinterpret_cast<float*>(smem + L.orm),
+                       reinterpret_cast<float*>(smem + L.ua), reinterpret_cast<unsigned short*>(smem + L.os),
+                       reinterpret_cast<unsigned short*>(smem + L.us), reinterpret_cast<int*>(smem + L.bs),
+                       reinterpret_cast<int*>(smem + L.bcur)};
+  float *oa = LS.oa, *orm = LS.orm;
+  unsigned short* os = LS.os;   // site | sigma << 15
+  int *bs = LS.bs, *bcur = LS.bcur;
+  int* pc = reinterpret_cast<int*>(smem + L.pc);
+  int* vhist = pc;                                              // [256] the bound's values per bin
+  unsigned* vmax = reinterpret_cast<unsigned*>(vhist + 256);    // [256] and their maxima
 
-  __shared__ int s_sel, s_near, s_ns, s_nsites, s_n2, s_bin, s_bin2, s_nl, s_nv, s_ocut;
-  __shared__ float wf[2 * kSW];
+  __shared__ int s_sel, s_near, s_ns, s_nv, s_ocut, s_cn, s_m0, s_m1;
+  __shared__ float wf[2 * NW];
   __shared__ int s_w[33];
-  __shared__ unsigned long long s_kmin, s_kmax;
+  __shared__ unsigned long long s_kmm[2 * NW];
+  __shared__ unsigned short s_ex[kSubSites];   // exchanges: the bound's sites of each spin class (positions)
 
   const int act0 = P.active[b];
   const InstDesc d = P.inst[b / P.R];
   const int n = d.n, W = d.W;
-  const int t_first = P.iter_t[b] + (F64 ? 1 : 0);   // the iteration of iter = 0
+  const int t_first = P.iter_t[b] + (ext ? 0 : 1);   // the iteration of iter = 0
   const int ring_t0 = P.ring_t0[b];
   int cnt = P.lst_count[b];
   // the parent's energy: E 2^q exact, or the bits of the FP64 mode's double
   long long Epq = F64 ? 0 : P.par_q[b];
   uint64_t ph = P.par_hash[b];
-  for (int r = tid; r < K1; r += kSNT) {
+  uint64_t* pw = P.pw + (long long)b * P.pw_n * Wm;   // words of the parent of iteration iter: pw + iter Wm
+  for (int r = tid; r < K1; r += NT) {
     okeyA[r] = P.lst_key[base + r];
     oslotA[r] = P.lst_ord[base + r];
-    ostamp[r] = P.lst_stamp[base + r];
+    ohash[r] = P.lst_hash[base + r];
     oused[r] = P.lst_used[base + r];
+    ogen[r] = 0;   // in lst_bits (else 1 + the iteration of this launch that generated it)
   }
-  for (int w = tid; w < W; w += kSNT) pb[w] = P.par_bits[(long long)b * Wm + w];
-  float mn = INFINITY, mx = -INFINITY;   // this thread's range of a_i (for the bound)
-  if (!F64 && act0)
-    for (int i = tid; i < n; i += kSNT) {
-      const float2 v = P.as32[(long long)b * NP + i];
-      as[i] = v;
-      mn = fminf(mn, v.x);
-      mx = fmaxf(mx, v.x);
-    }
+  for (int w = tid; w < W; w += NT) {
+    const uint64_t x = P.par_bits[(long long)b * Wm + w];
+    pb[w] = x;
+    if (ext) pw[w] = x;
+  }
   __syncthreads();
-  if (!F64 && act0 && P.e0_pend[b]) {   // block-uniform: the list is [psi0] and psi0 is the parent
+  if (!F64 && act0 && ext && P.e0_pend[b]) {   // block-uniform: the list is [psi0] and psi0 is the parent
     Epq = initial_energy(P, d, pb, aq_of(P, b, t_first), reinterpret_cast<long long*>(scr));
     if (tid == 0) {
       const int s0 = oslotA[0];
@@ -212,27 +319,44 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
     __syncthreads();
   }
 
-  int act = act0, t = F64 ? t_first - 1 : t_first, cur = 0;
-  int nprod = 0;
+  int act = act0, t = t_first - 1, cur = 0, nprod = 0;
+  int pgen = 0, pi0 = -1, pj0 = -1;   // the parent's generation in this launch and its flips
   unsigned long long npair = 0, nev = 0, nsurv = 0;
   const float scale_q = (float)d.inv_scale;
   const long long* Jq = P.Jq + d.off_mat;
   const float* J4 = P.J4 + d.off_mat;
+  const float* rm = P.rm4 + d.off_vec;
   unsigned long long* surv = P.surv + (long long)b * cap;
   // survivor slot s: shared memory below kSSV, the search's global buffer above (up to cap)
   auto put_surv = [&](int slot, unsigned long long e) {
     if (slot < kSSV) ssv[slot] = e;
     else if (slot < cap) surv[slot] = e;
   };
+  // the cut and the buckets of the candidate sites, guessed from the last iteration (ranged)
+  bool ranged = false;
+  float cut = INFINITY, lo = 0.f, inv = 0.f;
 
   for (int iter = 0; iter < n_iters; ++iter) {
     unsigned long long* okey = cur ? okeyB : okeyA;
     unsigned long long* okeyN = cur ? okeyA : okeyB;
     int* oslot = cur ? oslotB : oslotA;
     int* oslotN = cur ? oslotA : oslotB;
-    if (F64 || iter > 0) {
-      t += 1;
-      if (!act) continue;
+    t += 1;
+    if (!act) continue;
+    // this iteration's counters (the last one's reads are behind its last barrier)
+    if (tid == 0) {
+      s_near = 0;
+      s_ns = 0;
+      s_nv = 0;
+      s_cn = 0;
+      s_ocut = cnt;
+    }
+    for (int x = tid; x < HT; x += NT) htab[x] = kNoCand;
+    for (int x = tid; x < kSparseNB; x += NT) bcur[x] = 0;
+    for (int x = tid; x < 512; x += NT) vhist[x] = 0;
+    float mn = INFINITY, mx = -INFINITY;   // this thread's range of a_i
+    const long long* aqb = aq_of(P, b, t);
+    if (F64 || iter > 0 || !ext) {
       // ------------------------------------------------------------ pick (Alg. 3)
       if (warp == 0) {
         int sel = -1;
@@ -252,35 +376,49 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
       }
       const int pslot = oslot[sel];
       Epq = F64 ? __double_as_longlong(dkey_inv(okey[sel])) : (long long)(okey[sel] ^ (1ull << 63));
-      const uint64_t pst = ostamp[pslot];
-      ph = P.lst_hash[base + pslot];
-      for (int w = tid; w < W; w += kSNT) pb[w] = P.lst_bits[(base + pslot) * Wm + w];
-      __syncthreads();   // the parent's words; every thread has read s_sel and the used flags
-      if (tid == 0) {
-        oused[pslot] = 1;
-        P.lst_used[base + pslot] = 1;
+      ph = ohash[pslot];
+      // the iteration tg that generated it and its flips there
+      const int gen = ogen[pslot];
+      int i, j, tg;
+      if (gen) {
+        tg = t_first + gen - 1;
+        i = (int)(oflip[pslot] & 0xffffu);
+        j = (int)(short)(oflip[pslot] >> 16);
+      } else {
+        const uint64_t pst = P.lst_stamp[base + pslot];
+        tg = (int)(pst >> 32);
+        decode_candidate(n, (uint32_t)pst, i, j);
       }
+      pgen = gen;
+      pi0 = i;
+      pj0 = j;
+      // the parent's words: its own, or its generator's with the flipped bits
+      for (int w = tid; w < W; w += NT) {
+        const uint64_t x = gen ? pw[(long long)(gen - 1) * Wm + w] ^ flip_mask(w, i, j) : P.lst_bits[(base + pslot) * Wm + w];
+        pb[w] = x;
+        pw[(long long)iter * Wm + w] = x;
+      }
+      __syncthreads();   // the parent's words; every thread has read s_sel and the used flags
+      if (tid == 0) oused[pslot] = 1;
       ++nprod;
-      if (FL == QIS_FLIPS_SINGLE_PAIR) npair += (unsigned long long)n * (n - 1) / 2;
+      if (!EX) npair += (unsigned long long)n * (n - 1) / 2;
       if (EX) {
         int down = 0;
         for (int w = 0; w < W; ++w) down += __popcll(pb[w]);
         npair += (unsigned long long)down * (unsigned long long)(n - down);
       }
       // ------------------------------------------------------------ fields
-      // x = the parent, entered at iteration tg as candidate c of that iteration's parent g
-      const int tg = (int)(pst >> 32);
-      long long* __restrict__ ax = aq_of(P, b, t);
+      // x = the parent, a candidate of iteration tg's parent g
+      long long* ax = aq_of(P, b, t);
       if (tg >= 1 && tg > ring_t0 && tg < t && t - tg < P.ring_n) {
-        int i, j;
-        decode_candidate(n, (uint32_t)pst, i, j);
-        const long long* __restrict__ ag = aq_of(P, b, tg);
+        const long long* ag = aq_of(P, b, tg);
         const long long* __restrict__ Ji = Jq + (long long)i * d.n_pad;   // row i = column i
         const long long* __restrict__ Jj = Jq + (long long)max(j, 0) * d.n_pad;
         // one site per thread and pass, pipelined: the next site's three loads are issued before
         // the current site's fields are formed. With s_g = -s_x at the flipped sites i, j,
         //   aq_x,k = s_x,k s_g,k aq_g,k + 4 s_x,k (s_g,i Jq_ik + s_g,j Jq_jk),
-        // s_g,i = +1 where the parent's bit i is set (exact int64)
+        // s_g,i = +1 where the parent's bit i is set (exact int64). The sites up to the guessed cut
+        // are listed and counted into their buckets on the way.
         const bool pi = sigma_of(pb, i) != 0;
         const bool pj = j >= 0 && sigma_of(pb, j) != 0;
         long long g_n = 0, i_n = 0, j_n = 0;
@@ -293,27 +431,76 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
         };
         load(tid);
 #pragma unroll 1
-        for (int k = tid; k < n; k += kSNT) {
+        for (int k0 = 0; k0 < n; k0 += NT) {
+          const int k = k0 + tid;
           const long long vg = g_n, vi = i_n, vj = j_n;
-          load(k + kSNT);
-          const int sx = sigma_of(pb, k);
-          const long long tt = (pi ? vi : -vi) + (j >= 0 ? (pj ? vj : -vj) : 0);
-          const long long aq = ((k == i || k == j) ? -vg : vg) + (sx ? -4 * tt : 4 * tt);
-          const float a = __ll2float_rn(aq) * scale_q;
-          ax[k] = aq;
-          as[k] = make_float2(a, sx ? -1.f : 1.f);
-          mn = fminf(mn, a);
-          mx = fmaxf(mx, a);
+          load(k + NT);
+          bool in = false;
+          float v = 0.f;
+          int sx = 0;
+          if (k < n) {
+            sx = sigma_of(pb, k);
+            const long long tt = (pi ? vi : -vi) + (j >= 0 ? (pj ? vj : -vj) : 0);
+            const long long aq = ((k == i || k == j) ? -vg : vg) + (sx ? -4 * tt : 4 * tt);
+            v = __ll2float_rn(aq) * scale_q;
+            ax[k] = aq;
+            mn = fminf(mn, v);
+            mx = fmaxf(mx, v);
+            in = ranged && v <= cut;
+          }
+          const unsigned m = __ballot_sync(0xffffffffu, in);
+          if (m) {
+            int e = 0;
+            if (lane == 0) e = atomicAdd(&s_cn, __popc(m));
+            e = __shfl_sync(0xffffffffu, e, 0) + __popc(m & ((1u << lane) - 1u));
+            if (in) {
+              LS.ua[e] = v;
+              LS.us[e] = (unsigned short)(k | (sx << 15));
+              atomicAdd(&bcur[sparse_bucket(v, lo, inv)], 1);
+            }
+          }
         }
       } else {
-        fields_full(P, d, pb, ax, as, mn, mx);   // no stored generator
+        fields_full(P, d, pb, ax);   // no stored generator
+        ranged = false;
       }
-    } else if (!act) {
-      continue;
+    } else {
+      __syncthreads();   // the counters and tables are cleared
     }
-    // ---------------------------------------------------------------- bound
-    // range of a over the block; the kept states one or two flips from the parent (their
-    // candidate indices: the only candidates that can be duplicates, each equal to exactly one)
+    // ---------------------------------------------------------------- near states
+    // the kept states one or two flips from the parent: the only candidates that can be
+    // duplicates, each equal to exactly one. A state of the parent's own generation differs from it
+    // by the symmetric difference of their flips. Any other's hash XOR the parent's decodes to the
+    // flips it would be (near_sites), and only then are the words compared: the state is its
+    // generator's words with two flips at most, so its difference from the parent has to be exactly
+    // the bits that the four flips leave.
+    for (int r = tid; r < cnt; r += NT) {
+      const int g = ogen[r];
+      int i, j;
+      const int ci = (int)(oflip[r] & 0xffffu), cj = (int)(short)(oflip[r] >> 16);   // (of a state of this launch)
+      if (g && g == pgen) {
+        const bool a = ci != pi0 && ci != pj0, c = cj >= 0 && cj != pi0 && cj != pj0;
+        const bool e = pi0 != ci && pi0 != cj, f = pj0 >= 0 && pj0 != ci && pj0 != cj;
+        const int m = a + c + e + f;
+        if (m == 0 || m > 2) continue;
+        const int x = a ? ci : c ? cj : e ? pi0 : pj0;     // the first and the last of them
+        const int y = f ? pj0 : e ? pi0 : c ? cj : ci;
+        i = min(x, y);
+        j = m == 2 ? max(x, y) : -1;
+      } else {
+        if (!near_sites(ohash[r] ^ ph, P.gf, P.zob, n, i, j)) continue;
+        const uint64_t* src = g ? pw + (long long)(g - 1) * Wm : P.lst_bits + (base + r) * Wm;
+        uint64_t diff = 0;
+#pragma unroll 1
+        for (int w = 0; w < W; ++w)
+          diff |= src[w] ^ pb[w] ^ flip_mask(w, i, j) ^ (g ? flip_mask(w, ci, cj) : 0ull);
+        if (diff) continue;
+      }
+      const uint32_t c = j < 0 ? (uint32_t)i : pair_index(n, i, j);
+      atomicAdd(&s_near, 1);
+      uint32_t pos = chash(c) & (HT - 1);
+      while (atomicCAS(&htab[pos], kNoCand, c) != kNoCand) pos = (pos + 1) & (HT - 1);
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
@@ -321,57 +508,44 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
     }
     if (lane == 0) {
       wf[warp] = mn;
-      wf[kSW + warp] = mx;
+      wf[NW + warp] = mx;
     }
-    if (tid == 0) {
-      s_near = 0;
-      s_ns = 0;
-      s_nsites = 0;
-      s_n2 = 0;
-      s_nl = 0;
-      s_nv = 0;
-      s_ocut = cnt;
-      s_kmin = ~0ull;
-      s_kmax = 0;
-    }
-    for (int x = tid; x < HT; x += kSNT) htab[x] = kNoCand;
-    {
-      int* hist = reinterpret_cast<int*>(scr);   // the bound's histograms, cleared for this iteration
-      for (int x = tid; x < 4 * 256; x += kSNT) hist[x] = 0;
-    }
-    __syncthreads();   // the fields and the range are complete
-    float amin = wf[0], amax = wf[kSW];
+    __syncthreads();   // the fields, their range, the listed sites and the near states are complete
+    const int k = K1 + s_near;
+    float amin = wf[0], amax = wf[NW];
 #pragma unroll
-    for (int w = 1; w < kSW; ++w) {
+    for (int w = 1; w < NW; ++w) {
       amin = fminf(amin, wf[w]);
-      amax = fmaxf(amax, wf[kSW + w]);
+      amax = fmaxf(amax, wf[NW + w]);
     }
-    mn = INFINITY;
-    mx = -INFINITY;
-    for (int r = tid; r < cnt; r += kSNT) {
-      const long long c = near_code_sp(P.lst_bits + (base + r) * Wm, pb, W, n);
-      if (c >= 0) {
-        atomicAdd(&s_near, 1);
-        uint32_t pos = chash((uint32_t)c) & (HT - 1);
-        while (atomicCAS(&htab[pos], kNoCand, (uint32_t)c) != kNoCand) pos = (pos + 1) & (HT - 1);
+    // ---------------------------------------------------------------- candidate sites in order
+    int cn;
+    if (ranged) {   // block-uniform
+      cn = s_cn;
+      if (warp == 0) bucket_starts(bcur, bs);
+      __syncthreads();
+      for (int e = tid; e < cn; e += NT) {
+        const float v = LS.ua[e];
+        const unsigned short s = LS.us[e];
+        const int q = atomicAdd(&bcur[sparse_bucket(v, lo, inv)], 1);
+        oa[q] = v;
+        os[q] = s;
+        orm[q] = rm[s & 0x7fff];
       }
+      __syncthreads();
+    } else {
+      cut = INFINITY;
+      cn = low_sites_again(aqb, rm, n, scale_q, pb, LS, &s_cn, false, amin, amax, cut, lo, inv);
     }
-    __syncthreads();
-    const int ndup = s_near;
-    const int k = K1 + ndup;
+    // ---------------------------------------------------------------- bound
+    // an upper bound U of the k-th lowest candidate energy change: the k-th lowest among the flips of
+    // the lowest listed sites (any subset of the candidates bounds it)
     float Uf = INFINITY;
     int nu = 0;
     if (EX)
       for (int w = 0; w < W; ++w) nu += __popcll(pb[w]);
     const long long Ccand = EX ? (long long)nu * (n - nu) : (long long)n * (n + 1) / 2;
     if (Ccand > k && k <= kSubMax) {
-      // the bound's histograms (cleared before the fields barrier): site bins, the second spin
-      // class's site bins (exchanges), the subset values' counts and their per-bin maxima
-      int* hist = reinterpret_cast<int*>(scr);                        // [256]
-      int* hist2 = hist + 256;                                         // [256]
-      int* vhist = hist2 + 256;                                        // [256]
-      unsigned* vmax = reinterpret_cast<unsigned*>(vhist + 256);       // [256]
-      int* sites = reinterpret_cast<int*>(vmax + 256);                 // [kSubSites]
       const int want = min(3 * k, kSubMax);
       int t0 = 0, t1 = 0;
       if (EX) {
@@ -387,94 +561,74 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
           else if (md <= kSubSites / 2) mu = kSubSites - md;
           else mu = md = kSubSites / 2;
         }
-        t0 = mu;
-        t1 = md;
+        t0 = mu;   // down spins (sigma = 1)
+        t1 = md;   // up spins
       } else {
         int m = max(1, (int)((sqrtf(8.f * (float)want + 1.f) - 1.f) * 0.5f));
         while (m * (m + 1) / 2 < want) ++m;
         while (m > 1 && (m - 1) * m / 2 >= want) --m;
         t0 = min(min(m, n), kSubSites);
       }
-      const int lim0 = EX ? kSubSites - t1 : kSubSites;
-      const float scale = 255.99f / fmaxf(amax - amin, 1e-30f);
-      auto bin_of = [&](int i) { return min(255, (int)((as[i].x - amin) * scale)); };
-      for (int i = tid; i < n; i += kSNT) atomicAdd(&((EX && sigma_of(pb, i)) ? hist2 : hist)[bin_of(i)], 1);
-      __syncthreads();
-      if (warp == 0) {
-        int bin, within;
-        find_bin(hist, t0 - 1, bin, within);
-        if (lane == 0) s_bin = bin;
+      int m0 = 0, m1 = 0;
+      for (int again = 0; again < 2; ++again) {
         if (EX) {
-          find_bin(hist2, t1 - 1, bin, within);
-          if (lane == 0) s_bin2 = bin;
-        }
-      }
-      __syncthreads();
-      // the subset's values are binned as they are formed, over a range that holds them: every
-      // selected site has a below the upper edge of its class's cut bin (one bin of margin for
-      // the rounding of the binning), a pair lies within 4 max|J~| of a_i + a_j (values outside
-      // clamp to the end bins, which keeps the binning monotone)
-      const float cut0 = __fadd_ru(amin, __fdiv_ru((float)(s_bin + 2), scale));
-      const float cut1 = EX ? __fadd_ru(amin, __fdiv_ru((float)(s_bin2 + 2), scale)) : cut0;
-      const float hi_v = __fadd_ru(__fadd_ru(cut0, cut1), d.j4max);
-      const float lo_b = __fsub_rd(__fadd_rd(amin, amin), d.j4max);
-      const float scale_v = 255.99f / fmaxf(hi_v - lo_b, 1e-30f);
-      auto put_value = [&](float v) {
-        const int bin = min(255, max(0, (int)((v - lo_b) * scale_v)));
-        atomicAdd(&vhist[bin], 1);
-        atomicMax(&vmax[bin], fkey(v));
-      };
-      for (int i = tid; i < n; i += kSNT) {
-        const int c = EX ? sigma_of(pb, i) : 0;
-        if (bin_of(i) > (c ? s_bin2 : s_bin)) continue;
-        const int slot = atomicAdd(c ? &s_n2 : &s_nsites, 1);
-        if (slot < (c ? t1 : lim0)) sites[c ? lim0 + slot : slot] = i;
-      }
-      __syncthreads();
-      const int mm = min(s_nsites, lim0), m2 = min(s_n2, t1);
-      const int M = EX ? mm * m2 : mm + mm * (mm - 1) / 2;
-      auto member = [&](int q, int& i, int& j) {   // exchanges: (class 0 site, class 1 site)
-        i = sites[q / m2];
-        j = sites[lim0 + q % m2];
-        if (i > j) {
-          const int tmp = i;
-          i = j;
-          j = tmp;
-        }
-      };
-      if (M >= k) {
-        if (!EX) {
-          // the subset's singles, then its pairs row by row: warp w takes the rows x = w, w + 4,
-          // ..., its lanes the partners y > x (no index decoding; a warp reads one row of 4J~)
-          for (int q = tid; q < mm; q += kSNT) put_value(as[sites[q]].x);
-          for (int x = warp; x < mm; x += kSW) {
-            const int sx = sites[x];
-            for (int y = x + 1 + lane; y < mm; y += 32) {
-              const int sy = sites[y];
-              const int i = min(sx, sy), j = max(sx, sy);
-              const float j4 = J4[(long long)i * d.n_pad + j];
-              const float2 vj = as[j];
-              put_value(as[i].x + fmaf((sigma_of(pb, i) ? -j4 : j4), vj.y, vj.x));
+          // the first t0 down and t1 up positions of the order
+          if (warp == 0) {
+            int c0 = 0, c1 = 0;
+            for (int q0 = 0; q0 < cn && (c0 < t0 || c1 < t1); q0 += 32) {
+              const int q = q0 + lane;
+              const bool in = q < cn, dn = in && (os[q] >> 15);
+              const unsigned b0 = __ballot_sync(0xffffffffu, dn), b1 = __ballot_sync(0xffffffffu, in && !dn);
+              const unsigned below = (1u << lane) - 1u;
+              const int p = dn ? c0 + __popc(b0 & below) : c1 + __popc(b1 & below);
+              if (in && p < (dn ? t0 : t1)) s_ex[dn ? p : t0 + p] = (unsigned short)q;
+              c0 += __popc(b0);
+              c1 += __popc(b1);
+            }
+            if (lane == 0) {
+              s_m0 = min(c0, t0);
+              s_m1 = min(c1, t1);
             }
           }
+          __syncthreads();
+          m0 = s_m0;
+          m1 = s_m1;
         } else {
-          for (int q0 = 0; q0 < M; q0 += kSNT) {   // exchanges: pair q of the cross product
-            const int q = q0 + tid;
-            int i = 0, j = -1;
-            float j4 = 0.f;
-            if (q < M) {
-              member(q, i, j);
-              j4 = J4[(long long)i * d.n_pad + j];
-            }
-            if (q >= M) continue;
-            const float2 vj = as[j];
-            put_value(as[i].x + fmaf((sigma_of(pb, i) ? -j4 : j4), vj.y, vj.x));
-          }
+          m0 = min(t0, cn);
         }
+        if (cn == n || (m0 == t0 && (!EX || m1 == t1))) break;
+        // (rare) too few listed sites: every site
+        cut = INFINITY;
+        cn = low_sites_again(aqb, rm, n, scale_q, pb, LS, &s_cn, true, amin, amax, cut, lo, inv);
       }
-      if (M >= k) {
-        // U = the largest subset value in the bins up to the one holding the k-th smallest
-        // (binning is monotone, so at least k subset values are <= U): every warp alike
+      const int M = EX ? m0 * m1 : m0 * (m0 + 1) / 2;
+      if (M >= k) {   // block-uniform
+        // the values are binned as they are formed, over a range that holds nearly all of them (values
+        // outside clamp to the end bins, which keeps the binning monotone)
+        const float top = EX ? __fadd_rn(oa[s_ex[m0 - 1]], oa[s_ex[t0 + m1 - 1]]) : 2.f * oa[m0 - 1];
+        const float lo_b = __fsub_rd(__fadd_rd(amin, amin), d.j4max);
+        const float scale_v = 255.99f / fmaxf(__fadd_ru(top, d.j4max) - lo_b, 1e-30f);
+        auto put_value = [&](float v) {
+          const int bin = min(255, max(0, (int)((v - lo_b) * scale_v)));
+          atomicAdd(&vhist[bin], 1);
+          atomicMax(&vmax[bin], fkey(v));
+        };
+        auto pair_value = [&](int x, int y) {
+          const unsigned sx = os[x], sy = os[y];
+          const float j4 = J4[(long long)(sx & 0x7fff) * d.n_pad + (sy & 0x7fff)];
+          put_value(oa[x] + (oa[y] + (((sx ^ sy) & 0x8000u) ? -j4 : j4)));
+        };
+        if (!EX) {
+          // the sites' own flips, then their pairs row by row: warp w takes the rows x = w, w + NW, ..
+          for (int q = tid; q < m0; q += NT) put_value(oa[q]);
+          for (int x = warp; x < m0; x += NW)
+            for (int y = x + 1 + lane; y < m0; y += 32) pair_value(x, y);
+        } else {
+          for (int x = warp; x < m0; x += NW)
+            for (int y = lane; y < m1; y += 32) pair_value(s_ex[x], s_ex[t0 + y]);
+        }
+        // U = the largest value in the bins up to the one holding the k-th smallest (binning is
+        // monotone, so at least k values are <= U): every warp alike
         __syncthreads();
         int bsel, within;
         find_bin(vhist, k - 1, bsel, within);
@@ -505,197 +659,125 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
       const float delta = __fmul_ru(big, 0x1p-21f);
       thr = fminf(__fadd_ru(tE, delta), __fadd_ru(Uf, 2.f * delta));
     }
+    // every live row, single and partner has a_i <= need (rows: thr - a_i >= amin - rm_i, rm_i <= j4max;
+    // partners below); the listed sites have to reach it
+    const float need = fmaxf(thr, __fadd_ru(__fadd_ru(__fsub_ru(thr, amin), d.j4max),
+                                            __fmul_ru(0x1p-20f, fabsf(amin) + d.j4max + (isinf(thr) ? 0.f : fabsf(thr)))));
+    __syncthreads();   // the bound's values have been read: their place takes the rows' offsets
+    if (need > cut && cn < n) {   // block-uniform, rare
+      cut = need;
+      cn = low_sites_again(aqb, rm, n, scale_q, pb, LS, &s_cn, true, amin, amax, cut, lo, inv);
+    }
     // ---------------------------------------------------------------- scan (pairs; the single
-    // flips, dE_i = a_i, no candidates under exchanges, are tested in the live-row pass)
+    // flips, dE_i = a_i, no candidates under exchanges, are tested with the rows)
     {
-      int* li = reinterpret_cast<int*>(scr);   // [NP] live rows
-      int* pc = li + NP;                       // [NP] their rm, then list offsets
-      int* cj = pc + NP;                       // [NP] columns in bucket order
-      int* bs = cj + NP;                       // [kSparseNB + 1]
-      int* bcur = bs + kSparseNB + 1;          // [kSparseNB]
-      // the row of each pair, while the pairs fit the rest of the scratch
-      unsigned short* rowof = reinterpret_cast<unsigned short*>(bcur + kSparseNB);
-      const int rcap = (L.sc - (3 * NP + 2 * kSparseNB + 1) * 4) / 2;
-      const float* rm = P.rm4 + d.off_vec;
-      __syncthreads();   // the bound's scratch is free
-      for (int x = tid; x < kSparseNB; x += kSNT) bcur[x] = 0;
-      float bl = -INFINITY;
-      constexpr int SB = 5;
-      for (int i0 = 0; i0 < n; i0 += SB * kSNT) {
-        float r[SB];
-#pragma unroll
-        for (int u = 0; u < SB; ++u) {
-          const int i = i0 + tid + u * kSNT;
-          r[u] = (i < n) ? rm[i] : 0.f;
+      // the row of each pair, while the pairs fit the space of the sites as listed
+      unsigned short* rowof = reinterpret_cast<unsigned short*>(smem + L.ua);
+      const int rcap = P.NP * 3;
+      const int per = (cn + NT - 1) / NT, q0 = min(cn, tid * per), q1 = min(cn, q0 + per);
+      int sum = 0;
+      for (int q = q0; q < q1; ++q) {
+        const float ai = oa[q], r = orm[q];
+        if (!EX && ai <= thr) put_surv(atomicAdd(&s_ns, 1), surv_entry(os[q] & 0x7fff, -1));
+        const float c = __fsub_rn(thr, ai);
+        int len = 0;
+        if (c >= __fsub_rd(amin, r)) {   // a live row: its partners have a_j < nextup(c) + r
+          const float up = __fadd_ru(__fmaf_ru(fabsf(c), 0x1p-23f, c), 1.2e-38f);   // >= nextup(c)
+          len = max(0, bs[sparse_bucket(__fadd_ru(up, r), lo, inv) + 1] - q - 1);
         }
-#pragma unroll
-        for (int u = 0; u < SB; ++u) {
-          const int i = i0 + tid + u * kSNT;
-          if (i < n) {
-            const float ai = as[i].x;
-            if (!EX && ai <= thr) put_surv(atomicAdd(&s_ns, 1), surv_entry(i, -1));
-            const float c = __fsub_rn(thr, ai);
-            if (c >= __fsub_rd(amin, r[u])) {
-              const int q = atomicAdd(&s_nl, 1);
-              li[q] = i;
-              pc[q] = __float_as_int(r[u]);
-              bl = fmaxf(bl, __fadd_ru(nextafterf(c, INFINITY), r[u]));
-            }
-          }
-        }
+        pc[q] = len;
+        sum += len;
       }
+      int inc = sum;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) bl = fmaxf(bl, __shfl_xor_sync(0xffffffffu, bl, o));
-      if (lane == 0) wf[warp] = bl;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+      }
+      if (lane == 31) s_w[warp] = inc;
       __syncthreads();
-      const int nl = s_nl;
-      if (nl > 0) {   // block-uniform
-        float B = wf[0];
+      int acc = inc - sum, tot = 0;
 #pragma unroll
-        for (int w = 1; w < kSW; ++w) B = fmaxf(B, wf[w]);
-        const float span = __fsub_ru(B, amin);
-        const float inv = (span > 0.f && span < INFINITY) ? __fdiv_rn((float)kSparseNB, span) : 0.f;
-        for (int j = tid; j < n; j += kSNT)
-          if (as[j].x < B) atomicAdd(&bcur[sparse_bucket(as[j].x, amin, inv)], 1);
-        __syncthreads();
-        if (warp == 0) {
-          int x[kSparseNB / 32], s = 0;
-#pragma unroll
-          for (int q = 0; q < kSparseNB / 32; ++q) {
-            x[q] = bcur[lane * (kSparseNB / 32) + q];
-            s += x[q];
-          }
-          int inc = s;
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += y;
-          }
-          int acc = inc - s;
-#pragma unroll
-          for (int q = 0; q < kSparseNB / 32; ++q) {
-            bs[lane * (kSparseNB / 32) + q] = acc;
-            bcur[lane * (kSparseNB / 32) + q] = acc;
-            acc += x[q];
-          }
-          if (lane == 31) bs[kSparseNB] = acc;
-        }
-        __syncthreads();
-        // site code in place of s_j: (position in the column order << 1) | sigma_j, or INT_MIN |
-        // sigma_j for a site at or above B
-        for (int j = tid; j < n; j += kSNT) {
-          const float2 v = as[j];
-          const int sg = v.y < 0.f;
-          int code = INT_MIN | sg;
-          if (v.x < B) {
-            const int q = atomicAdd(&bcur[sparse_bucket(v.x, amin, inv)], 1);
-            cj[q] = j;
-            code = (q << 1) | sg;
-          }
-          as[j].y = __int_as_float(code);
-        }
-        for (int q = tid; q < nl; q += kSNT) {
-          const int i = li[q];
-          const float c = __fsub_rn(thr, as[i].x), rr = __int_as_float(pc[q]);
-          pc[q] = bs[sparse_bucket(__fadd_ru(nextafterf(c, INFINITY), rr), amin, inv) + 1];
-        }
-        __syncthreads();
-        {
-          const int per = (nl + kSNT - 1) / kSNT, q0 = min(nl, tid * per), q1 = min(nl, q0 + per);
-          int sum = 0;
-          for (int q = q0; q < q1; ++q) {
-            const int code = __float_as_int(as[li[q]].y);
-            const int x = code < 0 ? 0 : max(0, pc[q] - (code >> 1) - 1);
-            pc[q] = x;
-            sum += x;
-          }
-          int inc = sum;
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += y;
-          }
-          if (lane == 31) s_w[warp] = inc;
-          __syncthreads();
-          int acc = inc - sum;
-          for (int w = 0; w < warp; ++w) acc += s_w[w];
-          for (int q = q0; q < q1; ++q) {
-            const int x = pc[q];
-            pc[q] = acc;
-            for (int e = acc, e1 = min(acc + x, rcap); e < e1; ++e) rowof[e] = (unsigned short)q;
-            acc += x;
-          }
-        }
-        __syncthreads();
-        int tot = 0;
-#pragma unroll
-        for (int w = 0; w < kSW; ++w) tot += s_w[w];
-        const bool direct = tot <= rcap;   // every pair's row in rowof (block-uniform)
-        // one pair per thread and pass, pipelined: the coupling load of the next pass's pair is
-        // issued before the current pair is tested
-        int ij_n = 0;
-        float cv_n = 0.f, av_n = 0.f, jv_n = 0.f;
-        bool ok_n = false, neg_n = false;
-        auto stage = [&](int e) {
-          ok_n = false;
-          if (e < tot) {
-            int lo = 0;
-            if (direct) {
-              lo = rowof[e];
-            } else {
-              int hi = nl;
-              while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if (pc[mid] <= e) lo = mid; else hi = mid;
-              }
+      for (int w = 0; w < NW; ++w) {
+        const int x = s_w[w];
+        if (w < warp) acc += x;
+        tot += x;
+      }
+      for (int q = q0; q < q1; ++q) {
+        const int x = pc[q];
+        pc[q] = acc;
+        for (int e = acc, e1 = min(acc + x, rcap); e < e1; ++e) rowof[e] = (unsigned short)q;
+        acc += x;
+      }
+      __syncthreads();
+      const bool direct = tot <= rcap;   // every pair's row in rowof (block-uniform)
+      // one pair per thread and pass, pipelined: the coupling load of the next pass's pair is
+      // issued before the current pair is tested
+      int ij_n = 0;
+      float cv_n = 0.f, av_n = 0.f, jv_n = 0.f;
+      bool ok_n = false, neg_n = false;
+      auto stage = [&](int e) {
+        ok_n = false;
+        if (e < tot) {
+          int q = 0;
+          if (direct) {
+            q = rowof[e];
+          } else {
+            int hi = cn;
+            while (hi - q > 1) {
+              const int mid = (q + hi) >> 1;
+              if (pc[mid] <= e) q = mid; else hi = mid;
             }
-            const int i = li[lo];
-            const float2 vi = as[i];
-            const int ci = __float_as_int(vi.y);
-            const int j = cj[(ci >> 1) + 1 + e - pc[lo]];
-            const float2 vj = as[j];
-            ij_n = min(i, j) | (max(i, j) << 16);
-            neg_n = ((ci ^ __float_as_int(vj.y)) & 1) != 0;
-            cv_n = __fsub_rn(thr, vi.x);
-            av_n = vj.x;
-            ok_n = !EX || neg_n;
-            if (ok_n) jv_n = J4[(long long)i * d.n_pad + j];
           }
-        };
-        stage(tid);
-        for (int u0 = 0; u0 < tot; u0 += kSNT) {
-          const int ij = ij_n;
-          const float cv = cv_n, av = av_n, jv = jv_n;
-          const bool ok = ok_n, neg = neg_n;
-          stage(u0 + kSNT + tid);
-          bool hit = false;
-          if (ok) {
-            ++nev;
-            hit = fmaf(neg ? -1.f : 1.f, jv, av) <= cv;
-          }
-          const unsigned m = __ballot_sync(0xffffffffu, hit);
-          if (m) {
-            const int leader = __ffs(m) - 1;
-            int sb = 0;
-            if (lane == leader) sb = atomicAdd(&s_ns, __popc(m));
-            sb = __shfl_sync(0xffffffffu, sb, leader);
-            const int slot = sb + __popc(m & ((1u << lane) - 1u));
-            if (hit) put_surv(slot, surv_entry(ij & 0xffff, ij >> 16));
-          }
+          const int q2 = q + 1 + e - pc[q];
+          const int si = os[q], sj = os[q2];
+          const int i = si & 0x7fff, j = sj & 0x7fff;
+          ij_n = min(i, j) | (max(i, j) << 16);
+          neg_n = ((si ^ sj) & 0x8000) != 0;
+          cv_n = __fsub_rn(thr, oa[q]);
+          av_n = oa[q2];
+          ok_n = !EX || neg_n;
+          if (ok_n) jv_n = J4[(long long)i * d.n_pad + j];
+        }
+      };
+      stage(tid);
+      for (int u0 = 0; u0 < tot; u0 += NT) {
+        const int ij = ij_n;
+        const float cv = cv_n, av = av_n, jv = jv_n;
+        const bool ok = ok_n, neg = neg_n;
+        stage(u0 + NT + tid);
+        bool hit = false;
+        if (ok) {
+          ++nev;
+          hit = fmaf(neg ? -1.f : 1.f, jv, av) <= cv;
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, hit);
+        if (m) {
+          const int leader = __ffs(m) - 1;
+          int sb = 0;
+          if (lane == leader) sb = atomicAdd(&s_ns, __popc(m));
+          sb = __shfl_sync(0xffffffffu, sb, leader);
+          const int slot = sb + __popc(m & ((1u << lane) - 1u));
+          if (hit) put_surv(slot, surv_entry(ij & 0xffff, ij >> 16));
         }
       }
     }
+    // the next iteration's guess: this one's need and a quarter of its span as a margin (the bound and
+    // the lowest a_i move by a few per cent of the span per iteration; a guess too low costs a second
+    // pass over the sites, one too high longer lists)
+    cut = need + 0.25f * (need - amin);
+    set_buckets(amin, amax, cut, lo, inv);
+    ranged = true;
     // ---------------------------------------------------------------- merge (Alg. 2)
     unsigned long long* sk = reinterpret_cast<unsigned long long*>(scr);
     const int PCs = search_pcs(cap, P.merge_cand);
     unsigned long long* se = sk + PCs;
     // after the keys: mem [256] candidates by bucket, rank [256], bucket sizes [kMB], every
-    // warp's bucket starts [kSW][kMB + 4]; keep_lowest's histogram overlaps the starts only
+    // warp's bucket starts [NW][kMB + 4]; keep_lowest's histogram overlaps the starts only
     int* mem = reinterpret_cast<int*>(se + PCs);
     int* bcnt = mem + 512;
     int* rhist = bcnt + 2 * kMB;                     // [256] (keep_lowest, before the buckets)
     __syncthreads();   // every survivor written; the scan's scratch is free
-    for (int x = tid; x < kMB; x += kSNT) bcnt[x] = 0;
     const int S = s_ns;
     if (S > cap) {   // block-uniform: the buffer held only the first cap survivors
       if (tid == 0) atomicOr(P.status, kStatCapacity);
@@ -703,12 +785,12 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
       continue;
     }
     nsurv += (unsigned long long)S;
-    if constexpr (F64) {   // the survivors' sites (the FP32 fields have been read: their place is free)
-      unsigned* mark = reinterpret_cast<unsigned*>(as);                  // [32]
+    if constexpr (F64) {   // the survivors' sites (the scan's lists have been read: their place is free)
+      unsigned* mark = reinterpret_cast<unsigned*>(scr);                 // [32]
       unsigned short* list = reinterpret_cast<unsigned short*>(mark + 32);   // [NP]
       if (tid < 32) mark[tid] = 0u;
       __syncthreads();
-      for (int e = tid; e < S; e += kSNT) {
+      for (int e = tid; e < S; e += NT) {
         int i, j;
         surv_sites((e < kSSV) ? ssv[e] : surv[e], i, j);
         atomicOr(&mark[i >> 5], 1u << (i & 31));
@@ -724,15 +806,16 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
         if (lane >= o) inc += y;
       }
       const int m = __shfl_sync(0xffffffffu, inc, 31);
-      for (int w = warp; w < 32; w += kSW) {
+      for (int w = warp; w < 32; w += NW) {
         const unsigned x = __shfl_sync(0xffffffffu, mk, w);
         const int at = __shfl_sync(0xffffffffu, inc, w) - __popc(x);
         if ((x >> lane) & 1u) list[at + __popc(x & ((1u << lane) - 1u))] = (unsigned short)(w * 32 + lane);
       }
       __syncthreads();
-      fields_f64(P, d, pb, aq_of(P, b, t), list, m, ad);
+      fields_f64(P, d, pb, aqb, list, m, ad);
       __syncthreads();
     }
+    for (int x = tid; x < kMB; x += NT) bcnt[x] = 0;   // (after the sites' list: the places overlap)
     const bool big = S > PCs;
     if (big) {
       const long long stride = next_pow2(max(cap, 256));
@@ -741,9 +824,8 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
     }
     const long long Tq = (!F64 && cnt == K1) ? (long long)(okey[K1 - 1] ^ (1ull << 63)) : LLONG_MAX;
     const double T = (F64 && cnt == K1) ? dkey_inv(okey[K1 - 1]) : INFINITY;
-    const long long* aqb = F64 ? nullptr : aq_of(P, b, t);
     unsigned long long kmn = ~0ull, kmx = 0;
-    for (int u0 = 0; u0 < S; u0 += kSNT) {
+    for (int u0 = 0; u0 < S; u0 += NT) {
       const int e = u0 + tid;
       bool keep = false;
       unsigned long long kk = 0, ent = 0;
@@ -791,20 +873,22 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
         }
       }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      kmn = min(kmn, __shfl_xor_sync(0xffffffffu, kmn, o));
-      kmx = max(kmx, __shfl_xor_sync(0xffffffffu, kmx, o));
-    }
-    if (lane == 0 && kmn <= kmx) {
-      atomicMin(&s_kmin, kmn);
-      atomicMax(&s_kmax, kmx);
+    kmn = warp_min64(kmn);
+    kmx = warp_max64(kmx);
+    if (lane == 0) {
+      s_kmm[warp] = kmn;
+      s_kmm[NW + warp] = kmx;
     }
     __syncthreads();
     int nv = s_nv;
     // more kept candidates than the buckets take at once: only the K+1 lowest can enter the list
     if (nv > 256 && nv > K1) nv = keep_lowest(sk, se, nv, K1, rhist, s_w);
-    const unsigned long long kmin = s_kmin, kmax = s_kmax;
+    unsigned long long kmin = s_kmm[0], kmax = s_kmm[NW];
+#pragma unroll
+    for (int w = 1; w < NW; ++w) {
+      kmin = min(kmin, s_kmm[w]);
+      kmax = max(kmax, s_kmm[NW + w]);
+    }
     // the new candidates' order (E, c) as one 64-bit value, (E - Emin) << cb | c, where the keys'
     // span leaves room for c (always but for extreme ranges); equal energies are ordered by c
     const uint32_t n_cand = (uint32_t)n + (uint32_t)((long long)n * (n - 1) / 2);
@@ -816,14 +900,16 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
     if (bucketed) {
       // without sorting them: the order values packed in place, a counting sort by their top
       // bits into kMB buckets, then a count within the bucket (the values are distinct)
-      int wb0 = 0, wb1 = 0;
-      if (tid < nv) {
-        sk[tid] = ((sk[tid] - kmin) << cb) | (uint32_t)se[tid];
-        wb0 = atomicAdd(&bcnt[(int)(sk[tid] >> sh)], 1);
-      }
-      if (tid + kSNT < nv) {
-        sk[tid + kSNT] = ((sk[tid + kSNT] - kmin) << cb) | (uint32_t)se[tid + kSNT];
-        wb1 = atomicAdd(&bcnt[(int)(sk[tid + kSNT] >> sh)], 1);
+      constexpr int V = NT >= 256 ? 1 : 256 / NT;
+      int wb[V];
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        const int p = tid + v * NT;
+        wb[v] = 0;
+        if (p < nv) {
+          sk[p] = ((sk[p] - kmin) << cb) | (uint32_t)se[p];
+          wb[v] = atomicAdd(&bcnt[(int)(sk[p] >> sh)], 1);
+        }
       }
       __syncthreads();
       {   // every warp forms the bucket starts itself (no barrier)
@@ -848,10 +934,13 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
         if (lane == 31) bst[kMB] = acc;
         __syncwarp();
       }
-      if (tid < nv) mem[bst[(int)(sk[tid] >> sh)] + wb0] = tid;
-      if (tid + kSNT < nv) mem[bst[(int)(sk[tid + kSNT] >> sh)] + wb1] = tid + kSNT;
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        const int p = tid + v * NT;
+        if (p < nv) mem[bst[(int)(sk[p] >> sh)] + wb[v]] = p;
+      }
       __syncthreads();
-      for (int p = tid; p < nv; p += kSNT) {
+      for (int p = tid; p < nv; p += NT) {
         const unsigned long long vp = sk[p];
         const int bk = (int)(vp >> sh);
         int r = bst[bk];
@@ -860,10 +949,10 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
       }
     } else {
       sort_pairs_any(sk, se, nv);   // rare: sorted in place, the place of p is p
-      for (int p = tid; p < nv; p += kSNT) rnk[p] = p;
+      for (int p = tid; p < nv; p += NT) rnk[p] = p;
     }
     // old entries: their place plus the new candidates strictly below their key
-    for (int o = tid; o < cnt; o += kSNT) {
+    for (int o = tid; o < cnt; o += NT) {
       const unsigned long long ko = okey[o];
       int lo;
       if (nv == 0 || ko <= kmin) {
@@ -893,7 +982,7 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
     }
     __syncthreads();
     const int ocut = s_ocut, n_ev = cnt - ocut;
-    for (int p = tid; p < nv; p += kSNT) {
+    for (int p = tid; p < nv; p += NT) {
       const unsigned long long kp = bucketed ? (sk[p] >> cb) + kmin : sk[p];
       int lo = 0, hi = cnt;
       while (lo < hi) {
@@ -903,32 +992,13 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
       const int rn = rnk[p], rank = rn + lo;
       if (rank >= K1) continue;
       const int slot = (rn < n_ev) ? oslot[ocut + rn] : cnt + (rn - n_ev);
-      uint32_t c;
       int i, j;
-      surv_decode(se[p], c, i, j);
-      uint64_t* dst = P.lst_bits + (base + slot) * Wm;
-      {   // the parent's words, two per store when the rows are 16-byte aligned (fewer store
-          // instructions of scattered rows than one word each), then the words of the flipped
-          // sites stored again with their bits flipped (same thread and address: the later wins)
-        int x = 0;
-        if ((Wm & 1) == 0)
-          for (; x + 1 < W; x += 2)
-            *reinterpret_cast<ulonglong2*>(dst + x) = *reinterpret_cast<const ulonglong2*>(pb + x);
-        for (; x < W; ++x) dst[x] = pb[x];
-        const int wi = i >> 6;
-        uint64_t vi = pb[wi] ^ (1ull << (i & 63));
-        if (j >= 0 && (j >> 6) == wi) vi ^= 1ull << (j & 63);
-        dst[wi] = vi;
-        if (j >= 0 && (j >> 6) != wi) dst[j >> 6] = pb[j >> 6] ^ (1ull << (j & 63));
-      }
-      const uint64_t stamp = ((uint64_t)t << 32) | c;
-      if (F64) P.lst_E[base + slot] = dkey_inv(kp);
-      else P.lst_q[base + slot] = (long long)(kp ^ (1ull << 63));
-      P.lst_stamp[base + slot] = stamp;
-      ostamp[slot] = stamp;
-      P.lst_hash[base + slot] = ph ^ P.zob[i] ^ ((j >= 0) ? P.zob[j] : 0ull);
-      P.lst_used[base + slot] = 0;
+      surv_sites(se[p], i, j);
+      // the state is kept as (iteration, flips): its words are written at the end of the launch
+      oflip[slot] = (uint32_t)i | ((uint32_t)j << 16);
+      ohash[slot] = ph ^ P.zob[i] ^ ((j >= 0) ? P.zob[j] : 0ull);
       oused[slot] = 0;
+      ogen[slot] = (uint8_t)(iter + 1);
       oslotN[rank] = slot;
       okeyN[rank] = kp;
     }
@@ -939,13 +1009,28 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
   // ------------------------------------------------------------------ write back
   const unsigned long long* okey = cur ? okeyB : okeyA;
   const int* oslot = cur ? oslotB : oslotA;
-  for (int r = tid; r < cnt; r += kSNT) {
+  for (int r = tid; r < cnt; r += NT) {
+    const int slot = oslot[r];
     P.lst_key[base + r] = okey[r];
-    P.lst_ord[base + r] = oslot[r];
+    P.lst_ord[base + r] = slot;
+    P.lst_used[base + slot] = oused[slot];
+    if (ogen[slot]) {
+      if (F64) P.lst_E[base + slot] = dkey_inv(okey[r]);
+      else P.lst_q[base + slot] = (long long)(okey[r] ^ (1ull << 63));
+      const int i = (int)(oflip[slot] & 0xffffu), j = (int)(short)(oflip[slot] >> 16);
+      P.lst_stamp[base + slot] = ((uint64_t)(t_first + ogen[slot] - 1) << 32) | (j < 0 ? (uint32_t)i : pair_index(n, i, j));
+      P.lst_hash[base + slot] = ohash[slot];
+    }
   }
-  if (act0) {   // the last parent (what the per-kernel form leaves in these fields)
-    for (int w = tid; w < W; w += kSNT) P.par_bits[(long long)b * Wm + w] = pb[w];
+  for (int s = warp; s < cnt; s += NW) {   // (the slots in use are 0 .. cnt - 1)
+    const int g = ogen[s];
+    if (!g) continue;
+    const int i = (int)(oflip[s] & 0xffffu), j = (int)(short)(oflip[s] >> 16);
+    for (int w = lane; w < W; w += 32)
+      P.lst_bits[(base + s) * Wm + w] = pw[(long long)(g - 1) * Wm + w] ^ flip_mask(w, i, j);
   }
+  if (act0)   // the last parent (what the per-kernel form leaves in these fields)
+    for (int w = tid; w < W; w += NT) P.par_bits[(long long)b * Wm + w] = pb[w];
   if (tid == 0) {
     P.lst_count[b] = cnt;
     P.iter_t[b] = t_first + n_iters - 1;
@@ -966,27 +1051,27 @@ __global__ void __launch_bounds__(kSNT, kSMinBlocks) k_search(DevPtrs P, int n_i
   }
 }
 
-template <int FL, bool F64>
-static cudaError_t launch_search_as(const DevPtrs& P, int n_iters, cudaStream_t s) {
-  const size_t sm = (size_t)search_layout(P.NP, P.Wmax, P.K1, P.cap, P.merge_cand, F64).total;
+template <int FL, bool F64, int NT>
+static cudaError_t launch_search_as(const DevPtrs& P, int n_iters, int ext, cudaStream_t s) {
+  const size_t sm = (size_t)search_layout(P.NP, P.Wmax, P.K1, P.cap, P.merge_cand, NT / 32, F64).total;
   static size_t attr = 0;
   if (attr < sm) {
-    const cudaError_t e = cudaFuncSetAttribute(k_search<FL, F64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const cudaError_t e = cudaFuncSetAttribute(k_search<FL, F64, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     attr = sm;
   }
-  k_search<FL, F64><<<P.B, kSNT, sm, s>>>(P, n_iters);
+  k_search<FL, F64, NT><<<P.B, NT, sm, s>>>(P, n_iters, ext);
   return cudaGetLastError();
 }
 
-cudaError_t launch_search(const DevPtrs& P, int n_iters, cudaStream_t s) {
+cudaError_t launch_search(const DevPtrs& P, int n_iters, int ext, cudaStream_t s) {
   if (n_iters <= 0 || P.B == 0) return cudaSuccess;
   const bool ex = P.flips == QIS_FLIPS_EXCHANGE;
   if (P.mode == QIS_FP64)
-    return ex ? launch_search_as<QIS_FLIPS_EXCHANGE, true>(P, n_iters, s)
-              : launch_search_as<QIS_FLIPS_SINGLE_PAIR, true>(P, n_iters, s);
-  return ex ? launch_search_as<QIS_FLIPS_EXCHANGE, false>(P, n_iters, s)
-            : launch_search_as<QIS_FLIPS_SINGLE_PAIR, false>(P, n_iters, s);
+    return ex ? launch_search_as<QIS_FLIPS_EXCHANGE, true, 128>(P, n_iters, ext, s)
+              : launch_search_as<QIS_FLIPS_SINGLE_PAIR, true, 128>(P, n_iters, ext, s);
+  return ex ? launch_search_as<QIS_FLIPS_EXCHANGE, false, 128>(P, n_iters, ext, s)
+            : launch_search_as<QIS_FLIPS_SINGLE_PAIR, false, 128>(P, n_iters, ext, s);
 }
 
 }  // namespace qis
