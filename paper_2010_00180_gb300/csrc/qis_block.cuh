@@ -109,11 +109,11 @@ static __device__ __forceinline__ bool near_sites(uint64_t x, const GfTables* __
   return s1 != 0 && (zob[0] ^ zob[s1]) == x;
 }
 
-// Minimum / maximum of a 64-bit key over the warp (every lane gets it), in 32-bit reductions.
+// Minimum / maximum of a 64-bit key over the warp (every lane gets it).
 static __device__ __forceinline__ unsigned long long warp_min64(unsigned long long x) {
-  const unsigned h = __reduce_min_sync(0xffffffffu, (unsigned)(x >> 32));
-  const unsigned l = __reduce_min_sync(0xffffffffu, (unsigned)(x >> 32) == h ? (unsigned)x : 0xffffffffu);
-  return (unsigned long long)h << 32 | l;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x = min(x, __shfl_xor_sync(0xffffffffu, x, o));
+  return x;
 }
 static __device__ __forceinline__ unsigned long long warp_max64(unsigned long long x) { return ~warp_min64(~x); }
 

@@ -202,7 +202,11 @@ __device__ inline void decode_candidate(int n, uint32_t c, int& i, int& j) {
   j = r - (ii * n - ii * (ii + 1) / 2) + ii + 1;
 }
 
-__device__ inline int sigma_of(const uint64_t* bits, int i) { return (int)((bits[i >> 6] >> (i & 63)) & 1ull); }
+// (a select of the half and a 32-bit shift: no 64-bit variable shift)
+__device__ inline int sigma_of(const uint64_t* bits, int i) {
+  const uint64_t w = bits[i >> 6];
+  return (int)((((i & 32) ? (uint32_t)(w >> 32) : (uint32_t)w) >> (i & 31)) & 1u);
+}
 
 // SplitMix64 (Steele, Lea and Flood 2014): value number c of the stream started at key.
 __host__ __device__ inline uint64_t splitmix64(uint64_t key, uint64_t c) {

@@ -291,6 +291,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
   long long Epq = F64 ? 0 : P.par_q[b];
   uint64_t ph = P.par_hash[b];
   uint64_t* pw = P.pw + (long long)b * P.pw_n * Wm;   // words of the parent of iteration iter: pw + iter Wm
+#pragma unroll 1
   for (int r = tid; r < K1; r += NT) {
     okeyA[r] = P.lst_key[base + r];
     oslotA[r] = P.lst_ord[base + r];
@@ -298,6 +299,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
     oused[r] = P.lst_used[base + r];
     ogen[r] = 0;   // in lst_bits (else 1 + the iteration of this launch that generated it)
   }
+#pragma unroll 1
   for (int w = tid; w < W; w += NT) {
     const uint64_t x = P.par_bits[(long long)b * Wm + w];
     pb[w] = x;
@@ -351,8 +353,11 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
       s_cn = 0;
       s_ocut = cnt;
     }
+#pragma unroll 1
     for (int x = tid; x < HT; x += NT) htab[x] = kNoCand;
+#pragma unroll 1
     for (int x = tid; x < kSparseNB; x += NT) bcur[x] = 0;
+#pragma unroll 1
     for (int x = tid; x < 512; x += NT) vhist[x] = 0;
     float mn = INFINITY, mx = -INFINITY;   // this thread's range of a_i
     const long long* aqb = aq_of(P, b, t);
@@ -393,6 +398,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
       pi0 = i;
       pj0 = j;
       // the parent's words: its own, or its generator's with the flipped bits
+#pragma unroll 1
       for (int w = tid; w < W; w += NT) {
         const uint64_t x = gen ? pw[(long long)(gen - 1) * Wm + w] ^ flip_mask(w, i, j) : P.lst_bits[(base + pslot) * Wm + w];
         pb[w] = x;
@@ -404,6 +410,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
       if (!EX) npair += (unsigned long long)n * (n - 1) / 2;
       if (EX) {
         int down = 0;
+#pragma unroll 1
         for (int w = 0; w < W; ++w) down += __popcll(pb[w]);
         npair += (unsigned long long)down * (unsigned long long)(n - down);
       }
@@ -474,6 +481,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
     // flips it would be (near_sites), and only then are the words compared: the state is its
     // generator's words with two flips at most, so its difference from the parent has to be exactly
     // the bits that the four flips leave.
+#pragma unroll 1
     for (int r = tid; r < cnt; r += NT) {
       const int g = ogen[r];
       int i, j;
@@ -499,6 +507,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
       const uint32_t c = j < 0 ? (uint32_t)i : pair_index(n, i, j);
       atomicAdd(&s_near, 1);
       uint32_t pos = chash(c) & (HT - 1);
+#pragma unroll 1
       while (atomicCAS(&htab[pos], kNoCand, c) != kNoCand) pos = (pos + 1) & (HT - 1);
     }
 #pragma unroll
@@ -524,6 +533,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
       cn = s_cn;
       if (warp == 0) bucket_starts(bcur, bs);
       __syncthreads();
+#pragma unroll 1
       for (int e = tid; e < cn; e += NT) {
         const float v = LS.ua[e];
         const unsigned short s = LS.us[e];
@@ -551,7 +561,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
       if (EX) {
         const int nd = n - nu;
         int m0 = max(1, (int)sqrtf((float)want));
+#pragma unroll 1
         while (m0 * m0 < want) ++m0;
+#pragma unroll 1
         while (m0 > 1 && (m0 - 1) * (m0 - 1) >= want) --m0;
         int mu = min(nu, m0);
         int md = min(nd, (want + mu - 1) / mu);
@@ -565,7 +577,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
         t1 = md;   // up spins
       } else {
         int m = max(1, (int)((sqrtf(8.f * (float)want + 1.f) - 1.f) * 0.5f));
+#pragma unroll 1
         while (m * (m + 1) / 2 < want) ++m;
+#pragma unroll 1
         while (m > 1 && (m - 1) * m / 2 >= want) --m;
         t0 = min(min(m, n), kSubSites);
       }
@@ -620,10 +634,13 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
         };
         if (!EX) {
           // the sites' own flips, then their pairs row by row: warp w takes the rows x = w, w + NW, ..
+#pragma unroll 1
           for (int q = tid; q < m0; q += NT) put_value(oa[q]);
+#pragma unroll 1
           for (int x = warp; x < m0; x += NW)
             for (int y = x + 1 + lane; y < m0; y += 32) pair_value(x, y);
         } else {
+#pragma unroll 1
           for (int x = warp; x < m0; x += NW)
             for (int y = lane; y < m1; y += 32) pair_value(s_ex[x], s_ex[t0 + y]);
         }
@@ -633,6 +650,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
         int bsel, within;
         find_bin(vhist, k - 1, bsel, within);
         unsigned mk = 0u;
+#pragma unroll 1
         for (int x = lane; x <= bsel; x += 32) mk = max(mk, vmax[x]);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) mk = max(mk, __shfl_xor_sync(0xffffffffu, mk, o));
@@ -676,6 +694,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
       const int rcap = P.NP * 3;
       const int per = (cn + NT - 1) / NT, q0 = min(cn, tid * per), q1 = min(cn, q0 + per);
       int sum = 0;
+#pragma unroll 1
       for (int q = q0; q < q1; ++q) {
         const float ai = oa[q], r = orm[q];
         if (!EX && ai <= thr) put_surv(atomicAdd(&s_ns, 1), surv_entry(os[q] & 0x7fff, -1));
@@ -703,9 +722,11 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
         if (w < warp) acc += x;
         tot += x;
       }
+#pragma unroll 1
       for (int q = q0; q < q1; ++q) {
         const int x = pc[q];
         pc[q] = acc;
+#pragma unroll 1
         for (int e = acc, e1 = min(acc + x, rcap); e < e1; ++e) rowof[e] = (unsigned short)q;
         acc += x;
       }
@@ -724,6 +745,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
             q = rowof[e];
           } else {
             int hi = cn;
+#pragma unroll 1
             while (hi - q > 1) {
               const int mid = (q + hi) >> 1;
               if (pc[mid] <= e) q = mid; else hi = mid;
@@ -815,6 +837,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
       fields_f64(P, d, pb, aqb, list, m, ad);
       __syncthreads();
     }
+#pragma unroll 1
     for (int x = tid; x < kMB; x += NT) bcnt[x] = 0;   // (after the sites' list: the places overlap)
     const bool big = S > PCs;
     if (big) {
@@ -852,6 +875,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
         }
         if (keep) {
           const uint32_t c = (uint32_t)ent;
+#pragma unroll 1
           for (uint32_t pos = chash(c) & (HT - 1); htab[pos] != kNoCand; pos = (pos + 1) & (HT - 1))
             if (htab[pos] == c) {
               keep = false;   // a kept state (the binary search of Alg. 2)
@@ -940,18 +964,20 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
         if (p < nv) mem[bst[(int)(sk[p] >> sh)] + wb[v]] = p;
       }
       __syncthreads();
+#pragma unroll 1
       for (int p = tid; p < nv; p += NT) {
         const unsigned long long vp = sk[p];
         const int bk = (int)(vp >> sh);
         int r = bst[bk];
+#pragma unroll 1
         for (int q = bst[bk], q1 = bst[bk + 1]; q < q1; ++q) r += (sk[mem[q]] < vp) ? 1 : 0;
         rnk[p] = r;
       }
     } else {
-      sort_pairs_any(sk, se, nv);   // rare: sorted in place, the place of p is p
-      for (int p = tid; p < nv; p += NT) rnk[p] = p;
+      sort_pairs_any(sk, se, nv);   // rare: sorted in place, the place of p is p (nv may exceed rnk's)
     }
     // old entries: their place plus the new candidates strictly below their key
+#pragma unroll 1
     for (int o = tid; o < cnt; o += NT) {
       const unsigned long long ko = okey[o];
       int lo;
@@ -963,10 +989,12 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
         const unsigned long long vo = (ko - kmin) << cb;   // below every new value of energy ko
         const int bk = (int)(vo >> sh);
         lo = bst[bk];
+#pragma unroll 1
         for (int q = bst[bk], q1 = bst[bk + 1]; q < q1; ++q) lo += (sk[mem[q]] < vo) ? 1 : 0;
       } else {
         lo = 0;
         int hi = nv;
+#pragma unroll 1
         while (lo < hi) {
           const int mid = (lo + hi) >> 1;
           if (sk[mid] < ko) lo = mid + 1; else hi = mid;
@@ -982,14 +1010,16 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
     }
     __syncthreads();
     const int ocut = s_ocut, n_ev = cnt - ocut;
+#pragma unroll 1
     for (int p = tid; p < nv; p += NT) {
       const unsigned long long kp = bucketed ? (sk[p] >> cb) + kmin : sk[p];
       int lo = 0, hi = cnt;
+#pragma unroll 1
       while (lo < hi) {
         const int mid = (lo + hi) >> 1;
         if (okey[mid] <= kp) lo = mid + 1; else hi = mid;
       }
-      const int rn = rnk[p], rank = rn + lo;
+      const int rn = bucketed ? rnk[p] : p, rank = rn + lo;
       if (rank >= K1) continue;
       const int slot = (rn < n_ev) ? oslot[ocut + rn] : cnt + (rn - n_ev);
       int i, j;
@@ -1009,6 +1039,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
   // ------------------------------------------------------------------ write back
   const unsigned long long* okey = cur ? okeyB : okeyA;
   const int* oslot = cur ? oslotB : oslotA;
+#pragma unroll 1
   for (int r = tid; r < cnt; r += NT) {
     const int slot = oslot[r];
     P.lst_key[base + r] = okey[r];
@@ -1022,10 +1053,12 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
       P.lst_hash[base + slot] = ohash[slot];
     }
   }
+#pragma unroll 1
   for (int s = warp; s < cnt; s += NW) {   // (the slots in use are 0 .. cnt - 1)
     const int g = ogen[s];
     if (!g) continue;
     const int i = (int)(oflip[s] & 0xffffu), j = (int)(short)(oflip[s] >> 16);
+#pragma unroll 1
     for (int w = lane; w < W; w += 32)
       P.lst_bits[(base + s) * Wm + w] = pw[(long long)(g - 1) * Wm + w] ^ flip_mask(w, i, j);
   }
