@@ -253,7 +253,9 @@ static bool fused_search(const qis_ctx* ctx) {
 int launch_iterations_fused(qis_ctx* ctx, int n, cudaStream_t s) {
   ctx->P.dense_ctl = 0;
   const DevPtrs& P = ctx->P;
-  if (ctx->mode == QIS_FP64) {   // picks and computes the fields of every iteration itself
+  // the FP64 mode, and small instances (whose fields from scratch cost less than the launches below),
+  // pick and compute the fields of every iteration in the search kernel itself
+  if (ctx->mode == QIS_FP64 || (ctx->NP == kPad && ctx->cfg.flips != QIS_FLIPS_SINGLE)) {
     CK(prof_begin(ctx, 5));
     for (int i = 0; i < n; i += P.pw_n) LAUNCH(launch_search(P, std::min(n - i, P.pw_n), 0, s));
     CK(prof_end(ctx, 5));

@@ -15,7 +15,8 @@
 //           the flips of its own generation and from the hashes of the others (near_sites)
 //   bound   filter threshold: the last kept energy and an order-statistic bound from the flips of
 //           the lowest listed sites; a list that does not reach what the threshold needs is
-//           taken again
+//           taken again. In a kept list that has settled the last kept energy alone leaves few
+//           enough, and the order-statistic bound (a fifth of such an iteration) is not formed
 //   scan    pair flips dE_ij = a_i + a_j + 4 s_i s_j J_ij decided by the output-sensitive scan: a
 //           live row's partners are the sites after it in the order, up to the bucket of its bound
 //   merge   exact integer keys of the survivors, duplicates dropped, the new states ranked by
@@ -27,7 +28,9 @@
 // the list once, at the end of the launch. The aq ring and the survivors past 512 are in global
 // memory (written and read by this block only, within the L2 cache).
 // Split modes: the first iteration's parent is picked, and its fields computed (update, or the
-// tensor-core GEMM for a parent without a stored generator), by the kernels launched before this one.
+// tensor-core GEMM for a parent without a stored generator), by the kernels launched before this one;
+// not for instances of at most 128 spins, whose row sums here cost less than those launches (4 searches
+// of n = 16, 8 iterations: 82 us with them, 70 without).
 // FP64 mode: the same filter, the survivors' energies in the defining FP64 arithmetic.
 // Every decision is that of the per-kernel form (k_bound, k_scan_sparse, k_merge), so the kept
 // lists are identical bit for bit.
@@ -37,7 +40,9 @@
 // searches of n = 600, 120 iterations: 31.9 ms with passes over all sites for each of histogram,
 // selection, rows, bucket counts and order, with the near states found by comparing words, and with
 // every new state's words written in every iteration; 26.6 ms with the listed sites, hashes and
-// words at the end; 21.7 ms with the own generation's near states from their flips alone.
+// words at the end; 21.6 ms with the own generation's near states from their flips alone (3840 searches
+// of n = 64: 6.2 ms with the order-statistic bound in every iteration, 5.1 without it in settled lists;
+// of n = 200 8.2 and 7.9).
 #include "qis_block.cuh"
 
 namespace qis {
@@ -88,6 +93,7 @@ __host__ __device__ inline SearchLayout search_layout(int NP, int Wmax, int K1, 
   L.pc = take(NP * 4 > 2048 ? NP * 4 : 2048);
   L.bs = take((kSparseNB + 1) * 4);
   L.bcur = take(kSparseNB * 4);
+  // (keep_lowest's 256 bins lie 2 kMB past the bucket sizes: within the starts of three or more warps)
   const int merge = search_pcs(cap, merge_cand) * 16 + (512 + kMB + warps * (kMB + 4)) * 4;
   L.total = align_up(o - L.scratch > merge ? o : L.scratch + merge, 16);
   return L;
@@ -117,11 +123,42 @@ static __device__ __noinline__ void fields_full(const DevPtrs& P, const InstDesc
   }
 }
 
+// The k-th lowest dE of the m survivors held (radix select, the values formed anew in each pass). More
+// survivors than the buffer holds are rare: out of line.
+static __device__ __noinline__ float kth_survivor(const unsigned long long* ssv, const unsigned long long* surv, int m, int k,
+                                                  const long long* ax, float scale_q, const float* J4, int n_pad,
+                                                  const uint64_t* pb, int* hist) {
+  unsigned prefix = 0u;
+  int rank = k - 1;
+  for (int shift = 24; shift >= 0; shift -= 8) {
+    for (int x = threadIdx.x; x < 256; x += blockDim.x) hist[x] = 0;
+    __syncthreads();
+    for (int e = threadIdx.x; e < m; e += blockDim.x) {
+      int i, j;
+      surv_sites((e < kSSV) ? ssv[e] : surv[e], i, j);
+      float v = __ll2float_rn(ax[i]) * scale_q;
+      if (j >= 0) {
+        const float j4 = J4[(long long)i * n_pad + j];
+        v += fmaf(sigma_of(pb, i) != sigma_of(pb, j) ? -1.f : 1.f, j4, __ll2float_rn(ax[j]) * scale_q);
+      }
+      const unsigned key = fkey(v);
+      if (shift == 24 || key >> (shift + 8) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1);
+    }
+    __syncthreads();
+    int bin;
+    find_bin(hist, rank, bin, rank);   // every warp alike
+    prefix = (prefix << 8) | (unsigned)bin;
+    __syncthreads();
+  }
+  return fkey_inv(prefix);
+}
+
 // FP64 mode: a_i = -2 s_i f_i with f_i = (sum_{j != i} s_j J_ij, j ascending from +0.0) + h_i (the
 // order of k_fields_fp64) of the m sites of `list`, ascending. A chain of n additions per site, on
 // two FP64 lanes per SM, is what bounds the FP64 search, so only the sites of the survivors pay it
 // (the filter works on the fixed-point fields): 120 iterations of 3840 searches of n = 100 take
-// 15.3 ms, 17.2 with the chains of every site, and 86 ms in the per-kernel form (every pair in FP64). An instance exactly on its grid needs no
+// 9.7 ms, 12.4 with the sites of the duplicates too, and 86 ms in the per-kernel form (every pair in
+// FP64). An instance exactly on its grid needs no
 // chain: every partial sum is exact, so the fixed-point field is the same double.
 static __device__ __forceinline__ void fields_f64(const DevPtrs& P, const InstDesc& d, const uint64_t* pb,
                                                   const long long* aq, const unsigned short* list, int m, double* ad) {
@@ -275,8 +312,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
   int* vhist = pc;                                              // [256] the bound's values per bin
   unsigned* vmax = reinterpret_cast<unsigned*>(vhist + 256);    // [256] and their maxima
 
-  __shared__ int s_sel, s_near, s_ns, s_nv, s_ocut, s_cn, s_m0, s_m1;
-  __shared__ float wf[2 * NW];
+  __shared__ int s_sel, s_near, s_ns, s_nv, s_ocut, s_cn, s_m0, s_m1, s_set, s_nset;
+  __shared__ float wf[2 * NW], s_u, s_thr[2];
   __shared__ int s_w[33];
   __shared__ unsigned long long s_kmm[2 * NW];
   __shared__ unsigned short s_ex[kSubSites];   // exchanges: the bound's sites of each spin class (positions)
@@ -306,8 +343,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
     if (ext) pw[w] = x;
   }
   __syncthreads();
-  if (!F64 && act0 && ext && P.e0_pend[b]) {   // block-uniform: the list is [psi0] and psi0 is the parent
-    Epq = initial_energy(P, d, pb, aq_of(P, b, t_first), reinterpret_cast<long long*>(scr));
+  // E(psi0) is still to be formed from the exact fields of its first iteration (block-uniform: the
+  // list is [psi0] and psi0 is that iteration's parent)
+  auto form_e0 = [&]() {
+    Epq = initial_energy(P, d, pb, aq_of(P, b, t_first), reinterpret_cast<long long*>(s_kmm));
     if (tid == 0) {
       const int s0 = oslotA[0];
       const double E0 = ldexp((double)Epq, -d.q);
@@ -319,11 +358,12 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
       P.e0_pend[b] = 0;
     }
     __syncthreads();
-  }
+  };
 
-  int act = act0, t = t_first - 1, cur = 0, nprod = 0;
+  if (tid == 0) s_u = INFINITY;
+  int act = act0, cur = 0, nprod = 0;
   int pgen = 0, pi0 = -1, pj0 = -1;   // the parent's generation in this launch and its flips
-  unsigned long long npair = 0, nev = 0, nsurv = 0;
+  unsigned npair = 0, nev = 0, nsurv = 0;   // of this launch (at most 128 iterations: 32 bits); npair: exchanges
   const float scale_q = (float)d.inv_scale;
   const long long* Jq = P.Jq + d.off_mat;
   const float* J4 = P.J4 + d.off_mat;
@@ -343,10 +383,11 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
     unsigned long long* okeyN = cur ? okeyA : okeyB;
     int* oslot = cur ? oslotB : oslotA;
     int* oslotN = cur ? oslotA : oslotB;
-    t += 1;
     if (!act) continue;
+    const int t = t_first + iter;
     // this iteration's counters (the last one's reads are behind its last barrier)
     if (tid == 0) {
+      s_set = iter > 0 && s_nset && s_ns <= K1;   // (s_set, s_nset: see the bound)
       s_near = 0;
       s_ns = 0;
       s_nv = 0;
@@ -406,14 +447,6 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
       }
       __syncthreads();   // the parent's words; every thread has read s_sel and the used flags
       if (tid == 0) oused[pslot] = 1;
-      ++nprod;
-      if (!EX) npair += (unsigned long long)n * (n - 1) / 2;
-      if (EX) {
-        int down = 0;
-#pragma unroll 1
-        for (int w = 0; w < W; ++w) down += __popcll(pb[w]);
-        npair += (unsigned long long)down * (unsigned long long)(n - down);
-      }
       // ------------------------------------------------------------ fields
       // x = the parent, a candidate of iteration tg's parent g
       long long* ax = aq_of(P, b, t);
@@ -474,6 +507,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
     } else {
       __syncthreads();   // the counters and tables are cleared
     }
+    if (!F64 && iter == 0 && P.e0_pend[b]) form_e0();
     // ---------------------------------------------------------------- near states
     // the kept states one or two flips from the parent: the only candidates that can be
     // duplicates, each equal to exactly one. A state of the parent's own generation differs from it
@@ -550,12 +584,13 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
     // ---------------------------------------------------------------- bound
     // an upper bound U of the k-th lowest candidate energy change: the k-th lowest among the flips of
     // the lowest listed sites (any subset of the candidates bounds it)
-    float Uf = INFINITY;
     int nu = 0;
     if (EX)
       for (int w = 0; w < W; ++w) nu += __popcll(pb[w]);
-    const long long Ccand = EX ? (long long)nu * (n - nu) : (long long)n * (n + 1) / 2;
-    if (Ccand > k && k <= kSubMax) {
+    const int Ccand = EX ? nu * (n - nu) : n * (n + 1) / 2;
+    float Uf = s_u;
+    // (s_set: in the last iteration the last kept energy was the lower threshold and left at most K+1)
+    if (Ccand > k && k <= kSubMax && !s_set) {
       const int want = min(3 * k, kSubMax);
       int t0 = 0, t1 = 0;
       if (EX) {
@@ -654,7 +689,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
         for (int x = lane; x <= bsel; x += 32) mk = max(mk, vmax[x]);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) mk = max(mk, __shfl_xor_sync(0xffffffffu, mk, o));
-        Uf = fkey_inv(mk);
+        Uf = fminf(Uf, fkey_inv(mk));
       }
     }
     float thr;
@@ -676,6 +711,11 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
                                   isinf(tt) ? 0.f : fabsf(tt));
       const float delta = __fmul_ru(big, 0x1p-21f);
       thr = fminf(__fadd_ru(tE, delta), __fadd_ru(Uf, 2.f * delta));
+      if (tid == 0) {
+        s_nset = cnt == K1 && tE <= Uf;
+        s_thr[0] = thr;
+        s_thr[1] = 4.f * delta;   // (the next pass's delta is at most twice this one's)
+      }
     }
     // every live row, single and partner has a_i <= need (rows: thr - a_i >= amin - rm_i, rm_i <= j4max;
     // partners below); the listed sites have to reach it
@@ -784,6 +824,34 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
         }
       }
     }
+    __syncthreads();   // every survivor written; the scan's scratch is free
+    const int S = s_ns;
+    // Block-uniform, rare: the k-th lowest dE of the cap survivors held bounds that of all candidates, and
+    // the iteration runs again with it, each time over fewer; an error only when more than the buffer
+    // holds are equal
+    if (S > cap) {
+      const float v = kth_survivor(ssv, surv, cap, K1 + s_near, aqb, scale_q, J4, d.n_pad, pb, reinterpret_cast<int*>(pc));
+      const bool lower = __fadd_ru(v, s_thr[1]) < s_thr[0];
+      __syncthreads();
+      if (tid == 0) {
+        if (!lower) atomicOr(P.status, kStatCapacity);
+        else if (!(ext && iter == 0)) oused[oslot[s_sel]] = 0;
+        s_u = lower ? v : INFINITY;
+      }
+      if (lower) --iter; else act = 0;
+      __syncthreads();
+      continue;
+    }
+    if (!(ext && iter == 0)) {   // (that one has been counted where it was picked)
+      ++nprod;
+      if (EX) {
+        int down = 0;
+#pragma unroll 1
+        for (int w = 0; w < W; ++w) down += __popcll(pb[w]);
+        npair += (unsigned)(down * (n - down));
+      }
+    }
+    if (tid == 0) s_u = INFINITY;
     // the next iteration's guess: this one's need and a quarter of its span as a margin (the bound and
     // the lowest a_i move by a few per cent of the span per iteration; a guess too low costs a second
     // pass over the sites, one too high longer lists)
@@ -799,14 +867,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
     int* mem = reinterpret_cast<int*>(se + PCs);
     int* bcnt = mem + 512;
     int* rhist = bcnt + 2 * kMB;                     // [256] (keep_lowest, before the buckets)
-    __syncthreads();   // every survivor written; the scan's scratch is free
-    const int S = s_ns;
-    if (S > cap) {   // block-uniform: the buffer held only the first cap survivors
-      if (tid == 0) atomicOr(P.status, kStatCapacity);
-      act = 0;
-      continue;
-    }
-    nsurv += (unsigned long long)S;
+    nsurv += (unsigned)S;
     if constexpr (F64) {   // the survivors' sites (the scan's lists have been read: their place is free)
       unsigned* mark = reinterpret_cast<unsigned*>(scr);                 // [32]
       unsigned short* list = reinterpret_cast<unsigned short*>(mark + 32);   // [NP]
@@ -815,8 +876,18 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
       for (int e = tid; e < S; e += NT) {
         int i, j;
         surv_sites((e < kSSV) ? ssv[e] : surv[e], i, j);
-        atomicOr(&mark[i >> 5], 1u << (i & 31));
-        if (j >= 0) atomicOr(&mark[j >> 5], 1u << (j & 31));
+        // (a duplicate of a kept state is dropped before its energy counts: half of the survivors of a
+        // list that has settled)
+        const uint32_t c = (j < 0) ? (uint32_t)i : pair_index(n, i, j);
+        uint32_t pos = chash(c) & (HT - 1), h = htab[pos];
+        while (h != kNoCand && h != c) {
+          pos = (pos + 1) & (HT - 1);
+          h = htab[pos];
+        }
+        if (h == kNoCand) {
+          atomicOr(&mark[i >> 5], 1u << (i & 31));
+          if (j >= 0) atomicOr(&mark[j >> 5], 1u << (j & 31));
+        }
       }
       __syncthreads();
       // every warp counts for itself; warp w lists the words w, w + 4, ..
@@ -1073,20 +1144,21 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
       else P.par_q[b] = Epq;
       P.par_hash[b] = ph;
       P.nprod[b] += nprod;
-      P.npair[b] += npair;
-      if (nsurv) atomicAdd(P.surv_tot + (b & 63), nsurv);
+      P.npair[b] += EX ? (unsigned long long)npair : (unsigned long long)nprod * (unsigned)(n * (n - 1) / 2);
+      if (nsurv) atomicAdd(P.surv_tot + (b & 63), (unsigned long long)nsurv);
     }
   }
   if (act0) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) nev += __shfl_xor_sync(0xffffffffu, nev, o);
-    if (lane == 0 && nev) atomicAdd(P.eval_cnt + (b & 63), nev);
+    if (lane == 0 && nev) atomicAdd(P.eval_cnt + (b & 63), (unsigned long long)nev);
   }
 }
 
 template <int FL, bool F64, int NT>
 static cudaError_t launch_search_as(const DevPtrs& P, int n_iters, int ext, cudaStream_t s) {
-  const size_t sm = (size_t)search_layout(P.NP, P.Wmax, P.K1, P.cap, P.merge_cand, NT / 32, F64).total;
+  const SearchLayout L = search_layout(P.NP, P.Wmax, P.K1, P.cap, P.merge_cand, NT / 32, F64);
+  const size_t sm = (size_t)L.total;
   static size_t attr = 0;
   if (attr < sm) {
     const cudaError_t e = cudaFuncSetAttribute(k_search<FL, F64, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
@@ -1097,14 +1169,24 @@ static cudaError_t launch_search_as(const DevPtrs& P, int n_iters, int ext, cuda
   return cudaGetLastError();
 }
 
+template <bool F64, int NT>
+static cudaError_t launch_search_nt(const DevPtrs& P, int n_iters, int ext, cudaStream_t s) {
+  return P.flips == QIS_FLIPS_EXCHANGE ? launch_search_as<QIS_FLIPS_EXCHANGE, F64, NT>(P, n_iters, ext, s)
+                                       : launch_search_as<QIS_FLIPS_SINGLE_PAIR, F64, NT>(P, n_iters, ext, s);
+}
+
 cudaError_t launch_search(const DevPtrs& P, int n_iters, int ext, cudaStream_t s) {
   if (n_iters <= 0 || P.B == 0) return cudaSuccess;
-  const bool ex = P.flips == QIS_FLIPS_EXCHANGE;
+  // 256 threads shorten a search's chain of phases, 128 leave fewer of them waiting in each: 256 while
+  // all blocks are resident at once with either (four of 256 per SM). 100 iterations of n = 300, K = 100
+  // with 256 and 128 threads: 128 searches 1.22 and 1.65 ms, 512 1.63 and 1.87, 600 1.67 and 1.93, 640
+  // 2.54 and 1.94, 1024 3.05 and 2.23; FP64 n = 100: 150 searches 1.69 and 1.99, 600 2.13 and 2.17, 640
+  // 3.20 and 2.24. At n <= 128 the split modes' passes do not fill 256 threads: 600 searches of n = 60
+  // 1.02 and 0.95 ms, 4 of n = 16 72 and 70 us in 8 iterations.
+  const bool wide = P.B <= 4 * P.sms && (P.mode == QIS_FP64 || P.NP > kPad);
   if (P.mode == QIS_FP64)
-    return ex ? launch_search_as<QIS_FLIPS_EXCHANGE, true, 128>(P, n_iters, ext, s)
-              : launch_search_as<QIS_FLIPS_SINGLE_PAIR, true, 128>(P, n_iters, ext, s);
-  return ex ? launch_search_as<QIS_FLIPS_EXCHANGE, false, 128>(P, n_iters, ext, s)
-            : launch_search_as<QIS_FLIPS_SINGLE_PAIR, false, 128>(P, n_iters, ext, s);
+    return wide ? launch_search_nt<true, 256>(P, n_iters, ext, s) : launch_search_nt<true, 128>(P, n_iters, ext, s);
+  return wide ? launch_search_nt<false, 256>(P, n_iters, ext, s) : launch_search_nt<false, 128>(P, n_iters, ext, s);
 }
 
 }  // namespace qis
