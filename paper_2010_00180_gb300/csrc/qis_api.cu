@@ -555,6 +555,13 @@ int qis_create(const qis_config* cfg, qis_ctx** out) {
     ALLOC(P.mrg_ref, (size_t)ctx->max_inst * K1);
     ALLOC(P.mrg_src, (size_t)ctx->max_inst * K1);
     ALLOC(P.mrg_count, ctx->max_inst);
+    P.mrg_groups = merge_groups(ctx->R, ctx->mode);
+    if (P.mrg_groups > 1) {
+      const size_t g = (size_t)ctx->max_inst * P.mrg_groups;
+      ALLOC(P.grp_ref, g * K1);
+      ALLOC(P.grp_src, g * K1);
+      ALLOC(P.grp_count, g);
+    }
     ctx->scratch_states = 16384;   // states rescored per launch
     ALLOC(ctx->scratch_bits, (size_t)ctx->scratch_states * W);
     ALLOC(ctx->scratch_E, ctx->scratch_states);
@@ -1497,6 +1504,7 @@ int qis_topk_states(qis_ctx* ctx, int instance_id, int k, uint64_t* bits_out, do
   cudaStream_t s = ctx->stream;
   if (!ctx->merged_fresh) {
     LAUNCH(launch_final_merge(ctx->P, s));
+    ctx->launches += ctx->P.mrg_groups > 1;
     ctx->merged_fresh = true;
     ctx->counts_valid = false;
   }
@@ -1539,6 +1547,7 @@ int qis_topk_states_all(qis_ctx* ctx, int k, uint64_t* bits_out, double* E_out, 
   cudaStream_t s = ctx->stream;
   if (!ctx->merged_fresh) {
     LAUNCH(launch_final_merge(ctx->P, s));
+    ctx->launches += ctx->P.mrg_groups > 1;
     ctx->merged_fresh = true;
     ctx->counts_valid = false;
   }
@@ -1574,6 +1583,7 @@ int qis_merge(qis_ctx* ctx) {
   if (ctx->inst.empty()) return fail(ctx, QIS_ERR_STATE, "no instance");
   CK(cudaSetDevice(ctx->cfg.device));
   LAUNCH(launch_final_merge(ctx->P, ctx->stream));
+  ctx->launches += ctx->P.mrg_groups > 1;
   ctx->merged_fresh = true;
   ctx->counts_valid = false;
   return 0;

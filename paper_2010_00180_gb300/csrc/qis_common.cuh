@@ -134,6 +134,10 @@ struct DevPtrs {
   int* mrg_ref;           // [inst][K1] search*K1 + slot
   uint64_t* mrg_src;      // [inst][K1]
   int* mrg_count;         // [inst]
+  int mrg_groups;         // runs of searches that the Alg. 4 merge takes side by side (merge_groups)
+  int* grp_ref;           // [inst][mrg_groups][K1] the runs' lists, as mrg_ref, mrg_src, mrg_count
+  uint64_t* grp_src;
+  int* grp_count;         // [inst][mrg_groups]
   unsigned long long* en_acc;   // [states][2] integer sums of the energies from scratch (zero between calls)
   int* en_left;                 // [states / 128, rounded up per instance] blocks done of a state tile (zero between calls)
   int sms;                      // streaming multiprocessors of the device
@@ -385,6 +389,7 @@ cudaError_t launch_scan_pairs(const DevPtrs& P, const int4* tasks, int n_tasks, 
 cudaError_t launch_scan64(const DevPtrs& P, const int4* work, int n_work, cudaStream_t s);
 void scan_tasks_for(int inst, int n, int nc_max, int R, int RG, std::vector<int4>& out);
 cudaError_t launch_merge(const DevPtrs& P, cudaStream_t s);
+int merge_groups(int R, int mode);
 cudaError_t launch_final_merge(const DevPtrs& P, cudaStream_t s);
 size_t merge_smem(int K1, int cap, int merge_cand);
 size_t final_merge_smem(int K1);

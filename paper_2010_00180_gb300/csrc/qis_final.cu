@@ -13,6 +13,15 @@ namespace qis {
 // merged one), and its rank is its place among the kept incoming entries (a block prefix sum)
 // plus the merged entries at or below its energy; a merged entry's rank is its place plus the
 // kept incoming entries strictly below it.
+//
+// A round costs about 2.7 us of latency (five barriers, binary searches), so R lists in a row take R - 1
+// of them on one block. Where energies are exact the result does not depend on how the lists are
+// grouped: it is the K+1 lowest distinct states by (E, search, position), and a state dropped from a
+// full list, or again as a later copy, has K+1 states before it. Then merge_groups(R) blocks per
+// instance merge a run of consecutive searches each, and a second launch merges their lists (120
+// instances of 64 searches, K+1 = 121: 174 us in a row, 62 us in 8 runs). In the
+// FP64 mode copies of a state can differ in the last bits and the order of merging decides which one
+// stays: one run there.
 struct MergeSet {
   double* E;                // energy
   unsigned long long* S;    // source: search << 32 | position in its list
@@ -58,8 +67,14 @@ __device__ inline int bound_of(const double* v, int cnt, double x, bool strict) 
 
 constexpr int kSetBytes = 8 + 8 + 8 + 4;
 
-__global__ void __launch_bounds__(256) k_final_merge(DevPtrs P) {
+// part: 0 every search's list into the result; 1 the run blockIdx.y of the searches into P.grp_*; 2 the
+// runs' lists into the result.
+__global__ void __launch_bounds__(256) k_final_merge(DevPtrs P, int part) {
   const int inst = blockIdx.x;
+  const int G = P.mrg_groups;
+  const int lists = (part == 2) ? G : P.R;
+  const int l0 = (part == 1) ? (int)((long long)lists * blockIdx.y / G) : 0;
+  const int l1 = (part == 1) ? (int)((long long)lists * (blockIdx.y + 1) / G) : lists;
   const InstDesc d = P.inst[inst];
   const int K1 = P.K1, W = d.W;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -70,21 +85,22 @@ __global__ void __launch_bounds__(256) k_final_merge(DevPtrs P) {
   int* lev = cum + K1 + 1;                                         // [K1] merged entries <= E_p, or -1
   __shared__ int s_w[33];
   int acnt = 0;
-  for (int r = 0; r < P.R; ++r) {
+  for (int r = l0; r < l1; ++r) {
     const int b = d.first_search + r;
     const long long base = (long long)b * K1;
-    const int cnt = P.lst_count[b];
-    const MergeSet& D = (r == 0) ? A : N;
+    const long long grp = (long long)(inst * G + r) * K1;   // part 2: the run's list
+    const int cnt = (part == 2) ? P.grp_count[inst * G + r] : P.lst_count[b];
+    const MergeSet& D = (r == l0) ? A : N;
     for (int p = threadIdx.x; p < cnt; p += blockDim.x) {
-      const int slot = P.lst_ord[base + p];
+      const long long e = (part == 2) ? P.grp_ref[grp + p] : base + P.lst_ord[base + p];
       // split modes keep the exact integer E 2^q of a state; E = that times 2^-q (exact scaling)
-      D.E[p] = (P.mode == QIS_FP64) ? P.lst_E[base + slot] : (double)P.lst_q[base + slot] * d.inv_scale;
-      D.H[p] = P.lst_hash[base + slot];
-      D.R[p] = (int)(base + slot);
-      D.S[p] = ((unsigned long long)r << 32) | (unsigned)p;
+      D.E[p] = (P.mode == QIS_FP64) ? P.lst_E[e] : (double)P.lst_q[e] * d.inv_scale;
+      D.H[p] = P.lst_hash[e];
+      D.R[p] = (int)e;
+      D.S[p] = (part == 2) ? P.grp_src[grp + p] : ((unsigned long long)r << 32) | (unsigned)p;
     }
     __syncthreads();
-    if (r == 0) {
+    if (r == l0) {
       acnt = cnt;
       continue;
     }
@@ -132,6 +148,15 @@ __global__ void __launch_bounds__(256) k_final_merge(DevPtrs P) {
     A = T;
     T = t;
   }
+  if (part == 1) {
+    const long long g = (long long)inst * G + blockIdx.y;
+    for (int a = threadIdx.x; a < acnt; a += blockDim.x) {
+      P.grp_ref[g * K1 + a] = A.R[a];
+      P.grp_src[g * K1 + a] = A.S[a];
+    }
+    if (threadIdx.x == 0) P.grp_count[g] = acnt;
+    return;
+  }
   for (int a = threadIdx.x; a < K1; a += blockDim.x) {
     P.mrg_ref[inst * K1 + a] = (a < acnt) ? A.R[a] : -1;
     P.mrg_src[inst * K1 + a] = (a < acnt) ? A.S[a] : ~0ull;
@@ -141,6 +166,15 @@ __global__ void __launch_bounds__(256) k_final_merge(DevPtrs P) {
 
 size_t final_merge_smem(int K1) { return (size_t)3 * K1 * kSetBytes + (size_t)(2 * K1 + 1) * 4; }
 
+// Runs of consecutive searches merged side by side: about sqrt(R), so that both launches take as many
+// rounds; one run (one launch) while the rounds saved do not pay the second launch.
+int merge_groups(int R, int mode) {
+  if (mode == QIS_FP64 || R < 12) return 1;
+  int g = 1;
+  while (g * g < R) ++g;
+  return g;
+}
+
 cudaError_t launch_final_merge(const DevPtrs& P, cudaStream_t s) {
   const size_t sm = final_merge_smem(P.K1);
   static size_t attr = 0;
@@ -149,7 +183,12 @@ cudaError_t launch_final_merge(const DevPtrs& P, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     attr = sm;
   }
-  k_final_merge<<<P.n_inst, 256, sm, s>>>(P);
+  if (P.mrg_groups > 1) {
+    k_final_merge<<<dim3(P.n_inst, P.mrg_groups), 256, sm, s>>>(P, 1);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  k_final_merge<<<P.n_inst, 256, sm, s>>>(P, P.mrg_groups > 1 ? 2 : 0);
   return cudaGetLastError();
 }
 
