@@ -79,7 +79,6 @@ struct qis_ctx {
   double* scratch_E = nullptr;
   int scratch_states = 0;
   uint64_t launches = 0;
-  uint64_t cand_acc[2] = {0, 0};  // candidates of instances removed by qis_clear_instances
   // tunables (results never depend on them): scan chunk width 32 * tune_nc columns, searches
   // per scan task (0 = all R of the instance), searches per GEMM tile (0 = automatic)
   qis_tuning tune{8, 0, 0, 0};
@@ -183,10 +182,13 @@ int sync_and_check(qis_ctx* ctx) {
   return check_status(ctx);
 }
 
-// Candidates of the current instances: every productive iteration of a search of an n-spin
-// instance evaluates n(n-1)/2 pairs and n singles.
+// Candidates {pairs, singles} of the removed and the current instances: every productive iteration of
+// a search of an n-spin instance evaluates n(n-1)/2 pairs and n singles.
 int count_candidates(qis_ctx* ctx, uint64_t c[2]) {
-  c[0] = c[1] = 0;
+  unsigned long long acc[2];
+  CK(cudaMemcpy(acc, ctx->P.cand_acc, sizeof(acc), cudaMemcpyDeviceToHost));
+  c[0] = acc[0];
+  c[1] = acc[1];
   if (ctx->P.B == 0) return 0;
   std::vector<int> np(ctx->P.B);
   CK(cudaMemcpy(np.data(), ctx->P.nprod, sizeof(int) * np.size(), cudaMemcpyDeviceToHost));
@@ -549,6 +551,7 @@ int qis_create(const qis_config* cfg, qis_ctx** out) {
     CK(cudaMemset(P.e0_pend, 0, sizeof(int) * B));
     ALLOC(P.status, 4);
     ALLOC(P.nprod, B);
+    ALLOC(P.cand_acc, 2);
     ALLOC(P.npair, B);
     ALLOC(P.eval_cnt, 64);
     ALLOC(P.surv_tot, 64);
@@ -908,16 +911,7 @@ int qis_create_instances(qis_ctx* ctx, int count, const int* n, const double* co
 int qis_clear_instances(qis_ctx* ctx) {
   if (!ctx) return fail(nullptr, QIS_ERR_INVALID_ARG, "ctx is NULL");
   CK(cudaStreamSynchronize(ctx->stream));
-  {
-    uint64_t c[2];
-    int rc = count_candidates(ctx, c);
-    if (rc) return rc;
-    ctx->cand_acc[0] += c[0];
-    ctx->cand_acc[1] += c[1];
-    if (ctx->P.B > 0) CK(cudaMemset(ctx->P.nprod, 0, sizeof(int) * (size_t)ctx->P.B));
-    if (ctx->P.B > 0) CK(cudaMemset(ctx->P.npair, 0, sizeof(unsigned long long) * (size_t)ctx->P.B));
-  }
-  CK(cudaMemset(ctx->P.status, 0, sizeof(int)));   // device flags of the removed searches
+  if (ctx->P.B > 0) LAUNCH(launch_retire(ctx->P, ctx->stream));   // (before anything of the next instances)
   ctx->inst.clear();
   ctx->f64_wild = 0;
   ctx->inst_ready.clear();
@@ -1627,8 +1621,8 @@ int qis_candidate_count(qis_ctx* ctx, uint64_t* pairs, uint64_t* singles) {
   uint64_t c[2];
   int rc = count_candidates(ctx, c);
   if (rc) return rc;
-  if (pairs) *pairs = ctx->cand_acc[0] + c[0];
-  if (singles) *singles = ctx->cand_acc[1] + c[1];
+  if (pairs) *pairs = c[0];
+  if (singles) *singles = c[1];
   return 0;
 }
 
@@ -1652,7 +1646,7 @@ int qis_evaluated_pairs(qis_ctx* ctx, uint64_t* pairs) {
     uint64_t c[2];
     int rc = count_candidates(ctx, c);
     if (rc) return rc;
-    *pairs = ctx->cand_acc[0] + c[0];
+    *pairs = c[0];
     return 0;
   }
   unsigned long long v[64];

@@ -127,6 +127,7 @@ struct DevPtrs {
   int wait_probe;         // 1: the field GEMM's MMA thread first waits on a barrier that nothing
                           // completes (tests the timeout path); 0 otherwise
   int* nprod;             // [b] productive iterations (a parent was expanded) of search b
+  unsigned long long* cand_acc;  // [2] pair and single candidates of removed instances
   unsigned long long* npair;  // [b] pair candidates of the expanded parents of search b
   unsigned long long* eval_cnt;  // [64] pair terms the FP32 scan evaluated (live rows x chunk width)
   unsigned long long* surv_tot;  // [64] survivors the merge read (sum of the per-search counts)
@@ -389,6 +390,7 @@ cudaError_t launch_scan_pairs(const DevPtrs& P, const int4* tasks, int n_tasks, 
 cudaError_t launch_scan64(const DevPtrs& P, const int4* work, int n_work, cudaStream_t s);
 void scan_tasks_for(int inst, int n, int nc_max, int R, int RG, std::vector<int4>& out);
 cudaError_t launch_merge(const DevPtrs& P, cudaStream_t s);
+cudaError_t launch_retire(const DevPtrs& P, cudaStream_t s);
 int merge_groups(int R, int mode);
 cudaError_t launch_final_merge(const DevPtrs& P, cudaStream_t s);
 size_t merge_smem(int K1, int cap, int merge_cand);

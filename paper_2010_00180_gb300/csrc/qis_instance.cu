@@ -291,4 +291,35 @@ cudaError_t launch_hash_list(const DevPtrs& P, int b, int count, cudaStream_t s)
   return cudaGetLastError();
 }
 
+// The instances are removed: their candidates are added to those of earlier ones, their counts and the
+// device flags cleared. One block per instance, one launch: the same by copies to the host and memsets
+// were five blocking calls (a pipeline on one instance of n = 16, 4 searches, 8 iterations: 232 us with
+// them, 215 us with this launch).
+__global__ void __launch_bounds__(128) k_retire(DevPtrs P) {
+  const int n = P.inst[blockIdx.x].n;   // (up to date wherever a search has run)
+  unsigned long long pairs = 0, singles = 0;
+  for (int r = threadIdx.x; r < P.R; r += 128) {
+    const int b = blockIdx.x * P.R + r;
+    pairs += P.npair[b];
+    singles += (unsigned long long)P.nprod[b] * (unsigned)n;
+    P.npair[b] = 0;
+    P.nprod[b] = 0;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
+    singles += __shfl_xor_sync(0xffffffffu, singles, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    if (pairs) atomicAdd(P.cand_acc, pairs);
+    if (singles && P.flips != QIS_FLIPS_EXCHANGE) atomicAdd(P.cand_acc + 1, singles);
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) P.status[0] = 0;
+}
+
+cudaError_t launch_retire(const DevPtrs& P, cudaStream_t s) {
+  k_retire<<<P.n_inst, 128, 0, s>>>(P);
+  return cudaGetLastError();
+}
+
 }  // namespace qis
