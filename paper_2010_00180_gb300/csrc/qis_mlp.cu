@@ -83,10 +83,10 @@ __global__ void k_mlp_labels(const uint64_t* bits, int n, float* y) {
 // (K x H, row-major). A warp takes RT rows x 128 columns, a lane 4 adjacent columns: one weight
 // load per k serves RT rows, the activations are broadcast reads, and every sum is one chain of
 // FP32 fused multiply-adds over k ascending (the logits' bits do not depend on the tile). The
-// next eight rows of W are loaded while the current eight are used. put(row, column, the sums of
+// next D rows of W are loaded while the current D are used. put(row, column, the sums of
 // 4 columns) receives the results; in and the results must not share memory.
 constexpr int kCT = 4;   // columns of a lane
-template <int RT, typename Put>
+template <int RT, int D, typename Put>
 static __device__ __forceinline__ void mlp_layer(const float* in, int K, const __nv_bfloat16* __restrict__ W, int H, int TM,
                                                  Put put) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -99,19 +99,21 @@ static __device__ __forceinline__ void mlp_layer(const float* in, int K, const _
     for (int r = 0; r < RT; ++r)
 #pragma unroll
       for (int x = 0; x < kCT; ++x) acc[r][x] = 0.f;
-    uint2 w[8];
+    uint2 w[D];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) w[k] = *reinterpret_cast<const uint2*>(W + (long long)k * H + c);
+    for (int k = 0; k < D; ++k)
+      if (k < K) w[k] = *reinterpret_cast<const uint2*>(W + (long long)k * H + c);
 #pragma unroll 1
-    for (int k0 = 0; k0 < K; k0 += 8) {
-      uint2 v[8];
+    for (int k0 = 0; k0 < K; k0 += D) {
+      uint2 v[D];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
+      for (int k = 0; k < D; ++k) {
         v[k] = w[k];
-        if (k0 + 8 < K) w[k] = *reinterpret_cast<const uint2*>(W + (long long)(k0 + 8 + k) * H + c);
+        if (k0 + D + (k & ~7) < K) w[k] = *reinterpret_cast<const uint2*>(W + (long long)(k0 + D + k) * H + c);
       }
 #pragma unroll
-      for (int k4 = 0; k4 < 8; k4 += 4) {
+      for (int k4 = 0; k4 < D; k4 += 4) {
+        if (D > 8 && k0 + k4 >= K) break;   // (K is a multiple of 8)
         float4 a[RT];
 #pragma unroll
         for (int r = 0; r < RT; ++r) a[r] = *reinterpret_cast<const float4*>(in + (r0 + r) * K + k0 + k4);
@@ -146,14 +148,15 @@ static __device__ __forceinline__ void mlp_layer(const float* in, int K, const _
 // FP32 issue bounds it (M (4 H^2 + ..) multiply-adds); it replaces eleven launches whose tiles of
 // 64 x 64 fed four accumulators per shared-memory read. Loss and gradients of 4096 rows at H = 256
 // from host memory, with the weight gradients' kernel below (which took 3 x 90 us): 542 -> 195 us;
-// warm start of 120 instances of n = 300 and their searches: 44.1 -> 14.7 ms.
+// warm start of 120 instances of n = 300 and their searches: 44.1 -> 14.7 ms with the search kernel of
+// that time.
 struct MlpNet {
   const float* P;                   // master parameters (biases are read from it)
   const __nv_bfloat16 *Pb, *W2t, *W3t;
   int H, oW1, ob1, oW2, ob2, oW3, ob3, ow4, ob4;
 };
 
-template <int TM, int RT>
+template <int TM, int RT, int D>
 __global__ void __launch_bounds__(256) k_mlp_pass(MlpNet N, int M, const float* X, const float* y, float* z, float* dz,
                                                   double* loss, float inv_m, float* h1, float* h2, float* h3, float* d1,
                                                   float* d2, float* d3, float* G, int grads) {
@@ -170,7 +173,7 @@ __global__ void __launch_bounds__(256) k_mlp_pass(MlpNet N, int M, const float* 
   __syncthreads();
   // h = relu(in W + b) into `out`, and to global memory for a pass with labels
   auto forward = [&](const float* in, int K, int oW, int ob, float* out, float* h) {
-    mlp_layer<RT>(in, K, N.Pb + oW, H, TM, [&](int r, int c, const float* s) {
+    mlp_layer<RT, D>(in, K, N.Pb + oW, H, TM, [&](int r, int c, const float* s) {
 #pragma unroll
       for (int x = 0; x < kCT; x += 4) {
         const float4 b = *reinterpret_cast<const float4*>(N.P + ob + c + x);
@@ -225,7 +228,7 @@ __global__ void __launch_bounds__(256) k_mlp_pass(MlpNet N, int M, const float* 
   }
   __syncthreads();
   auto backward = [&](const float* in, const __nv_bfloat16* Wt, const float* h, float* out, float* d) {
-    mlp_layer<RT>(in, H, Wt, H, TM, [&](int r, int c, const float* s) {
+    mlp_layer<RT, D>(in, H, Wt, H, TM, [&](int r, int c, const float* s) {
 #pragma unroll
       for (int x = 0; x < kCT; x += 4) {
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -474,14 +477,14 @@ MlpNet net_of(const qis_mlp* m) {
   return MlpNet{m->P, m->Pb, m->W2t, m->W3t, m->H, m->oW1, m->ob1, m->oW2, m->ob2, m->oW3, m->ob3, m->ow4, m->ob4};
 }
 
-template <int TM, int RT>
+template <int TM, int RT, int D>
 cudaError_t pass_tm(qis_mlp* m, int M, const float* X, const float* y, cudaStream_t s) {
   const size_t sm = (size_t)2 * TM * m->H * sizeof(float);
   if (sm > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(k_mlp_pass<TM, RT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const cudaError_t e = cudaFuncSetAttribute(k_mlp_pass<TM, RT, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
   }
-  k_mlp_pass<TM, RT><<<(M + TM - 1) / TM, 256, sm, s>>>(net_of(m), M, X, y, m->zb, m->dzb, m->loss, 1.f / (float)M, m->h1,
+  k_mlp_pass<TM, RT, D><<<(M + TM - 1) / TM, 256, sm, s>>>(net_of(m), M, X, y, m->zb, m->dzb, m->loss, 1.f / (float)M, m->h1,
                                                             m->h2, m->h3, m->d1, m->d2, m->d3, y ? m->G : nullptr,
                                                             m->n_params);
   return cudaGetLastError();
@@ -493,10 +496,16 @@ cudaError_t pass_tm(qis_mlp* m, int M, const float* X, const float* y, cudaStrea
 // qis_mlp_forward at H = 256 with 4 / 8 / 16 / 32 (8 columns a lane) rows: M = 300 45 / 47 / 58 /
 // 72 us, M = 2000 72 / 60 / 60 / 73, M = 4096 104 / 92 / 72 / 81; of qis_mlp_loss_grad M = 700 111 /
 // 114 / 135 / 172, M = 2000 160 / 127 / 142 / 176, M = 4096 232 / 207 / 180 / 194.
+// With one block of 4 rows per SM at most, its loads from L2 bound it and 32 rows of W are in flight
+// (163 registers); beyond that two blocks per SM have to fit (56 registers with 8). 32 / 8 at M = 300:
+// qis_mlp_loss_grad H = 256 97 / 110 us, H = 512 220 / 267, qis_mlp_forward H = 512 82 / 107; at M = 700
+// qis_mlp_loss_grad H = 256 135 / 112. Warm starts of 120 instances of n = 300 and their searches
+// 12.4 / 13.0 ms.
 cudaError_t mlp_pass(qis_mlp* m, int M, const float* X, const float* y, cudaStream_t s) {
-  if (M <= 8 * m->sms) return pass_tm<4, 1>(m, M, X, y, s);
-  if (M <= 18 * m->sms) return pass_tm<8, 2>(m, M, X, y, s);
-  return pass_tm<16, 4>(m, M, X, y, s);
+  if (M <= 4 * m->sms) return pass_tm<4, 1, 32>(m, M, X, y, s);
+  if (M <= 8 * m->sms) return pass_tm<4, 1, 8>(m, M, X, y, s);
+  if (M <= 18 * m->sms) return pass_tm<8, 2, 8>(m, M, X, y, s);
+  return pass_tm<16, 4, 8>(m, M, X, y, s);
 }
 
 // Gradients of the mean loss over the rows of the last mlp_pass with labels, into G.
