@@ -160,6 +160,7 @@ static __device__ __noinline__ float kth_survivor(const unsigned long long* ssv,
 // 9.7 ms, 12.4 with the sites of the duplicates too, and 86 ms in the per-kernel form (every pair in
 // FP64). An instance exactly on its grid needs no
 // chain: every partial sum is exact, so the fixed-point field is the same double.
+template <int U = 8>
 static __device__ __forceinline__ void fields_f64(const DevPtrs& P, const InstDesc& d, const uint64_t* pb,
                                                   const long long* aq, const unsigned short* list, int m, double* ad) {
   const int n = d.n;
@@ -174,7 +175,7 @@ static __device__ __forceinline__ void fields_f64(const DevPtrs& P, const InstDe
     for (int j0 = 0; j0 < n; j0 += 64) {
       const uint64_t w = pb[j0 >> 6];
       const int e = min(64, n - j0);
-#pragma unroll 8
+#pragma unroll U
       for (int u = 0; u < e; ++u) {
         const double v = J[(long long)(j0 + u) * d.n_pad];
         const double x = __longlong_as_double(__double_as_longlong(v) ^ (long long)((w >> u) << 63));
@@ -184,6 +185,65 @@ static __device__ __forceinline__ void fields_f64(const DevPtrs& P, const InstDe
     const double f = __dadd_rn(acc, P.h64[d.off_vec + i]);
     ad[i] = sigma_of(pb, i) ? 2.0 * f : -2.0 * f;
   }
+}
+
+// FP64 mode, more survivors than the buffer holds and none to be told apart by the FP32 band (equal or
+// nearly equal changes of energy): the survivors taken again by their defining energies, as the per-kernel
+// form takes them, E' < T and E' at or below the k-th lowest of such candidates (radix select of the
+// order keys, the energies formed anew in each pass). Returns their number, of which the first cap are
+// held. Rare: out of line, every candidate nine times; it takes little from the caller, whose registers
+// are full, and finds the block's arrays again.
+static __device__ __noinline__ int exact_survivors(const DevPtrs& P, const long long* aq, double Ep, double T, int k, int* s_cnt) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int b = blockIdx.x;
+  const InstDesc& d = P.inst[b / P.R];
+  const bool ex = P.flips == QIS_FLIPS_EXCHANGE;
+  const SearchLayout L = search_layout(P.NP, P.Wmax, P.K1, P.cap, P.merge_cand, blockDim.x >> 5, true);
+  const uint64_t* pb = reinterpret_cast<const uint64_t*>(smem + L.pb);
+  unsigned long long* ssv = reinterpret_cast<unsigned long long*>(smem + L.ssv);
+  double* ad = reinterpret_cast<double*>(smem + L.ad);
+  unsigned short* list = reinterpret_cast<unsigned short*>(smem + L.us);
+  int* hist = reinterpret_cast<int*>(smem + L.pc);
+#pragma unroll 1
+  for (int i = threadIdx.x; i < d.n; i += blockDim.x) list[i] = (unsigned short)i;
+  if (threadIdx.x == 0) *s_cnt = 0;
+  __syncthreads();
+  fields_f64<1>(P, d, pb, aq, list, d.n, ad);
+  unsigned long long prefix = 0;
+  int rank = k - 1;
+  // passes over the candidates below T: eight bits of the k-th lowest key each (all ones where there are
+  // fewer than k: find_bin gives the last bin then), then the taking
+#pragma unroll 1
+  for (int shift = 56; shift >= -8; shift -= 8) {
+#pragma unroll 1
+    for (int x = threadIdx.x; x < 256; x += blockDim.x) hist[x] = 0;
+    __syncthreads();
+#pragma unroll 1
+    for (int i = threadIdx.x >> 5; i < d.n; i += blockDim.x >> 5)
+#pragma unroll 1
+      for (int j = i + (threadIdx.x & 31); j < d.n; j += 32) {
+        const int flip = sigma_of(pb, i) ^ sigma_of(pb, j);
+        if (ex && !flip) continue;
+        // (j = i: the flip of site i alone)
+        const double de = j == i ? ad[i] : dE64(ad[i], ad[j], P.J64[d.off_mat + (long long)i * d.n_pad + j], flip);
+        const double e = __dadd_rn(Ep, de);
+        if (!(e < T)) continue;
+        const unsigned long long key = dkey(e);
+        if (shift >= 0) {
+          if (shift == 56 || key >> (shift + 8) == prefix) atomicAdd(&hist[(int)(key >> shift) & 255], 1);
+        } else if (key <= prefix) {
+          const int slot = atomicAdd(s_cnt, 1);
+          if (slot < P.cap) *(slot < kSSV ? ssv + slot : P.surv + (long long)b * P.cap + slot) = surv_entry(i, j == i ? -1 : j);
+        }
+      }
+    __syncthreads();
+    if (shift < 0) break;
+    int bin;
+    find_bin(hist, rank, bin, rank);   // every warp alike
+    prefix = (prefix << 8) | (unsigned)bin;
+    __syncthreads();
+  }
+  return *s_cnt;
 }
 
 // The candidate sites of an iteration, from scratch (out of line: the first iteration of a launch, or
@@ -313,6 +373,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
   unsigned* vmax = reinterpret_cast<unsigned*>(vhist + 256);    // [256] and their maxima
 
   __shared__ int s_sel, s_near, s_ns, s_nv, s_ocut, s_cn, s_m0, s_m1, s_set, s_nset;
+  __shared__ int s_hold;   // FP64 mode: 1 + the survivors at hand before the scan, 0: none
   __shared__ float wf[2 * NW], s_u, s_thr[2];
   __shared__ int s_w[33];
   __shared__ unsigned long long s_kmm[2 * NW];
@@ -360,7 +421,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
     __syncthreads();
   };
 
-  if (tid == 0) s_u = INFINITY;
+  if (tid == 0) {
+    s_u = INFINITY;
+    s_hold = 0;
+  }
   int act = act0, cur = 0, nprod = 0;
   int pgen = 0, pi0 = -1, pj0 = -1;   // the parent's generation in this launch and its flips
   unsigned npair = 0, nev = 0, nsurv = 0;   // of this launch (at most 128 iterations: 32 bits); npair: exchanges
@@ -389,7 +453,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
     if (tid == 0) {
       s_set = iter > 0 && s_nset && s_ns <= K1;   // (s_set, s_nset: see the bound)
       s_near = 0;
-      s_ns = 0;
+      s_ns = F64 && s_hold ? s_hold - 1 : 0;
       s_nv = 0;
       s_cn = 0;
       s_ocut = cnt;
@@ -732,7 +796,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
       // the row of each pair, while the pairs fit the space of the sites as listed
       unsigned short* rowof = reinterpret_cast<unsigned short*>(smem + L.ua);
       const int rcap = P.NP * 3;
-      const int per = (cn + NT - 1) / NT, q0 = min(cn, tid * per), q1 = min(cn, q0 + per);
+      const int cs = F64 && s_hold ? 0 : cn;
+      const int per = (cs + NT - 1) / NT, q0 = min(cs, tid * per), q1 = min(cs, q0 + per);
       int sum = 0;
 #pragma unroll 1
       for (int q = q0; q < q1; ++q) {
@@ -827,18 +892,24 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
     __syncthreads();   // every survivor written; the scan's scratch is free
     const int S = s_ns;
     // Block-uniform, rare: the k-th lowest dE of the cap survivors held bounds that of all candidates, and
-    // the iteration runs again with it, each time over fewer; an error only when more than the buffer
-    // holds are equal
+    // the iteration runs again with it, each time over fewer (FP64 mode: where it tells none apart, with
+    // the survivors by their defining energies in place of the scan's); an error only when more than the
+    // buffer holds are equal
     if (S > cap) {
       const float v = kth_survivor(ssv, surv, cap, K1 + s_near, aqb, scale_q, J4, d.n_pad, pb, reinterpret_cast<int*>(pc));
       const bool lower = __fadd_ru(v, s_thr[1]) < s_thr[0];
       __syncthreads();
+      int held = cap + 1;
+      if (F64 && !lower)
+        held = exact_survivors(P, aqb, __longlong_as_double(Epq), cnt == K1 ? dkey_inv(okey[K1 - 1]) : INFINITY, K1 + s_near, &s_ns);
+      const bool again = lower || held <= cap;
       if (tid == 0) {
-        if (!lower) atomicOr(P.status, kStatCapacity);
+        if (!again) atomicOr(P.status, kStatCapacity);
         else if (!(ext && iter == 0)) oused[oslot[s_sel]] = 0;
         s_u = lower ? v : INFINITY;
+        if (F64) s_hold = held <= cap ? held + 1 : 0;
       }
-      if (lower) --iter; else act = 0;
+      if (again) --iter; else act = 0;
       __syncthreads();
       continue;
     }
@@ -851,7 +922,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
         npair += (unsigned)(down * (n - down));
       }
     }
-    if (tid == 0) s_u = INFINITY;
+    if (tid == 0) {
+      s_u = INFINITY;
+      if (F64) s_hold = 0;
+    }
     // the next iteration's guess: this one's need and a quarter of its span as a margin (the bound and
     // the lowest a_i move by a few per cent of the span per iteration; a guess too low costs a second
     // pass over the sites, one too high longer lists)
