@@ -764,16 +764,20 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
       // same value from the same operands.)
       const unsigned long long kT = okey[K1 - 1];
       // FP64 mode: E' = fl(E_p + dE) < T needs dE < T - E_p, and E' at or below the k-th lowest needs dE
-      // within an ulp of E' of its dE; |E'| <= n (|a|max + n j4max / 4) with n <= 1024, so that ulp and
-      // the roundings of the FP64 fields are below 2^-10 of delta; the grid 2^-q (2^q sum |J| >= 2^50)
-      // puts a_i + a_j off by at most 2 n 2^-q <= 2^-22 j4max, half of delta's margin.
+      // within an ulp of E' of its dE. An imported E_p can be any finite number, so four ulps of E_p join
+      // delta (that ulp is at most two of E_p's, or below 2^-20 of |dE|); of a computed E_p they are
+      // nothing beside it (|E_p| <= n (|a|max + n j4max / 4), n <= 1024), nor are the roundings of the FP64
+      // fields; the grid 2^-q (2^q sum |J| >= 2^50) puts a_i + a_j off by at most 2 n 2^-q <= 2^-22 j4max,
+      // half of delta's margin.
       const float tE = (cnt != K1) ? INFINITY
                        : F64 ? __double2float_ru(__dsub_ru(dkey_inv(kT), __longlong_as_double(Epq)))
                              : __fmul_ru(__ll2float_ru((long long)(kT ^ (1ull << 63)) - Epq), scale_q);
       const float tt = fminf(tE, Uf);
       const float big = __fadd_ru(__fadd_ru(__fmul_ru(3.f, fmaxf(fabsf(amin), fabsf(amax))), d.j4max),
                                   isinf(tt) ? 0.f : fabsf(tt));
-      const float delta = __fmul_ru(big, 0x1p-21f);
+      float delta = __fmul_ru(big, 0x1p-21f);
+      if (F64)   // 2^(e - 1073) of E_p's exponent field e, as a float's (infinite from 2^128 on)
+        delta = __fadd_ru(delta, __int_as_float(min(255, max(1, (int)(Epq >> 52 & 0x7ff) - 946)) << 23));
       thr = fminf(__fadd_ru(tE, delta), __fadd_ru(Uf, 2.f * delta));
       if (tid == 0) {
         s_nset = cnt == K1 && tE <= Uf;
