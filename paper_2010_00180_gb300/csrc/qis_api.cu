@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "qis_common.cuh"
+#include "qis_smem.cuh"
 
 using namespace qis;
 
@@ -369,6 +370,16 @@ void qis::gf_tables(GfTables& g) {
   }
   for (int e = 0; e < 2 * N; ++e) g.root[e] = sol[g.exp[e] ^ 1];
   g.root1 = sol[1];
+}
+
+cudaError_t qis::allow_smem(const void* kernel, size_t bytes) {
+  static SmemLimits limits;
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  return (cudaError_t)limits.raise(dev, kernel, bytes, [&] {
+    return (int)cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  });
 }
 
 void qis::set_global_error(const char* msg) { g_create_error = msg; }

@@ -353,6 +353,9 @@ cudaError_t mlp_propose_states(qis_mlp* m, const double* J64, long long stride, 
                                uint64_t key, uint64_t* init_bits, int Wstride, cudaStream_t s);
 int mlp_max_n(const qis_mlp* m);
 
+// Allow launches of `kernel` with `bytes` of dynamic shared memory on the current device; before each launch.
+cudaError_t allow_smem(const void* kernel, size_t bytes);
+
 // Kernel launchers (defined in the .cu files); each returns the cudaError_t of the launch.
 // Where one instance of a creation batch was staged and where its layout and statistics go.
 struct LayoutItem {

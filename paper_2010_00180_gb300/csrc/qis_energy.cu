@@ -28,7 +28,6 @@
 // n = 200 .. 700 1.38 -> 0.07 ms, of 120 of n = 600 on their grid 0.87 -> 0.2 ms. The block that
 // completes a state's sums forms its energy (a second launch cost a small call 6 us).
 #include <algorithm>
-#include <atomic>
 
 #include "qis_tc.cuh"
 
@@ -286,12 +285,8 @@ static cudaError_t launch_energy(const DevPtrs& P, const EnergyJob& E, int n_ins
   // asks for more than half of the shared memory
   size_t sm = 2 * (size_t)(kEnTileA + digits * kEnTileD) + 1024;
   if (ncols > 256) sm = std::max<size_t>(sm, 120 * 1024);
-  static std::atomic<bool> attr{false};
-  if (!attr.load()) {
-    const cudaError_t e = cudaFuncSetAttribute(k_energy, cudaFuncAttributeMaxDynamicSharedMemorySize, 120 * 1024);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  const cudaError_t ea = allow_smem((const void*)k_energy, sm);
+  if (ea != cudaSuccess) return ea;
   for (int z = 0; z < n_inst; z += 65535) {   // (the grid's third dimension)
     EnergyJob F = E;
     F.inst0 = E.inst0 + z;

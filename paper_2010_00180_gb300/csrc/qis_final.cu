@@ -177,12 +177,8 @@ int merge_groups(int R, int mode) {
 
 cudaError_t launch_final_merge(const DevPtrs& P, cudaStream_t s) {
   const size_t sm = final_merge_smem(P.K1);
-  static size_t attr = 0;
-  if (attr < sm) {
-    const cudaError_t e = cudaFuncSetAttribute(k_final_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    attr = sm;
-  }
+  const cudaError_t ea = allow_smem((const void*)k_final_merge, sm);
+  if (ea != cudaSuccess) return ea;
   if (P.mrg_groups > 1) {
     k_final_merge<<<dim3(P.n_inst, P.mrg_groups), 256, sm, s>>>(P, 1);
     const cudaError_t e = cudaGetLastError();

@@ -302,12 +302,8 @@ cudaError_t launch_fields_tc(const DevPtrs& P, const void* D16, const void* S16,
   G.stages = gemm_stages(digits_max, G.NT);
   G.nbuf = (2 * digits_max * G.NT <= 512) ? 2 : 1;   // double-buffered accumulators if TMEM holds two
   const size_t sm = gemm_smem(digits_max, G.NT);
-  static size_t attr = 0;
-  if (attr < sm) {
-    e = cudaFuncSetAttribute(k_fields_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    attr = sm;
-  }
+  e = allow_smem((const void*)k_fields_tc, sm);
+  if (e != cudaSuccess) return e;
   static int n_sm = 0;
   if (n_sm == 0) {
     int dev = 0;

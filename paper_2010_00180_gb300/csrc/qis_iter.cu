@@ -621,12 +621,8 @@ cudaError_t launch_bound(const DevPtrs& P, cudaStream_t s) {
   // the split modes keep the subset as floats: a smaller footprint, ten blocks per SM
   const size_t sm = (size_t)kSubMax * (P.mode == QIS_FP64 ? 8 : 4) + (size_t)P.NP * sizeof(float2) +
                     (size_t)P.Wmax * 8 + (size_t)(P.NP / 32) * 4;
-  static size_t attr = 0;
-  if (attr < sm) {
-    cudaError_t e = cudaFuncSetAttribute(k_bound, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    attr = sm;
-  }
+  const cudaError_t e = allow_smem((const void*)k_bound, sm);
+  if (e != cudaSuccess) return e;
   k_bound<<<P.B, 128, sm, s>>>(P);
   return cudaGetLastError();
 }

@@ -304,12 +304,8 @@ size_t merge_smem(int K1, int cap, int merge_cand) {
 
 cudaError_t launch_merge(const DevPtrs& P, cudaStream_t s) {
   const size_t sm = merge_smem(P.K1, P.cap, P.merge_cand);
-  static size_t attr = 0;
-  if (attr < sm) {
-    cudaError_t e = cudaFuncSetAttribute(k_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    attr = sm;
-  }
+  const cudaError_t e = allow_smem((const void*)k_merge, sm);
+  if (e != cudaSuccess) return e;
   k_merge<<<P.B, kMergeThreads, sm, s>>>(P);
   return cudaGetLastError();
 }

@@ -481,7 +481,7 @@ template <int TM, int RT, int D>
 cudaError_t pass_tm(qis_mlp* m, int M, const float* X, const float* y, cudaStream_t s) {
   const size_t sm = (size_t)2 * TM * m->H * sizeof(float);
   // (a launch without the attribute gets 48 KiB with the kernel's static arrays, not beside them)
-  const cudaError_t e = cudaFuncSetAttribute(k_mlp_pass<TM, RT, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  const cudaError_t e = allow_smem((const void*)k_mlp_pass<TM, RT, D>, sm);
   if (e != cudaSuccess) return e;
   k_mlp_pass<TM, RT, D><<<(M + TM - 1) / TM, 256, sm, s>>>(net_of(m), M, X, y, m->zb, m->dzb, m->loss, 1.f / (float)M, m->h1,
                                                             m->h2, m->h3, m->d1, m->d2, m->d3, y ? m->G : nullptr,

@@ -549,14 +549,9 @@ size_t scan_sparse_smem(int NP) { return (size_t)NP * 8 + (size_t)NP * 12; }
 
 cudaError_t launch_scan_sparse(const DevPtrs& P, cudaStream_t s) {
   const size_t sm = scan_sparse_smem(P.NP);
-  static size_t attr[2] = {0, 0};
-  const int ex = P.flips == QIS_FLIPS_EXCHANGE;
-  if (attr[ex] < sm) {
-    cudaError_t e = ex ? cudaFuncSetAttribute(k_scan_sparse<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)
-                       : cudaFuncSetAttribute(k_scan_sparse<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    attr[ex] = sm;
-  }
+  const bool ex = P.flips == QIS_FLIPS_EXCHANGE;
+  const cudaError_t e = allow_smem(ex ? (const void*)k_scan_sparse<true> : (const void*)k_scan_sparse<false>, sm);
+  if (e != cudaSuccess) return e;
   if (ex) k_scan_sparse<true><<<P.B, 128, sm, s>>>(P);
   else k_scan_sparse<false><<<P.B, 128, sm, s>>>(P);
   return cudaGetLastError();

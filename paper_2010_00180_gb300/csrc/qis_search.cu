@@ -1237,12 +1237,8 @@ template <int FL, bool F64, int NT>
 static cudaError_t launch_search_as(const DevPtrs& P, int n_iters, int ext, cudaStream_t s) {
   const SearchLayout L = search_layout(P.NP, P.Wmax, P.K1, P.cap, P.merge_cand, NT / 32, F64);
   const size_t sm = (size_t)L.total;
-  static size_t attr = 0;
-  if (attr < sm) {
-    const cudaError_t e = cudaFuncSetAttribute(k_search<FL, F64, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    attr = sm;
-  }
+  const cudaError_t e = allow_smem((const void*)k_search<FL, F64, NT>, sm);
+  if (e != cudaSuccess) return e;
   k_search<FL, F64, NT><<<P.B, NT, sm, s>>>(P, n_iters, ext);
   return cudaGetLastError();
 }

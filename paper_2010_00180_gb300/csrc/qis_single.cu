@@ -537,12 +537,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_single(DevPtrs P, int n_iters
 template <int NT>
 static cudaError_t launch_single_nt(const DevPtrs& P, int n_iters, int ext, cudaStream_t s) {
   const size_t sm = (size_t)single_layout(P.NP, P.Wmax, P.K1, NT / 32).total;
-  static size_t attr = 0;
-  if (attr < sm) {
-    const cudaError_t e = cudaFuncSetAttribute(k_single<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    attr = sm;
-  }
+  const cudaError_t e = allow_smem((const void*)k_single<NT>, sm);
+  if (e != cudaSuccess) return e;
   k_single<NT><<<P.B, NT, sm, s>>>(P, n_iters, ext);
   return cudaGetLastError();
 }
