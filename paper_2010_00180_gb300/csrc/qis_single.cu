@@ -330,10 +330,21 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_single(DevPtrs P, int n_iters
       block_exclusive_sum(mine, s_w, &tot);
       upto = tot;
     }
-    if (upto > cap) {   // block-uniform: more ties at the bound than the search's buffer holds
-      if (tid == 0) atomicOr(P.status, kStatCapacity);
-      act = 0;
-      continue;
+    const long long Tq = (cnt == K1) ? (long long)(okey[K1 - 1] ^ (1ull << 63)) : LLONG_MAX;
+    if (upto > cap) {
+      // block-uniform, rare: more ties at the bound than the search's buffer holds. Only those below the
+      // last kept energy, and no kept states, take a place in it; an error if they are too many
+      int mine = 0;
+      for (int i = tid; i < n; i += NT)
+        mine += (!fine || reinterpret_cast<unsigned*>(a)[i] <= kth) && Epq + ax[i] < Tq && !((dupm[i >> 5] >> (i & 31)) & 1u);
+      int tot;
+      block_exclusive_sum(mine, s_w, &tot);
+      upto = tot;
+      if (upto > cap) {
+        if (tid == 0) atomicOr(P.status, kStatCapacity);
+        act = 0;
+        continue;
+      }
     }
     if (upto > kSgBuf) {
       const long long stride = next_pow2(max(cap, 256));
@@ -342,7 +353,6 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_single(DevPtrs P, int n_iters
     }
     nsurv += (unsigned long long)upto;
     // ---------------------------------------------------------------- merge (Alg. 2)
-    const long long Tq = (cnt == K1) ? (long long)(okey[K1 - 1] ^ (1ull << 63)) : LLONG_MAX;
     unsigned long long kmn = ~0ull, kmx = 0;
     for (int u0 = 0; u0 < n; u0 += NT) {
       const int i = u0 + tid;
