@@ -786,6 +786,7 @@ namespace {
 // init_E / init_q when those still hold them.
 int flush_init(qis_ctx* ctx, bool defer) {
   const int ni = (int)ctx->init_pending.size();
+  CK(cudaSetDevice(ctx->cfg.device));
   if (ctx->e0_unresolved) {   // a deferred start whose kernel never ran: start those again
     for (int x = 0; x < ni; ++x)
       if (ctx->e0_deferred[x]) ctx->init_pending[x] = 1;
@@ -921,6 +922,7 @@ int qis_create_instances(qis_ctx* ctx, int count, const int* n, const double* co
 
 int qis_clear_instances(qis_ctx* ctx) {
   if (!ctx) return fail(nullptr, QIS_ERR_INVALID_ARG, "ctx is NULL");
+  CK(cudaSetDevice(ctx->cfg.device));
   CK(cudaStreamSynchronize(ctx->stream));
   if (ctx->P.B > 0) LAUNCH(launch_retire(ctx->P, ctx->stream));   // (before anything of the next instances)
   ctx->inst.clear();
