@@ -114,7 +114,10 @@ __global__ void __launch_bounds__(256) k_energy(DevPtrs P, EnergyJob E, int nseg
   uint64_t wd[4];   // the step's word of states r, r + 32, ..
   auto fetch = [&](int kc) {
 #pragma unroll
-    for (int m = 0; m < 4; ++m) wd[m] = kc < d.W ? st_ptr[r + 32 * m][kc] : 0ull;   // (the extra site: spin +1)
+    for (int m = 0; m < 4; ++m) wd[m] = kc < d.W ? st_ptr[r + 32 * m][kc] : 0ull;
+    if (kc == n >> 6)   // the extra site: spin +1, whatever the caller's word holds there (sites past it have no couplings)
+#pragma unroll
+      for (int m = 0; m < 4; ++m) wd[m] &= ~(1ull << (n & 63));
     const int j0 = kc * 64 + c * 8;
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
