@@ -47,7 +47,8 @@ struct qis_ctx {
   long long* hq = nullptr;
   uint64_t* zob = nullptr;
   double* stats = nullptr;
-  double* jstage = nullptr;   // [max_inst][NP * NP] couplings as copied from the host (FP64 mode)
+  double* jstage = nullptr;   // [jstage_n][max_n * max_n] couplings as copied from the host (FP64 mode without Jq)
+  int jstage_n = 0;           // (with Jq: staged in the instances' own regions of it)
   bool f64_filter = false;    // FP64 mode: the context holds the filter's fixed-point and FP32 couplings
   int f64_wild = 0;           // FP64 mode: instances whose magnitudes the FP32 filter does not cover
   LayoutItem* items_d = nullptr;   // [max_inst] staging places of a creation batch
@@ -451,13 +452,17 @@ int qis_create(const qis_config* cfg, qis_ctx** out) {
     ALLOC(ctx->zob, kMaxN);
     ALLOC(ctx->stats, (size_t)ctx->max_inst * (NP + 8));   // validation statistics of every instance
     ALLOC(ctx->items_d, (size_t)ctx->max_inst);
-    if (ctx->mode == QIS_FP64) ALLOC(ctx->jstage, (size_t)ctx->pool_mat);   // the split modes stage in Jq
     ctx->f64_filter = ctx->mode == QIS_FP64 && ctx->cfg.flips != QIS_FLIPS_SINGLE && ctx->NP <= kSearchMaxNP &&
                       ctx->K1 <= kSearchMaxK1;
     if (ctx->f64_filter) {   // the fixed-point fields and FP32 couplings of the fused search's filter
       ALLOC(ctx->Jq, ctx->pool_mat);
       ALLOC(ctx->J4, ctx->pool_mat);
       ALLOC(ctx->hq, ctx->pool_vec);
+    }
+    if (!ctx->Jq) {   // as many instances as fit in 64 MiB, one at least
+      const size_t one = (size_t)cfg->max_n * cfg->max_n;
+      ctx->jstage_n = (int)std::min<size_t>(ctx->max_inst, std::max<size_t>(1, (64ull << 20) / (one * sizeof(double))));
+      ALLOC(ctx->jstage, one * ctx->jstage_n);
     }
     ALLOC(ctx->all_bits, (size_t)ctx->max_inst * K1 * W);
     ALLOC(ctx->all_E, (size_t)ctx->max_inst * K1);
@@ -864,42 +869,51 @@ int qis_create_instances(qis_ctx* ctx, int count, const int* n, const double* co
     if (rc) return rc;
   }
   CK(cudaSetDevice(ctx->cfg.device));
-  // every copy, then every layout and validation, then one read-back of all statistics. Each
-  // instance is staged in its own region (split modes: of the fixed-point pool, written from J64
-  // later), so the copies run back to back.
+  // every copy, then every layout and validation, then one read-back of all statistics. Each instance is
+  // staged in its own region of the fixed-point pool (written from J64 later), so the copies run back to
+  // back; without that pool in jstage, whose places the next instances take once the layout of those in
+  // it is enqueued (the copies and launches are in order on the stream).
   {
     const int rc = copy_fields_h(ctx, first, count, n, h);
     if (rc) return rc;
   }
   {
-    // a page-locked J is read by the layout kernel itself (one pass over the host memory);
-    // any other J is staged with a copy first
-    std::vector<const double*> src(count);
-    for (int k = 0; k < count; ++k) {
-      src[k] = pinned_view(J[k]);
-      if (src[k]) continue;
-      double* stage = (ctx->mode == QIS_FP64 ? ctx->jstage : reinterpret_cast<double*>(ctx->Jq)) +
-                      (long long)(first + k) * ctx->NP * ctx->NP;
-      const int rc = copy_instance(ctx, n[k], J[k], stage);
-      if (rc) return rc;
-      src[k] = stage;
-    }
-    // padded layout and validation of the whole batch: two launches
     std::vector<LayoutItem> items(count);
-    int max_pad = 0;
+    CK(cudaMemsetAsync(ctx->stats, 0, sizeof(double) * (size_t)count * (ctx->NP + 8), ctx->stream));
+    int k0 = 0, max_pad = 0, staged = 0;   // the items not laid out yet, and the places of jstage they hold
+    // padded layout and validation of items k0 .. k1 - 1: two launches
+    auto lay_out = [&](int k1) -> int {
+      CK(cudaMemcpyAsync(ctx->items_d + k0, items.data() + k0, sizeof(LayoutItem) * (k1 - k0), cudaMemcpyHostToDevice, ctx->stream));
+      LAUNCH(launch_layout_batch(ctx->P, ctx->items_d + k0, k1 - k0, max_pad, ctx->J64, ctx->stream));
+      k0 = k1;
+      max_pad = staged = 0;
+      return 0;
+    };
     for (int k = 0; k < count; ++k) {
       LayoutItem& L = items[k];
-      L.src = src[k];
+      // a page-locked J is read by the layout kernel itself (one pass over the host memory);
+      // any other J is staged with a copy first
+      L.src = pinned_view(J[k]);
       L.off_mat = (long long)(first + k) * ctx->NP * ctx->NP;
       L.off_vec = (long long)(first + k) * ctx->NP;
       L.n = n[k];
       L.n_pad = pad_of(n[k]);
       L.stats = ctx->stats + (size_t)k * (ctx->NP + 8);
+      if (!L.src) {
+        if (ctx->jstage && staged == ctx->jstage_n) {
+          const int rc = lay_out(k);
+          if (rc) return rc;
+        }
+        double* stage = ctx->jstage ? ctx->jstage + (size_t)staged++ * ctx->cfg.max_n * ctx->cfg.max_n
+                                    : reinterpret_cast<double*>(ctx->Jq) + L.off_mat;
+        const int rc = copy_instance(ctx, n[k], J[k], stage);
+        if (rc) return rc;
+        L.src = stage;
+      }
       max_pad = std::max(max_pad, L.n_pad);
     }
-    CK(cudaMemsetAsync(ctx->stats, 0, sizeof(double) * (size_t)count * (ctx->NP + 8), ctx->stream));
-    CK(cudaMemcpyAsync(ctx->items_d, items.data(), sizeof(LayoutItem) * count, cudaMemcpyHostToDevice, ctx->stream));
-    LAUNCH(launch_layout_batch(ctx->P, ctx->items_d, count, max_pad, ctx->J64, ctx->stream));
+    const int rc = lay_out(count);
+    if (rc) return rc;
   }
   const size_t stride = (size_t)ctx->NP + 8;
   std::vector<double> st(stride * count);
