@@ -387,8 +387,11 @@ void qis::set_global_error(const char* msg) { g_create_error = msg; }
 
 extern "C" {
 
+namespace {
+int make_context(const qis_config* cfg, int cap, bool filter, qis_ctx** out);
+}
+
 int qis_create(const qis_config* cfg, qis_ctx** out) {
-  qis_ctx* ctx = nullptr;
   if (!cfg || !out) return fail(nullptr, QIS_ERR_INVALID_ARG, "cfg and out must not be NULL");
   *out = nullptr;
   if (cfg->K < 1 || cfg->K + 1 > 4096) return fail(nullptr, QIS_ERR_INVALID_ARG, "K must satisfy 1 <= K and K+1 <= 4096");
@@ -406,7 +409,14 @@ int qis_create(const qis_config* cfg, qis_ctx** out) {
     cudaError_t e = cudaSetDevice(cfg->device);
     if (e != cudaSuccess) return fail(nullptr, QIS_ERR_CUDA, std::string("cudaSetDevice: ") + cudaGetErrorString(e));
   }
-  ctx = new qis_ctx();
+  return make_context(cfg, cap, true, out);
+}
+
+namespace {
+
+// filter: the FP64 mode with the fused search's filter, where the sizes allow it.
+int make_context(const qis_config* cfg, int cap, bool filter, qis_ctx** out) {
+  qis_ctx* ctx = new qis_ctx();
   ctx->cfg = *cfg;
   ctx->K1 = cfg->K + 1;
   ctx->R = cfg->R;
@@ -430,9 +440,11 @@ int qis_create(const qis_config* cfg, qis_ctx** out) {
     ctx->no_fused = fz && fz[0] == '0';
   }
   auto bail = [&](int rc) {
+    const bool plain = rc == QIS_ERR_OOM && ctx->f64_filter;
     g_create_error = ctx->err;
     qis_destroy(ctx);
-    return rc;
+    // the filter's planes (12 bytes per coupling) and rings do not fit: the per-kernel form needs none
+    return plain ? make_context(cfg, cap, false, out) : rc;
   };
   int rc = 0;
   auto run = [&]() -> int {
@@ -452,8 +464,8 @@ int qis_create(const qis_config* cfg, qis_ctx** out) {
     ALLOC(ctx->zob, kMaxN);
     ALLOC(ctx->stats, (size_t)ctx->max_inst * (NP + 8));   // validation statistics of every instance
     ALLOC(ctx->items_d, (size_t)ctx->max_inst);
-    ctx->f64_filter = ctx->mode == QIS_FP64 && ctx->cfg.flips != QIS_FLIPS_SINGLE && ctx->NP <= kSearchMaxNP &&
-                      ctx->K1 <= kSearchMaxK1;
+    ctx->f64_filter = filter && !ctx->no_fused && ctx->mode == QIS_FP64 && ctx->cfg.flips != QIS_FLIPS_SINGLE &&
+                      ctx->NP <= kSearchMaxNP && ctx->K1 <= kSearchMaxK1;
     if (ctx->f64_filter) {   // the fixed-point fields and FP32 couplings of the fused search's filter
       ALLOC(ctx->Jq, ctx->pool_mat);
       ALLOC(ctx->J4, ctx->pool_mat);
@@ -501,8 +513,8 @@ int qis_create(const qis_config* cfg, qis_ctx** out) {
     ALLOC(P.lst_ord, B * K1);
     ALLOC(P.lst_count, B);
     P.pw_n = 0;
-    if (ctx->K1 <= kSearchMaxK1 && (ctx->mode == QIS_FP64 ? ctx->f64_filter
-                                                          : ctx->cfg.flips == QIS_FLIPS_SINGLE || ctx->NP <= kSearchMaxNP)) {
+    if (!ctx->no_fused && ctx->K1 <= kSearchMaxK1 &&
+        (ctx->mode == QIS_FP64 ? ctx->f64_filter : ctx->cfg.flips == QIS_FLIPS_SINGLE || ctx->NP <= kSearchMaxNP)) {
       // the parents' words of a launch's iterations: as many as fit in 1 GiB, 8 .. 128
       P.pw_n = (int)std::min<size_t>(128, std::max<size_t>(8, (1ull << 30) / (B * W * sizeof(uint64_t))));
       ALLOC(P.pw, B * (size_t)P.pw_n * W);
@@ -615,6 +627,8 @@ int qis_create(const qis_config* cfg, qis_ctx** out) {
   *out = ctx;
   return 0;
 }
+
+}  // namespace
 
 void qis_destroy(qis_ctx* ctx) {
   if (!ctx) return;
