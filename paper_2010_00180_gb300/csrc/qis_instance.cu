@@ -12,6 +12,8 @@
 
 namespace qis {
 
+constexpr int kMaxGridY = 65535;   // a grid's second dimension: instances per launch of the batch kernels
+
 // ---------------------------------------------------------------- validation
 // stats layout (doubles): [0] bad flags (as bits of an int), [1] max frac bits, [2] max|J| bits,
 // [3] max|h| bits, [4 .. 4+n) row sums sum_{j>i} |J_ij|; the host adds [4+n] = sum_i |h_i|.
@@ -98,13 +100,17 @@ __global__ void k_restride_batch(const LayoutItem* items, double* J64) {
   }
 }
 
-// Layout and validation of `count` staged instances (items on the device), two launches.
+// Layout and validation of `count` staged instances (items on the device), two launches per kMaxGridY.
 cudaError_t launch_layout_batch(const DevPtrs& P, const LayoutItem* items, int count, int max_n_pad, double* J64,
                                 cudaStream_t s) {
-  if (count <= 0) return cudaSuccess;
-  k_restride_batch<<<dim3(max_n_pad, count), 256, 0, s>>>(items, J64);
-  k_validate_batch<<<dim3((max_n_pad + 7) / 8, count), 256, 0, s>>>(items, P.J64, P.h64);
-  return cudaGetLastError();
+  for (int y = 0; y < count; y += kMaxGridY) {
+    const int c = std::min(count - y, kMaxGridY);
+    k_restride_batch<<<dim3(max_n_pad, c), 256, 0, s>>>(items + y, J64);
+    k_validate_batch<<<dim3((max_n_pad + 7) / 8, c), 256, 0, s>>>(items + y, P.J64, P.h64);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 // ---------------------------------------------------------------- fixed point + digits
@@ -155,13 +161,17 @@ __global__ void __launch_bounds__(256) k_rowmax4_batch(DevPtrs P, int first) {
   if (lane == 0) P.rm4[d.off_vec + i] = m;
 }
 
-// Fixed-point planes, digits and row maxima of instances first .. first+count-1, two launches.
+// Fixed-point planes, digits and row maxima of instances first .. first+count-1, two launches per kMaxGridY.
 cudaError_t launch_prepare_batch(const DevPtrs& P, int first, int count, int max_n_pad, __half* D16, long long* Jq,
                                  float* J4, long long* hq, cudaStream_t s) {
-  if (count <= 0) return cudaSuccess;
-  k_quantize_batch<<<dim3(max_n_pad, count), 256, 0, s>>>(P, first, D16, Jq, J4, hq);
-  k_rowmax4_batch<<<dim3((max_n_pad + 7) / 8, count), 256, 0, s>>>(P, first);
-  return cudaGetLastError();
+  for (int y = 0; y < count; y += kMaxGridY) {
+    const int c = std::min(count - y, kMaxGridY);
+    k_quantize_batch<<<dim3(max_n_pad, c), 256, 0, s>>>(P, first + y, D16, Jq, J4, hq);
+    k_rowmax4_batch<<<dim3((max_n_pad + 7) / 8, c), 256, 0, s>>>(P, first + y);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 // ---------------------------------------------------------------- search initialisation
@@ -194,8 +204,8 @@ __global__ void __launch_bounds__(32) k_init_energy_f64(DevPtrs P, int inst0) {
 }
 
 cudaError_t launch_init_energy_f64(const DevPtrs& P, int inst0, int n_inst, cudaStream_t s) {
-  for (int y = 0; y < n_inst; y += 65535)   // (the grid's second dimension)
-    k_init_energy_f64<<<dim3((P.R + 31) / 32, std::min(n_inst - y, 65535)), 32, 0, s>>>(P, inst0 + y);
+  for (int y = 0; y < n_inst; y += kMaxGridY)
+    k_init_energy_f64<<<dim3((P.R + 31) / 32, std::min(n_inst - y, kMaxGridY)), 32, 0, s>>>(P, inst0 + y);
   return cudaGetLastError();
 }
 
