@@ -221,12 +221,13 @@ int qis_energies(qis_ctx* ctx, int instance_id, int count, const uint64_t* bits,
 int qis_synchronize(qis_ctx* ctx);
 
 /* Bound of every device-side wait of the context's kernels (the mbarrier waits of the tensor-core
- * field GEMM and of the dense pair scan's staging ring), in ns of %globaltimer (2 s by default;
- * 1e3 <= limit_ns <= 6e10). A wait that runs out sets the context's timeout flag, reported as
+ * field GEMM, of the energies from scratch and of the dense pair scan's staging ring), in ns of
+ * %globaltimer (2 s by default; 1e3 <= limit_ns <= 6e10). A wait that runs out sets the context's timeout flag, reported as
  * QIS_ERR_DEVICE_TIMEOUT by the next synchronising call; the kernel then waits (at most 2 s) for
  * the copies and tensor-core operations it already issued, frees its tensor memory and returns,
- * so the context stays usable: qis_reset clears the flag and restarts the searches.
- * probe = 1 makes every later field GEMM first wait on a barrier that nothing ever completes, so
+ * so the context stays usable: qis_reset clears the flag and restarts the searches. In qis_energies and
+ * in the energies of qis_topk_states it fails that call alone and sets no flag.
+ * probe = 1 makes every later field GEMM and energy from scratch first wait on a barrier that nothing ever completes, so
  * that path can be exercised without any fault (failure-detection tests); 0 for normal work. */
 int qis_set_wait_limit(qis_ctx* ctx, uint64_t limit_ns, int probe);
 

@@ -169,13 +169,14 @@ int check_status(qis_ctx* ctx) {
   return 0;
 }
 
-// After the last copy of rescored energies is enqueued: wait for the stream, and fail if a wait of
-// the rescoring kernel (or of an earlier one) gave up.
-int sync_energies(qis_ctx* ctx) {
-  int st = 0;
-  CK(cudaMemcpyAsync(&st, ctx->P.status, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+// After the copy of `count` rescored energies into E (NULL: not wanted) is enqueued: wait for the stream,
+// and fail if a wait of the rescoring kernel gave up, which leaves NaN in their place (an energy is never
+// one). Read from what was copied: a copy of the status word took a small call (n = 16) from 32 to 40 us.
+int sync_energies(qis_ctx* ctx, const double* E, int count) {
   CK(cudaStreamSynchronize(ctx->stream));
-  if (st & kStatTimeout) return check_status(ctx);
+  bool bad = false;
+  for (int k = 0; E && k < count; ++k) bad |= E[k] != E[k];
+  if (bad) return fail(ctx, QIS_ERR_DEVICE_TIMEOUT, "a bounded device-side wait gave up");
   return 0;
 }
 
@@ -1566,7 +1567,7 @@ int qis_topk_states(qis_ctx* ctx, int instance_id, int k, uint64_t* bits_out, do
     if (src_out && off == 0)
       CK(cudaMemcpyAsync(src_out, ctx->P.mrg_src + (size_t)instance_id * ctx->K1, sizeof(uint64_t) * m,
                          cudaMemcpyDeviceToHost, s));
-    const int rc = sync_energies(ctx);
+    const int rc = sync_energies(ctx, E_out ? E_out + off : nullptr, c);
     if (rc) return rc;
   }
   if (n_out) *n_out = m;
@@ -1636,7 +1637,7 @@ int qis_energies(qis_ctx* ctx, int instance_id, int count, const uint64_t* bits,
     CK(cudaMemcpyAsync(ctx->scratch_bits, bits + (size_t)off * d.W, sizeof(uint64_t) * c * d.W, cudaMemcpyHostToDevice, s));
     LAUNCH(launch_energies(ctx->P, instance_id, d, ctx->scratch_bits, c, d.W, ctx->scratch_E, s));
     CK(cudaMemcpyAsync(E_out + off, ctx->scratch_E, sizeof(double) * c, cudaMemcpyDeviceToHost, s));
-    const int rc = sync_energies(ctx);
+    const int rc = sync_energies(ctx, E_out + off, c);
     if (rc) return rc;
   }
   return 0;

@@ -124,7 +124,7 @@ struct DevPtrs {
                           // iteration forms it from psi0's exact fields (split modes)
   int* status;            // [0] error bits
   unsigned long long wait_ns;  // bound of every device-side wait (%globaltimer ns; 2 s by default)
-  int wait_probe;         // 1: the field GEMM's MMA thread first waits on a barrier that nothing
+  int wait_probe;         // 1: the field GEMM's MMA thread and k_energy first wait on a barrier that nothing
                           // completes (tests the timeout path); 0 otherwise
   int* nprod;             // [b] productive iterations (a parent was expanded) of search b
   unsigned long long* cand_acc;  // [2] pair and single candidates of removed instances

@@ -36,6 +36,7 @@ namespace qis {
 constexpr int kEnSeg = 16;          // 64-column steps per block (1024 columns: |F_d| <= 2^21, the magic add below)
 constexpr int kEnTileA = 128 * 64 * 2;   // spins of 128 states
 constexpr int kEnTileD = 64 * 64 * 2;    // one digit of 64 x 64 couplings
+constexpr int kEnFailed = 1 << 20;  // (at most 4352 blocks share a state)
 constexpr float kMagic = 12582912.f;     // 1.5 2^23: x + kMagic has the integer x in its low bits, |x| <= 2^21
 
 // Where the states of a call are, and where their integer sums go.
@@ -47,8 +48,8 @@ struct EnergyJob {
   const uint64_t* states;    // [inst][per][Wn], or NULL: the merged lists (mrg_ref)
   int from_q;                // 1: the fixed-point couplings of every instance (split modes)
   unsigned long long* acc;   // [inst][per][2]: sum of the digits 2.. and of 0, 1 (zero between calls)
-  int* left;                 // [inst][tile of 128 states]: blocks done (zero between calls)
-  double* E_out;             // [inst][per] energies, or NULL: init_q and init_E of search first_search + s
+  int* left;                 // [inst][tile of 128 states]: blocks done, kEnFailed per failed one (zero between calls)
+  double* E_out;             // [inst][per] energies (NaN: a wait gave up), or NULL: init_q and init_E of search first_search + s
   uint64_t* words_out;       // [inst][per][Wmax] the states' words (may be NULL)
 };
 
@@ -134,7 +135,7 @@ __global__ void __launch_bounds__(256) k_energy(DevPtrs P, EnergyJob E, int nseg
   };
   fetch(kc0);
   const uint32_t idesc = idesc_f16(64);
-  bool ok = true;
+  bool ok = !P.wait_probe || mbar_wait(&done[0], 0, t0, P.wait_ns);   // (the probe: a wait that nothing completes)
   int it = 0;
   for (int kc = kc0; kc < kc1; ++kc, ++it) {
     const int buf = it & 1;
@@ -212,8 +213,10 @@ __global__ void __launch_bounds__(256) k_energy(DevPtrs P, EnergyJob E, int nseg
   const bool mine = tid < 128 && s0 + tid < cnt;
   long long hi = 0, lo = 0;   // this thread's state: the sums of digits 2.. and of 0, 1
   unsigned long long* a = E.acc + 2 * ((long long)blockIdx.z * E.per + s0 + tid);
-  if (__syncthreads_or(!ok)) {
-    if (tid == 0) atomicOr(P.status, kStatTimeout);
+  bool failed = __syncthreads_or(!ok);
+  if (failed) {
+    // (the host finds the NaN of given states in what it copies; the searches are none the worse)
+    if (tid == 0 && !(E.E_out && E.states)) atomicOr(P.status, kStatTimeout);
   } else if (warp < 4) {
     // thread = state: T_d = sum over the 64 rows i of s_i F_d (|T_d| <= 2^27, int32)
     const uint64_t w = st_ptr[tid][rb];   // i0 < n: word rb is within the state
@@ -247,14 +250,17 @@ __global__ void __launch_bounds__(256) k_energy(DevPtrs P, EnergyJob E, int nseg
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
   // the last block of these states turns the sums into energies and clears them for the next call
   if (total > 1) {
-    __shared__ int s_last;
+    __shared__ int s_last, s_failed;
     if (tid == 0) {
       int* c = E.left + (long long)blockIdx.z * gridDim.y + blockIdx.y;
-      s_last = atomicAdd(c, 1) == total - 1;
+      const int done_before = atomicAdd(c, failed ? kEnFailed + 1 : 1);
+      s_last = (done_before & (kEnFailed - 1)) == total - 1;
+      s_failed = failed || done_before >= kEnFailed;
       if (s_last) *c = 0;
     }
     __syncthreads();
     if (!s_last) return;
+    failed = s_failed;
     __threadfence();
     if (mine) {
       hi = (long long)atomicExch(a, 0ull);
@@ -271,7 +277,8 @@ __global__ void __launch_bounds__(256) k_energy(DevPtrs P, EnergyJob E, int nseg
   if (!mine) return;
   if (E.E_out) {
     // hi 2^24 + lo rounded once (hi has at most 53 bits unless the couplings need all 58)
-    E.E_out[(long long)blockIdx.z * E.per + s0 + tid] = ldexp((double)hi * 16777216.0 + (double)lo, -Q);
+    E.E_out[(long long)blockIdx.z * E.per + s0 + tid] =
+        failed ? __longlong_as_double(0x7ff8000000000000ll) : ldexp((double)hi * 16777216.0 + (double)lo, -Q);
   } else {
     const long long b2 = (long long)d.first_search + s0 + tid, Eq = (hi << 24) + lo;   // |E 2^q| < 2^52
     P.init_q[b2] = Eq;
