@@ -500,7 +500,15 @@ cudaError_t pass_tm(qis_mlp* m, int M, const float* X, const float* y, cudaStrea
 // qis_mlp_loss_grad H = 256 97 / 110 us, H = 512 220 / 267, qis_mlp_forward H = 512 82 / 107; at M = 700
 // qis_mlp_loss_grad H = 256 135 / 112. Warm starts of 120 instances of n = 300 and their searches
 // 12.4 / 13.0 ms.
+// Widths above 512 have more than four groups of columns, so a warp that takes one or two rows of a block
+// reads the weights once for each of several units of work; it takes all of the block's rows there.
+// Calls of qis_mlp_forward / qis_mlp_loss_grad in us, with the forms of narrow networks and so (in
+// brackets the layers as launches of their own, which both replaced): H = 1024 M = 1 242 / 814 and 118 / 552
+// (209 / 630), M = 700 345 / 966 and 181 / 581 (326 / 1158), M = 4096 944 / 2503 and 539 / 1615 (938 / 3194);
+// H = 768 M = 700 207 / 539 and 143 / 402 (192 / 703), M = 4096 378 / 1079 and 399 / 1079 (639 / 2104); H = 640
+// M = 300 120 / 330 and 81 / 252 (163 / 570), M = 2000 213 / 566 and 160 / 451 (288 / 1028).
 cudaError_t mlp_pass(qis_mlp* m, int M, const float* X, const float* y, cudaStream_t s) {
+  if (m->H > 512) return M <= 4 * m->sms ? pass_tm<4, 4, 16>(m, M, X, y, s) : pass_tm<8, 8, 8>(m, M, X, y, s);
   if (M <= 4 * m->sms) return pass_tm<4, 1, 32>(m, M, X, y, s);
   if (M <= 8 * m->sms) return pass_tm<4, 1, 8>(m, M, X, y, s);
   if (M <= 18 * m->sms) return pass_tm<8, 2, 8>(m, M, X, y, s);
