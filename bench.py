@@ -638,21 +638,20 @@ def roofline_search(res, pk, src):
     """The fused search kernel (one block per search through every iteration of a call) against
     the measured HBM bandwidth, with its algorithmic bytes: per expanded parent the fields by
     update (the generator's exact fields and two coupling rows read, the parent's written: 32
-    bytes a site), the row maxima of the pair scan (4 bytes a site), the kept states' words for
-    the near-duplicate test (8 bytes a word of each of the K+1 states); 4 bytes per pair tested
-    (4J~_ij); 32 bytes per survivor (entry, aq_i, aq_j, Jq_ij). The list order, keys, stamps,
-    used flags and {a_i, s_i} live in shared memory and cost no HBM traffic; the new states'
-    words are not counted."""
+    bytes a site; single flips read one row: 24); 4 bytes per pair tested (4J~_ij; the FP64 mode
+    does not report how many, and they are left out); 32 bytes per survivor (entry, aq_i, aq_j,
+    Jq_ij; single flips 8, aq_i). The list order, keys, hashes, flips, used flags and the listed
+    sites live in shared memory and cost no HBM traffic; the row maxima of the listed sites, the
+    words of the few states whose hashes propose them as near and the new states' words are not
+    counted."""
     ms, nl = res["prof"].get("search", (0.0, 0))
     if nl == 0 or ms <= 0:
         return None
-    n, K1 = res["n"], res["K"] + 1
-    words = (n + 63) // 64
+    n, single, fp64 = res["n"], res["flips"] == "single", res["prec"] == "fp64"
     parents = res["parents"] / nl                 # expanded parents per launch
-    tested = res["evald"] / nl
+    tested = 0.0 if fp64 else res["evald"] / nl
     surv = res.get("survivors", 0.0) / nl
-    per_parent = 32.0 * n + 4.0 * n + 8.0 * words * K1
-    bytes_per_launch = parents * per_parent + 4.0 * tested + 32.0 * surv
+    bytes_per_launch = parents * (24.0 if single else 32.0) * n + 4.0 * tested + (8.0 if single else 32.0) * surv
     dur = ms / nl / 1e3
     achieved = bytes_per_launch / dur / 1e9
     peak = float(pk.get("hbm_gbs", 6800.0))
@@ -664,10 +663,11 @@ def roofline_search(res, pk, src):
     logical = res["pairs"] / (res["ms"] / 1e3)
     return {"bound": "hbm", "achieved": round(achieved, 1), "peak": round(peak, 1), "unit": "GB/s",
             "frac": round(achieved / peak, 4), "traffic": kernel_traffic(res.get("workload"), "k_search"),
-            "kernel": "k_search", "launch_us": round(dur * 1e6, 2), "bytes_per_launch": bytes_per_launch,
+            "kernel": "k_single" if single else "k_search", "launch_us": round(dur * 1e6, 2), "bytes_per_launch": bytes_per_launch,
             "parents_per_launch": parents, "tested_pairs_per_launch": tested, "survivors_per_launch": surv,
-            "per_unit": "per expanded parent 32 B/site (fields by update) + 4 B/site (row maxima) + 8 B per word "
-                        "of each of the K+1 kept states; 4 B per pair tested; 32 B per survivor",
+            "per_unit": "per expanded parent 24 B/site (fields by update); 8 B per survivor" if single else
+                        "per expanded parent 32 B/site (fields by update); 32 B per survivor" if fp64 else
+                        "per expanded parent 32 B/site (fields by update); 4 B per pair tested; 32 B per survivor",
             "peak_source": src,
             "logical_pairs_vs_dense_alu": {"achieved": logical, "peak": alu_peak,
                                            "frac": round(logical / alu_peak, 4),

@@ -302,8 +302,9 @@ int qis_set_incremental_fields(qis_ctx* ctx, int on);
 /* Pair terms the candidate scan evaluated one by one since the context was created: in the
  * split modes the scan skips every row whose bound c_i = thr - a_i lies below a lower bound
  * of all its pair terms, and counts (rows evaluated) x (chunk width, masked entries
- * included); in QIS_FP64 it is the qis_candidate_count pairs. The pairs
- * of qis_candidate_count are all decided exactly either way. The output-sensitive scan
+ * included); in QIS_FP64 it is the qis_candidate_count pairs, whichever form decided them (the
+ * fused search evaluates few of them one by one). The pairs of qis_candidate_count are all decided
+ * exactly either way. The output-sensitive scan
  * (pair_scan 1) counts the pairs it tests one by one (those in the live rows' prefixes, each
  * once). Synchronises the stream. */
 int qis_evaluated_pairs(qis_ctx* ctx, uint64_t* pairs);

@@ -1684,7 +1684,7 @@ int qis_evaluated_pairs(qis_ctx* ctx, uint64_t* pairs) {
   if (!ctx || !pairs) return fail(ctx, QIS_ERR_INVALID_ARG, "NULL argument");
   FLUSH_INIT(ctx);
   CK(cudaStreamSynchronize(ctx->stream));
-  if (ctx->mode == QIS_FP64) {   // the plain form evaluates every pair
+  if (ctx->mode == QIS_FP64) {   // the pairs decided, whichever form ran (the fused one evaluates few of them one by one)
     uint64_t c[2];
     int rc = count_candidates(ctx, c);
     if (rc) return rc;

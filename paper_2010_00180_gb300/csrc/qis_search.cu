@@ -968,7 +968,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_search(DevPtrs P, int n_iters
         }
       }
       __syncthreads();
-      // every warp counts for itself; warp w lists the words w, w + 4, ..
+      // every warp counts for itself; warp w lists the words w, w + NW, ..
       const unsigned mk = mark[lane];
       int inc = __popc(mk);
 #pragma unroll

@@ -1,6 +1,7 @@
-"""Wide networks. Network passes whose activations in shared memory come to 48 KiB exactly (a width of 384 with 16 rows
-per block, of 768 with 8): the logits' bits are those of smaller batches. Widths above 512, where a warp takes all rows of a block: logits and gradients against the FP64 oracle (tolerances
-of the other widths' tests), logits' bits independent of the batch."""
+"""Wide networks. Passes whose activations in shared memory come to 48 KiB exactly (a width of 384 with 16
+rows per block, of 768 with 8): the logits' bits are those of smaller batches. Widths above 512, where a
+warp takes all rows of a block: logits and gradients against the FP64 oracle (tolerances of the other
+widths' tests), logits' bits independent of the batch."""
 import numpy as np
 import pytest
 
