@@ -330,22 +330,6 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_single(DevPtrs P, int n_iters
       block_exclusive_sum(mine, s_w, &tot);
       upto = tot;
     }
-    const long long Tq = (cnt == K1) ? (long long)(okey[K1 - 1] ^ (1ull << 63)) : LLONG_MAX;
-    if (upto > cap) {
-      // block-uniform, rare: more ties at the bound than the search's buffer holds. Only those below the
-      // last kept energy, and no kept states, take a place in it; an error if they are too many
-      int mine = 0;
-      for (int i = tid; i < n; i += NT)
-        mine += (!fine || reinterpret_cast<unsigned*>(a)[i] <= kth) && Epq + ax[i] < Tq && !((dupm[i >> 5] >> (i & 31)) & 1u);
-      int tot;
-      block_exclusive_sum(mine, s_w, &tot);
-      upto = tot;
-      if (upto > cap) {
-        if (tid == 0) atomicOr(P.status, kStatCapacity);
-        act = 0;
-        continue;
-      }
-    }
     if (upto > kSgBuf) {
       const long long stride = next_pow2(max(cap, 256));
       sk = P.mrg_scratch + (long long)b * 2 * stride;
@@ -353,6 +337,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_single(DevPtrs P, int n_iters
     }
     nsurv += (unsigned long long)upto;
     // ---------------------------------------------------------------- merge (Alg. 2)
+    const long long Tq = (cnt == K1) ? (long long)(okey[K1 - 1] ^ (1ull << 63)) : LLONG_MAX;
     unsigned long long kmn = ~0ull, kmx = 0;
     for (int u0 = 0; u0 < n; u0 += NT) {
       const int i = u0 + tid;
@@ -368,8 +353,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_single(DevPtrs P, int n_iters
         int wb = 0;
         if (lane == 0) wb = atomicAdd(&s_nv, __popc(bal));
         wb = __shfl_sync(0xffffffffu, wb, 0);
-        if (keep) {
-          const int slot = wb + __popc(bal & ((1u << lane) - 1));
+        const int slot = wb + __popc(bal & ((1u << lane) - 1));
+        if (keep && slot < cap) {
           sk[slot] = kk;
           se[slot] = (unsigned long long)i;
           kmn = min(kmn, kk);
@@ -388,6 +373,12 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_single(DevPtrs P, int n_iters
     }
     __syncthreads();
     int nv = s_nv;
+    // (ties at the bound that cannot enter the list, however many, take no place in the buffer)
+    if (nv > cap) {   // block-uniform: more candidates than the search's buffer holds
+      if (tid == 0) atomicOr(P.status, kStatCapacity);
+      act = 0;
+      continue;
+    }
     // more kept candidates than the buckets take at once: only the K+1 lowest can enter the list
     if (nv > 256 && nv > K1) nv = keep_lowest(sk, se, nv, K1, hist, s_w);
     const unsigned long long kmin = s_kmin, kmax = s_kmax;
