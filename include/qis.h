@@ -90,7 +90,8 @@ typedef struct {
 #define QIS_FLIPS_EXCHANGE 2
 
 /* Create a context and allocate every device buffer it will use (sized by max_n,
- * max_instances, K, R). Nothing else allocates device memory afterwards. */
+ * max_instances, K, R). Nothing else allocates device memory afterwards. A QIS_FP64 context whose
+ * fused-search planes and rings do not fit is created without them and runs the per-kernel form. */
 int qis_create(const qis_config* cfg, qis_ctx** out);
 
 /* Free the context and all its device memory. NULL is ignored. */

@@ -23,7 +23,7 @@
 // What bounds it: issue of the conversion (about 60 instructions per coupling and 128 states; the
 // MMAs need a fifth of that and the couplings are read once per 128 states). The form it
 // replaced added every coupling to 16 states with predicated FP64 or int64 adds (FP64 has two
-// lanes per SM here): 5000 states of n = 1000 from host memory 906 -> 148 us; the merged lists of
+// lanes per SM here): 5000 states of n = 1000 from host memory 906 -> 149 us (106 of them this kernel); the merged lists of
 // 32 instances of n = 2048 off their grid 18.7 -> 0.5 ms, of 2 of n = 10000 26.2 -> 0.4 ms, of 4 of
 // n = 200 .. 700 1.38 -> 0.07 ms, of 120 of n = 600 on their grid 0.87 -> 0.2 ms. The block that
 // completes a state's sums forms its energy (a second launch cost a small call 6 us).

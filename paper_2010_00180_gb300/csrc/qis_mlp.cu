@@ -27,7 +27,7 @@ constexpr int kF = 8;   // features per site
 
 // ---------------------------------------------------------------- features
 // J row i at J + i * stride (n valid entries), h[0..n). A warp per row, its lanes over the columns
-// (a thread per row read them uncoalesced, a chain of n FP64 additions: 148 us at n = 300, now 4).
+// (a thread per row read them uncoalesced, a chain of n FP64 additions: 148 us at n = 300, now 16).
 // |v|, the signs of h and the extrema are integer operations on the bits (FP64 has two lanes per SM).
 __global__ void __launch_bounds__(256) k_mlp_features(const double* J, long long stride, const double* h, int n, float* X) {
   const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
