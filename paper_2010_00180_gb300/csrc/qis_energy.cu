@@ -36,7 +36,7 @@ namespace qis {
 constexpr int kEnSeg = 16;          // 64-column steps per block (1024 columns: |F_d| <= 2^21, the magic add below)
 constexpr int kEnTileA = 128 * 64 * 2;   // spins of 128 states
 constexpr int kEnTileD = 64 * 64 * 2;    // one digit of 64 x 64 couplings
-constexpr int kEnFailed = 1 << 20;  // (at most 4352 blocks share a state)
+constexpr unsigned kEnFailed = 1u << 20;  // (at most 2192 blocks share a state: their sum stays below 2^32)
 constexpr float kMagic = 12582912.f;     // 1.5 2^23: x + kMagic has the integer x in its low bits, |x| <= 2^21
 
 // Where the states of a call are, and where their integer sums go.
@@ -253,8 +253,8 @@ __global__ void __launch_bounds__(256) k_energy(DevPtrs P, EnergyJob E, int nseg
     __shared__ int s_last, s_failed;
     if (tid == 0) {
       int* c = E.left + (long long)blockIdx.z * gridDim.y + blockIdx.y;
-      const int done_before = atomicAdd(c, failed ? kEnFailed + 1 : 1);
-      s_last = (done_before & (kEnFailed - 1)) == total - 1;
+      const unsigned done_before = (unsigned)atomicAdd(c, failed ? (int)(kEnFailed + 1) : 1);
+      s_last = (int)(done_before & (kEnFailed - 1)) == total - 1;
       s_failed = failed || done_before >= kEnFailed;
       if (s_last) *c = 0;
     }
